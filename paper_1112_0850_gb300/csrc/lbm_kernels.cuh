@@ -16,34 +16,86 @@
 
 namespace lbm {
 
-// Element access of canonical arrays in a storage format (values are
-// converted through double, rounding to nearest even when narrowing).
+// v rounded once, to nearest even, to an element of a canonical or stored
+// array. Each is the direct conversion of the value's own type: GB300 runs
+// conversions to and from double on its FP64 pipe (2 a clock and SM), and a
+// detour over double kept that pipe 90% busy in the 16-bit state kernels.
+template <class T> struct Rn;
+template <> struct Rn<double> {
+    static __device__ __forceinline__ double of(double v) { return v; }
+    static __device__ __forceinline__ double of(float v) { return (double)v; }
+};
+template <> struct Rn<float> {
+    static __device__ __forceinline__ float of(double v) { return __double2float_rn(v); }
+    static __device__ __forceinline__ float of(float v) { return v; }
+};
+template <> struct Rn<__half> {
+    static __device__ __forceinline__ __half of(double v) { return __double2half(v); }
+    static __device__ __forceinline__ __half of(float v) { return __float2half_rn(v); }
+};
+template <> struct Rn<__nv_bfloat16> {
+    static __device__ __forceinline__ __nv_bfloat16 of(double v) { return __double2bfloat16(v); }
+    static __device__ __forceinline__ __nv_bfloat16 of(float v) { return __float2bfloat16_rn(v); }
+};
+
+// Element access of canonical arrays in a storage format: values are read in
+// the narrowest arithmetic type that holds them exactly (V).
 template <int D> struct IOFmt;
 template <> struct IOFmt<LBM_F64> {
     typedef double T;
-    static __device__ __forceinline__ double get(const T *p) { return *p; }
-    static __device__ __forceinline__ void put(T *p, double v) { *p = v; }
+    typedef double V;
+    static __device__ __forceinline__ V get(const T *p) { return __ldg(p); }
 };
 template <> struct IOFmt<LBM_F32> {
     typedef float T;
-    static __device__ __forceinline__ double get(const T *p) { return (double)*p; }
-    static __device__ __forceinline__ void put(T *p, double v) { *p = __double2float_rn(v); }
+    typedef float V;
+    static __device__ __forceinline__ V get(const T *p) { return __ldg(p); }
 };
 template <> struct IOFmt<LBM_F16S> {
     typedef __half T;
-    static __device__ __forceinline__ double get(const T *p) { return (double)__half2float(*p); }
-    static __device__ __forceinline__ void put(T *p, double v) { *p = __double2half(v); }
+    typedef float V;
+    static __device__ __forceinline__ V get(const T *p) { return Stor<LBM_F16S>::ld(p); }
 };
 template <> struct IOFmt<LBM_BF16S> {
     typedef __nv_bfloat16 T;
-    static __device__ __forceinline__ double get(const T *p) { return (double)__bfloat162float(*p); }
-    static __device__ __forceinline__ void put(T *p, double v) { *p = __double2bfloat16(v); }
+    typedef float V;
+    static __device__ __forceinline__ V get(const T *p) { return Stor<LBM_BF16S>::ld(p); }
 };
+
+// Elements p[0], p[1] of a canonical array; whole pairs move at once where
+// `pair` says that they are aligned (pair_aligned).
+template <int D, class P>
+__device__ __forceinline__ void get2(const P *p, bool pair, bool has1, typename IOFmt<D>::V &a,
+                                     typename IOFmt<D>::V &b) {
+    if (pair) {
+        Stor<D>::ld2(p, a, b);
+    } else {
+        a = IOFmt<D>::get(p);
+        b = IOFmt<D>::get(p + (has1 ? 1 : 0));  // (no branch between a thread's loads)
+    }
+}
+template <class T> struct alignas(2 * sizeof(T)) Two {
+    T a, b;
+};
+template <class T, class V> __device__ __forceinline__ void put2(T *p, bool pair, bool has1, V a, V b) {
+    if (pair) {
+        *reinterpret_cast<Two<T> *>(p) = Two<T>{Rn<T>::of(a), Rn<T>::of(b)};
+    } else {
+        p[0] = Rn<T>::of(a);
+        if (has1) p[1] = Rn<T>::of(b);
+    }
+}
 
 // Canonical state arrays of a moment-split context hold plain shifted
 // deviations in the format's 16-bit element type.
 template <> struct IOFmt<LBM_F16M> : IOFmt<LBM_F16S> {};
 template <> struct IOFmt<LBM_BF16M> : IOFmt<LBM_BF16S> {};
+
+// Whether every pair (x0, x0 + 1), x0 even, of every array [k][nz][ny][nx] at
+// p starts on a whole-pair boundary (host side).
+inline bool pair_aligned(const Geom &g, const void *p, size_t elem) {
+    return (g.nx & 1) == 0 && reinterpret_cast<uintptr_t>(p) % (2 * elem) == 0;
+}
 
 // ---------------------------------------------------------------------------
 // Moment-split storage (LBM_F16M, LBM_BF16M): a cell holds, for its 19
@@ -127,11 +179,11 @@ __device__ __forceinline__ void split_store(const Dev &d, typename Stor<S>::T *P
     }
     const unsigned wx = split_pack<S>(jx, jy), wy = split_pack<S>(jz, V(0));
     const uint2 w = make_uint2(wx, wy);
-    IOFmt<S>::put(P + c, (double)v[0]);
+    P[c] = Rn<typename Stor<S>::T>::of(v[0]);
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const V g = fma(V(-split_k(i)), V(split_edot<S>(split_first(i), w)), v[i]);
-        IOFmt<S>::put(P + (long long)i * d.g.qs + c, (double)g);
+        P[(long long)i * d.g.qs + c] = Rn<typename Stor<S>::T>::of(g);
     }
     split_words(d, P)[c] = w;
     split_ghost(d, split_words(d, P), x, c, w);
@@ -574,31 +626,16 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
     }
 }
 
-// The fused step of step_pair for the moment-split formats: the gather
-// rebuilds each value from its source cell's remainder and momentum word, the
-// bounce-back reload (the mask-guided form) rebuilds the cell's own opposite
-// values from its own word, and the store writes the pair's momentum word,
-// J = j + F (the momentum of the post-collision values: the Guo collision
-// adds F), rounded, then the remainders against it.
-template <int S, bool FLAGS, int FORCE, bool RECORD, bool RED = false, bool ODD = false>
-__device__ __forceinline__ void step_pair_split(const Dev &d, const typename Stor<S>::T *__restrict__ src,
-                                                typename Stor<S>::T *__restrict__ dst, float *__restrict__ tape,
-                                                int x0, int y, int z, double *red = nullptr) {
+// The pre-collision values of the cell pair (x0, x0 + 1) of row (y, z) in a
+// moment-split lattice, m0 and m1 the push masks of its cells.
+template <int S, bool FLAGS>
+__device__ __forceinline__ void gather_pair_split(const Dev &d, const typename Stor<S>::T *__restrict__ src, int x0,
+                                                  int y, int z, int c, bool has1, uint32_t m0, uint32_t m1,
+                                                  float2 s[Q]) {
     typedef typename Stor<S>::T T;
     typedef float R;
     typedef float2 V;  // lane x: cell x0, lane y: cell x0 + 1
     const Geom &g = d.g;
-    const bool has1 = x0 + 1 < g.nx;
-    const int c = cell_index(g, x0, y, z);
-    uint32_t m0 = 0u, m1 = 0u;
-    bool live0 = true, live1 = has1;
-    if (FLAGS) {
-        const uint2 mm = ld_resident2(d.mask + c);
-        m0 = mm.x;
-        m1 = mm.y;
-        live0 = !(m0 & SOLID_BIT);
-        live1 = has1 && !(m1 & SOLID_BIT);
-    }
     const int xa = wrap1(x0 - 1, g.nx);              // e_x = +1, cell x0
     const int xb = wrap1(x0 + 1, g.nx);              // e_x = -1, cell x0
     const int xc = has1 ? wrap1(x0 + 2, g.nx) : x0;  // e_x = -1, cell x0 + 1 (e_x = +1 pulls from x0)
@@ -621,7 +658,6 @@ __device__ __forceinline__ void step_pair_split(const Dev &d, const typename Sto
             jc[r] = __ldg(Js + rb + xc);
         }
     }
-    V s[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const T *Pi = src + (long long)i * g.qs + (wrap1(z - ez(i), g.nz) * g.ny + wrap1(y - ey(i), g.ny)) * g.pitch;
@@ -686,6 +722,35 @@ __device__ __forceinline__ void step_pair_split(const Dev &d, const typename Sto
             if (((m1 >> opp(i)) & 1u) && d.flags[pull_src(g, x0 + 1, y, z, i)] == 2) s[i].y += wall_term<R>(d, i);
         }
     }
+}
+
+// The fused step of step_pair for the moment-split formats: the gather
+// rebuilds each value from its source cell's remainder and momentum word, the
+// bounce-back reload (the mask-guided form) rebuilds the cell's own opposite
+// values from its own word, and the store writes the pair's momentum word,
+// J = j + F (the momentum of the post-collision values: the Guo collision
+// adds F), rounded, then the remainders against it.
+template <int S, bool FLAGS, int FORCE, bool RECORD, bool RED = false, bool ODD = false>
+__device__ __forceinline__ void step_pair_split(const Dev &d, const typename Stor<S>::T *__restrict__ src,
+                                                typename Stor<S>::T *__restrict__ dst, float *__restrict__ tape,
+                                                int x0, int y, int z, double *red = nullptr) {
+    typedef typename Stor<S>::T T;
+    typedef float R;
+    typedef float2 V;  // lane x: cell x0, lane y: cell x0 + 1
+    const Geom &g = d.g;
+    const bool has1 = x0 + 1 < g.nx;
+    const int c = cell_index(g, x0, y, z);
+    uint32_t m0 = 0u, m1 = 0u;
+    bool live0 = true, live1 = has1;
+    if (FLAGS) {
+        const uint2 mm = ld_resident2(d.mask + c);
+        m0 = mm.x;
+        m1 = mm.y;
+        live0 = !(m0 & SOLID_BIT);
+        live1 = has1 && !(m1 & SOLID_BIT);
+    }
+    V s[Q];
+    gather_pair_split<S, FLAGS>(d, src, x0, y, z, c, has1, m0, m1, s);
     V Fx = vsplat(R(0)), Fy = vsplat(R(0)), Fz = vsplat(R(0));
     Guo2<R> G;
     if (FORCE == 1) {
@@ -1081,73 +1146,239 @@ __global__ void __launch_bounds__(256)
 }
 
 // ---------------------------------------------------------------------------
-// get_state: canonical shifted f^n = gather(P), format D; solid cells 0.
-template <int S, int D, bool FLAGS>
-__global__ void __launch_bounds__(256)
-    k_get_state(const Dev d, const typename Stor<S>::T *__restrict__ P, typename IOFmt<D>::T *__restrict__ out) {
-    typedef typename Stor<S>::R R;
-    int x, y, z;
-    if (!row_cell(d.g, d.L.nxb, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x,
-                  threadIdx.y, x, y, z))
-        return;
-    const int c = cell_index(d.g, x, y, z);
-    const long long N = d.n_cells, cc = canon_index(d.g, x, y, z);
-    if (FLAGS && d.flags[c]) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) IOFmt<D>::put(out + i * N + cc, 0.0);
-        return;
+// Readers and writers of the whole lattice run on the flat paired launch over
+// all rows (solid ones too): two x-adjacent cells per thread, d.PF.
+inline RowLaunch all_pairs(const Geom &g) { return flat_launch(pair_launch(g)); }
+inline dim3 pairs_grid(const RowLaunch &P) { return dim3(P.nyb, P.nzr); }
+
+// The push masks of the pair at cell c, 0 for a cell that is solid or past the
+// row's end, and which of the two cells are fluid.
+template <bool FLAGS>
+__device__ __forceinline__ void pair_masks(const Dev &d, int c, bool has1, uint32_t &m0, uint32_t &m1, bool &live0,
+                                           bool &live1) {
+    m0 = m1 = 0u;
+    live0 = true;
+    live1 = has1;
+    if (FLAGS) {
+        const uint2 mm = ld_resident2(d.mask + c);
+        live0 = !(mm.x & SOLID_BIT);
+        live1 = has1 && !(mm.y & SOLID_BIT);
+        m0 = live0 ? mm.x : 0u;
+        m1 = live1 ? mm.y : 0u;
     }
-    R s[Q];
-    gather<S, FLAGS>(d, P, x, y, z, c, s);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) IOFmt<D>::put(out + i * N + cc, (double)s[i]);
 }
 
-// set_state: P_i(y) = s_i(y + e_i) if fluid there, else s_{opp(i)}(y).
-template <int S, int D, bool FLAGS>
-__global__ void __launch_bounds__(256)
-    k_set_state(const Dev d, typename Stor<S>::T *__restrict__ P, const typename IOFmt<D>::T *__restrict__ in) {
-    int x, y, z;
-    if (!row_cell(d.g, d.L.nxb, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x,
-                  threadIdx.y, x, y, z))
+// gather() for the pair (x0, x0 + 1) of row (y, z), with the push masks in
+// place of the neighbours' flags: every value is loaded from its source, and
+// pairs next to a solid then load their bounced values over it. (One mask word
+// a cell instead of 18 flag bytes, and loads that do not wait for them.)
+template <int S, bool FLAGS>
+__device__ __forceinline__ void gather_pair(const Dev &d, const typename Stor<S>::T *__restrict__ P, int x0, int y,
+                                            int z, int c, bool has1, uint32_t m0, uint32_t m1,
+                                            typename Pair2<typename Stor<S>::R>::V s[Q]) {
+    typedef typename Stor<S>::T T;
+    typedef typename Stor<S>::R R;
+    const Geom &g = d.g;
+    if constexpr (is_split(S)) {
+        gather_pair_split<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
         return;
-    const int c = cell_index(d.g, x, y, z);
-    if (FLAGS && d.flags[c]) {
-        if (nan_marked<S>(d))
+    } else {
+        if (d.layout == LAYOUT_AA_NAT) {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) IOFmt<S>::put(P + (long long)i * d.g.qs + c, (double)quiet_nan<float>());
-        return;
-    }
-    const long long N = d.n_cells, cc = canon_index(d.g, x, y, z);
-    if constexpr (is_split(S)) {  // the 19 values this cell holds, written as J and remainders
-        double v[Q];
+            for (int i = 0; i < Q; ++i) Stor<S>::ld2(P + (long long)i * g.qs + c, s[i].x, s[i].y);
+            return;
+        }
+        const bool mirror = d.layout == LAYOUT_AA_SWAP;
+        const int xa = wrap1(x0 - 1, g.nx), xb = wrap1(x0 + 1, g.nx);
+        const int xc = has1 ? wrap1(x0 + 2, g.nx) : x0;
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const int t = push_dst(d.g, x, y, z, i);
-            long long off = (long long)i * N + canon_neighbor(d.g, x, y, z, i);
-            const bool bounce = FLAGS && d.flags[t];
-            if (bounce) off = (long long)opp(i) * N + cc;
-            v[i] = IOFmt<D>::get(in + off) + (bounce && d.flags[t] == 2 && d.moving_on ? d.wc[i] : 0.0);
+            const T *Pi = P + (mirror ? opp(i) : i) * g.qs +
+                          (wrap1(z - ez(i), g.nz) * g.ny + wrap1(y - ey(i), g.ny)) * g.pitch;
+            if (ex(i) == 0) {
+                Stor<S>::ld2(Pi + x0, s[i].x, s[i].y);
+            } else {
+                s[i].x = Stor<S>::ld(Pi + (ex(i) > 0 ? xa : xb));
+                s[i].y = Stor<S>::ld(Pi + (ex(i) > 0 ? x0 : xc));
+            }
         }
-        split_store<S>(d, P, x, c, v);
+        // (the link form's solid slots hold the bounced values already)
+        if (FLAGS && !(bounce_in_solid(S) && !mirror) && ((m0 | m1) & 0x7fffeu)) {
+#pragma unroll
+            for (int i = 1; i < Q; ++i) {
+                const T *Po = P + (mirror ? i : opp(i)) * g.qs + c;
+                if ((m0 >> opp(i)) & 1u) s[i].x = Stor<S>::ld(Po);
+                if ((m1 >> opp(i)) & 1u) s[i].y = Stor<S>::ld(Po + 1);
+            }
+            if (d.moving_on && ((m0 | m1) & MOVING_BIT)) {
+#pragma unroll
+                for (int i = 1; i < Q; ++i) {
+                    if (((m0 >> opp(i)) & 1u) && d.flags[pull_src(g, x0, y, z, i)] == 2) s[i].x += wall_term<R>(d, i);
+                    if (((m1 >> opp(i)) & 1u) && d.flags[pull_src(g, x0 + 1, y, z, i)] == 2)
+                        s[i].y += wall_term<R>(d, i);
+                }
+            }
+        }
+    }
+}
+
+// Resident 256-thread blocks per SM of the state kernels (<= 255 / 80 registers).
+template <int S> struct FieldBlocks {
+    static constexpr int value = S == LBM_F64 ? 2 : 3;
+};
+
+// get_state: canonical shifted f^n = gather(P), format D; solid cells 0.
+// Bound by HBM (19 values read and 19 written a cell). One cell a thread with
+// 18 flag loads and every value converted over double took 1622 us for the
+// 384x256x256 porous channel (FP16 to BF16: 1.9 GB, 0.17 of copy bandwidth).
+template <int S, int D, bool FLAGS>
+__global__ void __launch_bounds__(256, FieldBlocks<S>::value)
+    k_get_state(const Dev d, const typename Stor<S>::T *__restrict__ P, typename IOFmt<D>::T *__restrict__ out,
+                bool pair) {
+    typedef typename Stor<S>::R R;
+    int x0, y, z;
+    if (!pair_cell<true>(d.g, d.PF, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x0, y,
+                         z))
+        return;
+    const bool has1 = x0 + 1 < d.g.nx;
+    const int c = cell_index(d.g, x0, y, z);
+    const long long N = d.n_cells, cc = canon_index(d.g, x0, y, z);
+    uint32_t m0, m1;
+    bool live0, live1;
+    pair_masks<FLAGS>(d, c, has1, m0, m1, live0, live1);
+    if (FLAGS && !live0 && !live1) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) put2(out + i * N + cc, pair, has1, 0.0f, 0.0f);
         return;
     }
-    if (d.layout == LAYOUT_AA_NAT) {  // AA natural layout: s_i(x) at the cell itself
+    typename Pair2<R>::V s[Q];
+    gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) IOFmt<S>::put(P + (long long)i * d.g.qs + c, IOFmt<D>::get(in + i * N + cc));
+    for (int i = 0; i < Q; ++i)
+        put2(out + i * N + cc, pair, has1, !FLAGS || live0 ? s[i].x : R(0), !FLAGS || live1 ? s[i].y : R(0));
+}
+
+// set_state: P_i(y) = s_i(y + e_i) if fluid there, else s_{opp(i)}(y). The
+// loads follow the reverse step's gather (sources y + e_i, the pair's own
+// values over them where a mask bit is set). Moment-split storage: the 19
+// values a cell holds, in double, one cell a thread.
+template <int S, int D, bool FLAGS>
+__global__ void __launch_bounds__(256, FieldBlocks<S>::value)
+    k_set_state(const Dev d, typename Stor<S>::T *__restrict__ P, const typename IOFmt<D>::T *__restrict__ in,
+                bool pair) {
+    typedef typename Stor<S>::T T;
+    typedef typename IOFmt<D>::T TD;
+    typedef typename IOFmt<D>::V V;
+    const Geom &g = d.g;
+    int x0, y, z;
+    if (!pair_cell<true>(g, d.PF, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x0, y, z))
         return;
-    }
+    const bool has1 = x0 + 1 < g.nx;
+    const int c = cell_index(g, x0, y, z);
+    const long long N = d.n_cells, cc = canon_index(g, x0, y, z);
+    uint32_t m0, m1;
+    bool live0, live1;
+    pair_masks<FLAGS>(d, c, has1, m0, m1, live0, live1);
+    const bool mark = FLAGS && nan_marked<S>(d);
+    if (FLAGS && !mark && !live0 && !live1) return;
+    V s0[Q], s1[Q];
+    if (!is_split(S) && d.layout == LAYOUT_AA_NAT) {  // AA natural layout: s_i(x) at the cell itself
+        if (pair) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int t = push_dst(d.g, x, y, z, i);
-        long long off = (long long)i * N + canon_neighbor(d.g, x, y, z, i);
-        const bool bounce = FLAGS && d.flags[t];
-        if (bounce) off = (long long)opp(i) * N + cc;
-        const double v = IOFmt<D>::get(in + off);
-        const double wv = !bounce_in_solid(S) && bounce && d.flags[t] == 2 && d.moving_on ? d.wc[i] : 0.0;
-        IOFmt<S>::put(P + (long long)i * d.g.qs + c, v + wv);
-        // the solid neighbour's slot that the link form pulls f_opp(i)(x) from
-        if (bounce && bounce_in_solid(S)) IOFmt<S>::put(P + (long long)opp(i) * d.g.qs + t, v);
+            for (int i = 0; i < Q; ++i) get2<D>(in + i * N + cc, true, true, s0[i], s1[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) get2<D>(in + i * N + cc, false, has1, s0[i], s1[i]);
+        }
+    } else {
+        const int xa = wrap1(x0 - 1, g.nx), xb = wrap1(x0 + 1, g.nx);
+        const int xc = has1 ? wrap1(x0 + 2, g.nx) : x0;
+        // (the loads of one kind together, so that `pair` is tested once and
+        // all of them are in flight at the same time)
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            if (ex(i) == 0) continue;
+            const TD *row = in + i * N + (long long)(wrap1(z + ez(i), g.nz) * g.ny + wrap1(y + ey(i), g.ny)) * g.nx;
+            s0[i] = IOFmt<D>::get(row + (ex(i) > 0 ? xb : xa));
+            s1[i] = IOFmt<D>::get(row + (ex(i) > 0 ? xc : x0));
+        }
+        if (pair) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i)
+                if (ex(i) == 0)
+                    get2<D>(in + i * N + x0 +
+                                (long long)(wrap1(z + ez(i), g.nz) * g.ny + wrap1(y + ey(i), g.ny)) * g.nx,
+                            true, true, s0[i], s1[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < Q; ++i)
+                if (ex(i) == 0)
+                    get2<D>(in + i * N + x0 +
+                                (long long)(wrap1(z + ez(i), g.nz) * g.ny + wrap1(y + ey(i), g.ny)) * g.nx,
+                            false, has1, s0[i], s1[i]);
+        }
+        if (FLAGS && ((m0 | m1) & 0x7fffeu)) {
+#pragma unroll
+            for (int i = 1; i < Q; ++i) {
+                const TD *own = in + opp(i) * N + cc;
+                if ((m0 >> i) & 1u) s0[i] = IOFmt<D>::get(own);
+                if ((m1 >> i) & 1u) s1[i] = IOFmt<D>::get(own + 1);
+            }
+        }
+    }
+    const bool mv = FLAGS && d.moving_on && d.layout == LAYOUT_PULL && ((m0 | m1) & MOVING_BIT);
+    if constexpr (is_split(S)) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (!(k ? live1 : live0)) continue;
+            double v[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                v[i] = (double)(k ? s1[i] : s0[i]);
+                if (mv && (((k ? m1 : m0) >> i) & 1u) && i > 0 && d.flags[push_dst(g, x0 + k, y, z, i)] == 2)
+                    v[i] += d.wc[i];
+            }
+            split_store<S>(d, P, x0 + k, c + k, v);
+        }
+        return;
+    } else {
+        if (FLAGS && bounce_in_solid(S) && d.has_moving && !mark && !(live0 && live1)) {
+            // (other threads write a solid cell's moving-wall links, below)
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                if (live0) P[i * g.qs + c] = Rn<T>::of(s0[i]);
+                if (live1) P[i * g.qs + c + 1] = Rn<T>::of(s1[i]);
+            }
+        } else {
+            // a pair is stored whole, a solid cell as zeros (never read, or
+            // filled by the link kernel after this one) or as the NaN that
+            // marks it: storing the fluid cell alone took 870 us for the
+            // porous channel (384x256x256, FP16 from BF16) against 634
+            const V solid = mark ? V(quiet_nan<float>()) : V(0);
+#pragma unroll
+            for (int i = 0; i < Q; ++i)
+                put2(P + i * g.qs + c, true, true, !FLAGS || live0 ? s0[i] : solid, !FLAGS || live1 ? s1[i] : solid);
+        }
+        // links into moving walls, which the link kernel leaves to their fluid
+        // cell: the solid slot that the link form pulls f_opp(i)(x) from; in
+        // the other forms the gather adds the moving-wall term, taken off here
+        // (summed in double, rounded once)
+        if (FLAGS && d.layout == LAYOUT_PULL && ((m0 | m1) & MOVING_BIT) && (mv || bounce_in_solid(S))) {
+#pragma unroll
+            for (int i = 1; i < Q; ++i) {
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    if (!(((k ? m1 : m0) >> i) & 1u)) continue;
+                    const V v = k ? s1[i] : s0[i];
+                    const int t = push_dst(g, x0 + k, y, z, i);
+                    if (d.flags[t] != 2) continue;
+                    if (bounce_in_solid(S))
+                        P[(long long)opp(i) * g.qs + t] = Rn<T>::of(v);
+                    else
+                        P[i * g.qs + c + k] = Rn<T>::of((double)v + d.wc[i]);
+                }
+            }
+        }
     }
 }
 
@@ -1513,29 +1744,40 @@ cudaError_t Ops<S>::init_eq(const Dev &d, void *lat, const void *rho0, const voi
 }
 
 template <int S, int D>
-static cudaError_t launch_get(const Dev &d, const void *lat, void *dst) {
+static cudaError_t launch_get(const Dev &d0, const void *lat, void *dst) {
     typedef typename Stor<S>::T T;
     typedef typename IOFmt<D>::T TD;
+    if (d0.flags && !d0.mask) return cudaErrorInvalidValue;
+    Dev d = d0;
+    d.PF = all_pairs(d.g);
+    const bool pair = pair_aligned(d.g, dst, sizeof(TD));
     if (d.flags)
-        k_get_state<S, D, true><<<row_grid(d), row_block(d), 0, d.stream>>>(d, static_cast<const T *>(lat),
-                                                                          static_cast<TD *>(dst));
+        k_get_state<S, D, true><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(d, static_cast<const T *>(lat),
+                                                                                   static_cast<TD *>(dst), pair);
     else
-        k_get_state<S, D, false><<<row_grid(d), row_block(d), 0, d.stream>>>(d, static_cast<const T *>(lat),
-                                                                           static_cast<TD *>(dst));
+        k_get_state<S, D, false><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(d, static_cast<const T *>(lat),
+                                                                                    static_cast<TD *>(dst), pair);
     return cudaGetLastError();
 }
 
 template <int S, int D>
-static cudaError_t launch_set(const Dev &d, void *lat, const void *src) {
+static cudaError_t launch_set(const Dev &d0, void *lat, const void *src) {
     typedef typename Stor<S>::T T;
     typedef typename IOFmt<D>::T TD;
+    if (d0.flags && !d0.mask) return cudaErrorInvalidValue;
+    Dev d = d0;
+    d.PF = all_pairs(d.g);
+    const bool pair = pair_aligned(d.g, src, sizeof(TD));
     if (d.flags)
-        k_set_state<S, D, true><<<row_grid(d), row_block(d), 0, d.stream>>>(d, static_cast<T *>(lat),
-                                                                          static_cast<const TD *>(src));
+        k_set_state<S, D, true><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
+            d, static_cast<T *>(lat), static_cast<const TD *>(src), pair);
     else
-        k_set_state<S, D, false><<<row_grid(d), row_block(d), 0, d.stream>>>(d, static_cast<T *>(lat),
-                                                                           static_cast<const TD *>(src));
-    return cudaGetLastError();
+        k_set_state<S, D, false><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
+            d, static_cast<T *>(lat), static_cast<const TD *>(src), pair);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || d.layout != LAYOUT_PULL) return e;
+    return Ops<S>::bounce(d, lat);  // the link form's solid slots, from their fluid cells' own (1343 us for the
+                                    // porous channel with scattered stores from the kernel above)
 }
 
 template <int S>
