@@ -189,6 +189,11 @@ __device__ __forceinline__ void split_store(const Dev &d, typename Stor<S>::T *P
     split_ghost(d, split_words(d, P), x, c, w);
 }
 
+// The same values, as if newly read: what a rare branch computes from them is
+// not computed ahead of it and kept in registers.
+__device__ __forceinline__ void forget(int &a) { asm volatile("" : "+r"(a)); }
+__device__ __forceinline__ void forget(int &a, int &b, int &c) { asm volatile("" : "+r"(a), "+r"(b), "+r"(c)); }
+
 __device__ __forceinline__ bool is_solid(const uint8_t *flags, int c) { return flags && flags[c]; }
 
 // Moving-wall term of a population bounced into direction i: 6 w_i (e_i . u_w).
@@ -1204,6 +1209,7 @@ __device__ __forceinline__ void gather_pair(const Dev &d, const typename Stor<S>
         }
         // (the link form's solid slots hold the bounced values already)
         if (FLAGS && !(bounce_in_solid(S) && !mirror) && ((m0 | m1) & 0x7fffeu)) {
+            forget(c);
 #pragma unroll
             for (int i = 1; i < Q; ++i) {
                 const T *Po = P + (mirror ? i : opp(i)) * g.qs + c;
@@ -1211,6 +1217,7 @@ __device__ __forceinline__ void gather_pair(const Dev &d, const typename Stor<S>
                 if ((m1 >> opp(i)) & 1u) s[i].y = Stor<S>::ld(Po + 1);
             }
             if (d.moving_on && ((m0 | m1) & MOVING_BIT)) {
+                forget(x0, y, z);
 #pragma unroll
                 for (int i = 1; i < Q; ++i) {
                     if (((m0 >> opp(i)) & 1u) && d.flags[pull_src(g, x0, y, z, i)] == 2) s[i].x += wall_term<R>(d, i);
@@ -1222,9 +1229,12 @@ __device__ __forceinline__ void gather_pair(const Dev &d, const typename Stor<S>
     }
 }
 
-// Resident 256-thread blocks per SM of the state kernels (<= 255 / 80 registers).
-template <int S> struct FieldBlocks {
-    static constexpr int value = S == LBM_F64 ? 2 : 3;
+// Resident 256-thread blocks per SM of the readers and writers, the measured
+// best of 2 and 3: FP64 2 (3 spilled: get_state of the channel 210 against 343
+// us), moment-split storage with flags 2 (macros 101 against 148 us), else 3
+// (FP16 channel, macros 65 against 75 us, set_state 95 against 133).
+template <int S, bool FLAGS> struct FieldBlocks {
+    static constexpr int value = S == LBM_F64 ? 2 : (FLAGS && is_split(S) ? 2 : 3);
 };
 
 // get_state: canonical shifted f^n = gather(P), format D; solid cells 0.
@@ -1232,7 +1242,7 @@ template <int S> struct FieldBlocks {
 // 18 flag loads and every value converted over double took 1622 us for the
 // 384x256x256 porous channel (FP16 to BF16: 1.9 GB, 0.17 of copy bandwidth).
 template <int S, int D, bool FLAGS>
-__global__ void __launch_bounds__(256, FieldBlocks<S>::value)
+__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
     k_get_state(const Dev d, const typename Stor<S>::T *__restrict__ P, typename IOFmt<D>::T *__restrict__ out,
                 bool pair) {
     typedef typename Stor<S>::R R;
@@ -1263,7 +1273,7 @@ __global__ void __launch_bounds__(256, FieldBlocks<S>::value)
 // values over them where a mask bit is set). Moment-split storage: the 19
 // values a cell holds, in double, one cell a thread.
 template <int S, int D, bool FLAGS>
-__global__ void __launch_bounds__(256, FieldBlocks<S>::value)
+__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
     k_set_state(const Dev d, typename Stor<S>::T *__restrict__ P, const typename IOFmt<D>::T *__restrict__ in,
                 bool pair) {
     typedef typename Stor<S>::T T;
@@ -1383,32 +1393,59 @@ __global__ void __launch_bounds__(256, FieldBlocks<S>::value)
 }
 
 // ---------------------------------------------------------------------------
-// Macroscopic fields (Sec. 2 step 1): rho and u = (j + F/2)/rho; solid 0.
-template <int S, bool FLAGS, bool FORCE>
-__global__ void __launch_bounds__(256)
-    k_macros(const Dev d, const typename Stor<S>::T *__restrict__ P, typename Stor<S>::R *__restrict__ rho,
-             typename Stor<S>::R *__restrict__ u) {
-    typedef typename Stor<S>::R R;
-    int x, y, z;
-    if (!row_cell(d.g, d.L.nxb, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x,
-                  threadIdx.y, x, y, z))
-        return;
-    const int c = cell_index(d.g, x, y, z);
-    const long long N = d.n_cells, cc = canon_index(d.g, x, y, z);
-    if (FLAGS && d.flags[c]) {
-        if (rho) rho[cc] = R(0);
-        u[cc] = u[N + cc] = u[2 * N + cc] = R(0);
-        return;
+// The pair's body force: uniform, or the force field at cell c.
+template <class R, bool FORCE>
+__device__ __forceinline__ void pair_force_at(const Dev &d, int c, typename Pair2<R>::V &Fx,
+                                              typename Pair2<R>::V &Fy, typename Pair2<R>::V &Fz) {
+    Fx = Fy = Fz = vsplat(R(0));
+    if (!FORCE) return;
+    if (d.Ffield) {
+        const R *F = static_cast<const R *>(d.Ffield);
+        ld2_real(F + c, Fx.x, Fx.y);
+        ld2_real(F + d.g.qs + c, Fy.x, Fy.y);
+        ld2_real(F + 2 * d.g.qs + c, Fz.x, Fz.y);
+    } else {
+        Fx = vsplat(DevR<R>::F(d, 0));
+        Fy = vsplat(DevR<R>::F(d, 1));
+        Fz = vsplat(DevR<R>::F(d, 2));
     }
-    R s[Q];
-    gather<S, FLAGS>(d, P, x, y, z, c, s);
-    R Fx = R(0), Fy = R(0), Fz = R(0);
-    if (FORCE) force_at<R>(d, c, Fx, Fy, Fz);
-    const Mom<R> m = moments<R>(s, Fx, Fy, Fz, d.incomp);
-    if (rho) rho[cc] = m.rho;
-    u[cc] = m.ux;
-    u[N + cc] = m.uy;
-    u[2 * N + cc] = m.uz;
+}
+
+// Macroscopic fields (Sec. 2 step 1): rho and u = (j + F/2)/rho; solid 0.
+// Bound by HBM (19 values read, 4 reals written a cell).
+template <int S, bool FLAGS, bool FORCE>
+__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
+    k_macros(const Dev d, const typename Stor<S>::T *__restrict__ P, typename Stor<S>::R *__restrict__ rho,
+             typename Stor<S>::R *__restrict__ u, bool pair) {
+    typedef typename Stor<S>::R R;
+    typedef typename Pair2<R>::V V;
+    int x0, y, z;
+    if (!pair_cell<true>(d.g, d.PF, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x0, y,
+                         z))
+        return;
+    const bool has1 = x0 + 1 < d.g.nx;
+    const int c = cell_index(d.g, x0, y, z);
+    const long long N = d.n_cells, cc = canon_index(d.g, x0, y, z);
+    uint32_t m0, m1;
+    bool live0, live1;
+    pair_masks<FLAGS>(d, c, has1, m0, m1, live0, live1);
+    V o[4] = {vsplat(R(0)), vsplat(R(0)), vsplat(R(0)), vsplat(R(0))};
+    if (!FLAGS || live0 || live1) {
+        V s[Q], Fx, Fy, Fz;
+        gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
+        pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
+        const Mom2<R> m = moments2<R, FORCE>(s, Fx, Fy, Fz, d.incomp);
+        o[0] = m.rho;
+        o[1] = m.ux;
+        o[2] = m.uy;
+        o[3] = m.uz;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        R *p = k ? u + (k - 1) * N : rho;
+        if (k || rho)
+            put2(p + cc, pair, has1, !FLAGS || live0 ? o[k].x : R(0), !FLAGS || live1 ? o[k].y : R(0));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1471,33 +1508,53 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double *__re
 // g = dL/du, at the gathered state; grad_F += g / (2 rho) (u contains F/2).
 // Incompressible model (u = j + F/2): lambda^T_m = dL/drho + g.e_m, grad_F += g/2.
 template <int S, bool FLAGS, bool FORCE>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
     k_adj_seed(const Dev d, const typename Stor<S>::T *__restrict__ P, const typename Stor<S>::R *__restrict__ dL_du,
                const typename Stor<S>::R *__restrict__ dL_drho, typename Stor<S>::R *__restrict__ lam,
-               typename Stor<S>::R *__restrict__ grad_F) {
+               typename Stor<S>::R *__restrict__ grad_F, bool pair) {
     typedef typename Stor<S>::R R;
-    int x, y, z;
-    if (!row_cell(d.g, d.L.nxb, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x,
-                  threadIdx.y, x, y, z))
+    typedef typename Pair2<R>::V V;
+    constexpr int RF = sizeof(R) == 8 ? LBM_F64 : LBM_F32;  // canonical format of R
+    int x0, y, z;
+    if (!pair_cell<true>(d.g, d.PF, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x0, y,
+                         z))
         return;
-    const int c = cell_index(d.g, x, y, z);
-    const long long qs = d.g.qs, N = d.n_cells, cc = canon_index(d.g, x, y, z);
-    if (FLAGS && d.flags[c]) return;  // solid cells' adjoint slots are never read
-    R s[Q];
-    gather<S, FLAGS>(d, P, x, y, z, c, s);
-    R Fx = R(0), Fy = R(0), Fz = R(0);
-    if (FORCE) force_at<R>(d, c, Fx, Fy, Fz);
-    const Mom<R> m = moments<R>(s, Fx, Fy, Fz, d.incomp);
-    const R gx = dL_du[cc], gy = dL_du[N + cc], gz = dL_du[2 * N + cc];
-    const R dr = dL_drho ? dL_drho[cc] : R(0);
-    const R inv = d.incomp ? R(1) : R(1) / m.rho;
-    const R base = d.incomp ? dr : dr - (gx * m.ux + gy * m.uy + gz * m.uz) * inv;
+    const bool has1 = x0 + 1 < d.g.nx;
+    const int c = cell_index(d.g, x0, y, z);
+    const long long qs = d.g.qs, N = d.n_cells, cc = canon_index(d.g, x0, y, z);
+    uint32_t m0, m1;
+    bool live0, live1;
+    pair_masks<FLAGS>(d, c, has1, m0, m1, live0, live1);
+    if (FLAGS && !live0 && !live1) return;  // solid cells' adjoint slots are never read
+    V s[Q], Fx, Fy, Fz, gx, gy, gz, dr = vsplat(R(0));
+    get2<RF>(dL_du + cc, pair, has1, gx.x, gx.y);
+    get2<RF>(dL_du + N + cc, pair, has1, gy.x, gy.y);
+    get2<RF>(dL_du + 2 * N + cc, pair, has1, gz.x, gz.y);
+    if (dL_drho) get2<RF>(dL_drho + cc, pair, has1, dr.x, dr.y);
+    gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
+    pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
+    const Mom2<R> m = moments2<R, FORCE>(s, Fx, Fy, Fz, d.incomp);
+    const V inv = d.incomp ? vsplat(R(1)) : vrcp(m.rho);
+    const V gu = vfma(gz, m.uz, vfma(gy, m.uy, vmul(gx, m.ux)));
+    const V base = d.incomp ? dr : vsub(dr, vmul(gu, inv));
+    const V hx = vmul(gx, inv), hy = vmul(gy, inv), hz = vmul(gz, inv);
+    // (a solid cell of a mixed pair gets a value nobody reads)
+    st2_real(lam + c, base.x, base.y);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) lam[i * qs + c] = base + (R(ex(i)) * gx + R(ey(i)) * gy + R(ez(i)) * gz) * inv;
+    for (int p = 0; p < NPAIR; ++p) {
+        const int i = pair_first(p), o = opp(i);
+        const V e = edot_first(i, hx, hy, hz), a = vadd(base, e), b = vsub(base, e);
+        st2_real(lam + i * qs + c, a.x, a.y);
+        st2_real(lam + o * qs + c, b.x, b.y);
+    }
     if (grad_F) {
-        grad_F[cc] += R(0.5) * gx * inv;
-        grad_F[N + cc] += R(0.5) * gy * inv;
-        grad_F[2 * N + cc] += R(0.5) * gz * inv;
+        const V h[3] = {hx, hy, hz};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            R *G = grad_F + k * N + cc;
+            if (live0) G[0] += R(0.5) * h[k].x;
+            if (live1) G[1] += R(0.5) * h[k].y;
+        }
     }
 }
 
@@ -1803,15 +1860,19 @@ cudaError_t Ops<S>::set_state(const Dev &d, void *lat, const void *src, int fmt)
 }
 
 template <int S, bool FLAGS>
-static cudaError_t launch_macros(const Dev &d, const void *lat, void *rho, void *u) {
+static cudaError_t launch_macros(const Dev &d0, const void *lat, void *rho, void *u) {
     typedef typename Stor<S>::T T;
     typedef typename Stor<S>::R R;
+    if (d0.flags && !d0.mask) return cudaErrorInvalidValue;
+    Dev d = d0;
+    d.PF = all_pairs(d.g);
+    const bool pair = pair_aligned(d.g, u, sizeof(R)) && (!rho || pair_aligned(d.g, rho, sizeof(R)));
     if (d.force_on)
-        k_macros<S, FLAGS, true><<<row_grid(d), row_block(d), 0, d.stream>>>(
-            d, static_cast<const T *>(lat), static_cast<R *>(rho), static_cast<R *>(u));
+        k_macros<S, FLAGS, true><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
+            d, static_cast<const T *>(lat), static_cast<R *>(rho), static_cast<R *>(u), pair);
     else
-        k_macros<S, FLAGS, false><<<row_grid(d), row_block(d), 0, d.stream>>>(
-            d, static_cast<const T *>(lat), static_cast<R *>(rho), static_cast<R *>(u));
+        k_macros<S, FLAGS, false><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
+            d, static_cast<const T *>(lat), static_cast<R *>(rho), static_cast<R *>(u), pair);
     return cudaGetLastError();
 }
 
@@ -1842,18 +1903,22 @@ cudaError_t Ops<S>::reduce(const Dev &d, const void *lat, int z0, int z1, double
 }
 
 template <int S, bool FLAGS>
-static cudaError_t launch_seed(const Dev &d, const void *lat, const void *dL_du, const void *dL_drho, void *lam,
+static cudaError_t launch_seed(const Dev &d0, const void *lat, const void *dL_du, const void *dL_drho, void *lam,
                                void *grad_F) {
     typedef typename Stor<S>::T T;
     typedef typename Stor<S>::R R;
+    if (d0.flags && !d0.mask) return cudaErrorInvalidValue;
+    Dev d = d0;
+    d.PF = all_pairs(d.g);
+    const bool pair = pair_aligned(d.g, dL_du, sizeof(R)) && (!dL_drho || pair_aligned(d.g, dL_drho, sizeof(R)));
     if (d.force_on)
-        k_adj_seed<S, FLAGS, true><<<row_grid(d), row_block(d), 0, d.stream>>>(
+        k_adj_seed<S, FLAGS, true><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
             d, static_cast<const T *>(lat), static_cast<const R *>(dL_du), static_cast<const R *>(dL_drho),
-            static_cast<R *>(lam), static_cast<R *>(grad_F));
+            static_cast<R *>(lam), static_cast<R *>(grad_F), pair);
     else
-        k_adj_seed<S, FLAGS, false><<<row_grid(d), row_block(d), 0, d.stream>>>(
+        k_adj_seed<S, FLAGS, false><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
             d, static_cast<const T *>(lat), static_cast<const R *>(dL_du), static_cast<const R *>(dL_drho),
-            static_cast<R *>(lam), static_cast<R *>(grad_F));
+            static_cast<R *>(lam), static_cast<R *>(grad_F), pair);
     return cudaGetLastError();
 }
 
