@@ -1071,86 +1071,6 @@ __global__ void __launch_bounds__(256) k_bounce(const Dev d, typename Stor<S>::T
 }
 
 // ---------------------------------------------------------------------------
-// Initial state: P^{-1}_i(y) = f_eq_i at y + e_i if that cell is fluid, else
-// f_eq_{opp(i)}(y) (so that the gather yields f^0 = f_eq(rho0, u0)), stored
-// shifted by -w_i.
-template <class R>
-__device__ __forceinline__ R feq_shifted(int i, R rho1, R ux, R uy, R uz, bool incomp) {
-    const R eu = R(ex(i)) * ux + R(ey(i)) * uy + R(ez(i)) * uz;
-    const R usq = ux * ux + uy * uy + uz * uz;
-    const R rho = incomp ? R(1) : R(1) + rho1;  // (He & Luo: velocity terms of the reference density)
-    return R(weight(i)) * (rho1 + rho * (R(3) * eu + R(4.5) * eu * eu - R(1.5) * usq));
-}
-
-__device__ __forceinline__ long long canon_neighbor(const Geom &g, int x, int y, int z, int i) {
-    return canon_index(g, wrap1(x + ex(i), g.nx), wrap1(y + ey(i), g.ny), wrap1(z + ez(i), g.nz));
-}
-
-template <int S, bool FLAGS>
-__global__ void __launch_bounds__(256)
-    k_init_eq(const Dev d, typename Stor<S>::T *__restrict__ P, const typename Stor<S>::R *__restrict__ rho0,
-              const typename Stor<S>::R *__restrict__ u0) {
-    typedef typename Stor<S>::R R;
-    int x, y, z;
-    if (!row_cell(d.g, d.L.nxb, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x,
-                  threadIdx.y, x, y, z))
-        return;
-    const int c = cell_index(d.g, x, y, z);
-    if (FLAGS && d.flags[c]) {
-        if (nan_marked<S>(d))
-#pragma unroll
-            for (int i = 0; i < Q; ++i) P[(long long)i * d.g.qs + c] = Stor<S>::enc(quiet_nan<R>());
-        return;
-    }
-    const long long N = d.n_cells, cc = canon_index(d.g, x, y, z);
-    if constexpr (is_split(S)) {  // the 19 values this cell holds, written as J and remainders
-        R v[Q];
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int t = push_dst(d.g, x, y, z, i);
-            int k = i;
-            long long ct = canon_neighbor(d.g, x, y, z, i);
-            const bool bounce = FLAGS && d.flags[t];
-            if (bounce) {
-                k = opp(i);
-                ct = cc;
-            }
-            const R r1 = rho0 ? rho0[ct] - R(1) : R(0);
-            v[i] = feq_shifted<R>(k, r1, u0[ct], u0[N + ct], u0[2 * N + ct], d.incomp);
-            if (bounce && d.flags[t] == 2 && d.moving_on) v[i] += wall_term<R>(d, i);
-        }
-        split_store<S>(d, P, x, c, v);
-        return;
-    }
-    if (d.layout == LAYOUT_AA_NAT) {  // AA natural layout: f^0_i(x) at the cell itself
-        const R r1 = rho0 ? rho0[cc] - R(1) : R(0);
-#pragma unroll
-        for (int i = 0; i < Q; ++i)
-            P[(long long)i * d.g.qs + c] =
-                Stor<S>::enc(feq_shifted<R>(i, r1, u0[cc], u0[N + cc], u0[2 * N + cc], d.incomp));
-        return;
-    }
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int t = push_dst(d.g, x, y, z, i);
-        int k = i;
-        long long ct = canon_neighbor(d.g, x, y, z, i);
-        const bool bounce = FLAGS && d.flags[t];
-        if (bounce) {
-            k = opp(i);
-            ct = cc;
-        }
-        const R r1 = rho0 ? rho0[ct] - R(1) : R(0);
-        const R v = feq_shifted<R>(k, r1, u0[ct], u0[N + ct], u0[2 * N + ct], d.incomp);
-        // (the gather adds the moving-wall term to a value bounced off a moving wall)
-        const R wv = !bounce_in_solid(S) && bounce && d.flags[t] == 2 && d.moving_on ? wall_term<R>(d, i) : R(0);
-        P[(long long)i * d.g.qs + c] = Stor<S>::enc(v + wv);
-        // the solid neighbour's slot that the link form pulls f_opp(i)(x) from
-        if (bounce && bounce_in_solid(S)) P[(long long)opp(i) * d.g.qs + t] = Stor<S>::enc(v);
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Readers and writers of the whole lattice run on the flat paired launch over
 // all rows (solid ones too): two x-adjacent cells per thread, d.PF.
 inline RowLaunch all_pairs(const Geom &g) { return flat_launch(pair_launch(g)); }
@@ -1237,6 +1157,139 @@ template <int S, bool FLAGS> struct FieldBlocks {
     static constexpr int value = S == LBM_F64 ? 2 : (FLAGS && is_split(S) ? 2 : 3);
 };
 
+// ---------------------------------------------------------------------------
+// Initial state: P^{-1}_i(y) = f_eq_i at y + e_i if that cell is fluid, else
+// f_eq_{opp(i)}(y) (so that the gather yields f^0 = f_eq(rho0, u0)), stored
+// shifted by -w_i. Each fluid cell x forms its own 19 values once and pushes
+// them: f_eq_i(x) to slot i of x - e_i, and f_eq_opp(i)(x) to its own slot i
+// where x + e_i is solid. A solid x - e_i takes its push too: in the link form
+// that is the value its slot must hold, and in the others nobody reads it.
+// Bound by HBM (4 reals read and 19 values written a cell); every cell forming
+// the values of its 18 neighbours was bound by their 76 loads and by arithmetic
+// (FP64: its pipe 85% busy). Channel: FP32 165 to 111 us (floor 57), FP16 187 to
+// 86, FP64 2358 to 593; 256^3 box, FP32 435 to 288 us (floor 227).
+template <class R>
+__device__ __forceinline__ R feq_shifted(int i, R rho1, R ux, R uy, R uz, bool incomp) {
+    const R eu = R(ex(i)) * ux + R(ey(i)) * uy + R(ez(i)) * uz;
+    const R usq = ux * ux + uy * uy + uz * uz;
+    const R rho = incomp ? R(1) : R(1) + rho1;  // (He & Luo: velocity terms of the reference density)
+    return R(weight(i)) * (rho1 + rho * (R(3) * eu + R(4.5) * eu * eu - R(1.5) * usq));
+}
+
+// The 19 of a cell at once, opposite directions from their even and odd parts.
+template <class R> __device__ __forceinline__ void feq_all(R f[Q], R rho1, R ux, R uy, R uz, bool incomp) {
+    const R rho = incomp ? R(1) : R(1) + rho1;
+    const R usq = R(-1.5) * (ux * ux + uy * uy + uz * uz);
+    f[0] = R(1.0 / 3.0) * (rho1 + rho * usq);
+#pragma unroll
+    for (int p = 0; p < NPAIR; ++p) {
+        const int i = pair_first(p);
+        const R w = i <= 6 ? R(1.0 / 18.0) : R(1.0 / 36.0);
+        const R eu = R(ex(i)) * ux + R(ey(i)) * uy + R(ez(i)) * uz;
+        const R even = w * (rho1 + rho * (R(4.5) * eu * eu + usq)), odd = (R(3) * w * rho) * eu;
+        f[i] = even + odd;
+        f[opp(i)] = even - odd;
+    }
+}
+
+__device__ __forceinline__ long long canon_neighbor(const Geom &g, int x, int y, int z, int i) {
+    return canon_index(g, wrap1(x + ex(i), g.nx), wrap1(y + ey(i), g.ny), wrap1(z + ez(i), g.nz));
+}
+
+// Moment-split storage: the 19 values a cell holds, gathered from its
+// neighbours' fields, written as J and remainders; one cell a thread.
+template <int S, bool FLAGS>
+__global__ void __launch_bounds__(256)
+    k_init_eq_split(const Dev d, typename Stor<S>::T *__restrict__ P, const float *__restrict__ rho0,
+                    const float *__restrict__ u0) {
+    typedef float R;
+    const Geom &g = d.g;
+    int x, y, z;
+    if (!row_cell(g, d.L.nxb, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x, y, z))
+        return;
+    const int c = cell_index(g, x, y, z);
+    const uint32_t m = FLAGS ? __ldg(d.mask + c) : 0u;
+    if (m & SOLID_BIT) return;
+    const long long N = d.n_cells, cc = canon_index(g, x, y, z);
+    R v[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const bool bounce = FLAGS && i > 0 && ((m >> i) & 1u);
+        const long long ct = bounce ? cc : canon_neighbor(g, x, y, z, i);
+        const R r1 = rho0 ? rho0[ct] - R(1) : R(0);
+        v[i] = feq_shifted<R>(i, r1, bounce ? -u0[ct] : u0[ct], bounce ? -u0[N + ct] : u0[N + ct],
+                              bounce ? -u0[2 * N + ct] : u0[2 * N + ct], d.incomp);
+        if (bounce && d.moving_on && d.flags[push_dst(g, x, y, z, i)] == 2) v[i] += wall_term<R>(d, i);
+    }
+    split_store<S>(d, P, x, c, v);
+}
+
+template <int S, bool FLAGS>
+__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
+    k_init_eq(const Dev d, typename Stor<S>::T *__restrict__ P, const typename Stor<S>::R *__restrict__ rho0,
+              const typename Stor<S>::R *__restrict__ u0, bool pair) {
+    typedef typename Stor<S>::R R;
+    typedef typename Stor<S>::T T;
+    constexpr int RF = sizeof(R) == 8 ? LBM_F64 : LBM_F32;  // canonical format of R
+    const Geom &g = d.g;
+    int x0, y, z;
+    if (!pair_cell<true>(g, d.PF, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x0, y, z))
+        return;
+    const bool has1 = x0 + 1 < g.nx;
+    const int c = cell_index(g, x0, y, z);
+    const long long N = d.n_cells, cc = canon_index(g, x0, y, z);
+    uint32_t m0, m1;
+    bool live0, live1;
+    pair_masks<FLAGS>(d, c, has1, m0, m1, live0, live1);
+    const bool mark = FLAGS && nan_marked<S>(d);
+    if (FLAGS && !live0 && !live1 && !mark) return;
+    R r[2], ux[2], uy[2], uz[2];
+    if (rho0) get2<RF>(rho0 + cc, pair, has1, r[0], r[1]);
+    else r[0] = r[1] = R(1);
+    get2<RF>(u0 + cc, pair, has1, ux[0], ux[1]);
+    get2<RF>(u0 + N + cc, pair, has1, uy[0], uy[1]);
+    get2<RF>(u0 + 2 * N + cc, pair, has1, uz[0], uz[1]);
+    R f0[Q], f1[Q];
+    feq_all(f0, r[0] - R(1), ux[0], uy[0], uz[0], d.incomp);
+    feq_all(f1, r[1] - R(1), ux[1], uy[1], uz[1], d.incomp);
+    if (d.layout == LAYOUT_AA_NAT) {  // AA natural layout: f^0_i(x) at the cell itself
+        const R nan = quiet_nan<R>();
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            put2(P + i * g.qs + c, true, true, !FLAGS || live0 ? f0[i] : nan, !FLAGS || live1 ? f1[i] : nan);
+        return;
+    }
+    // cells x0 and x0 + 1 to columns x0 - e_x and x0 + 1 - e_x
+    const int xa = wrap1(x0 - 1, g.nx), xb = wrap1(x0 + 1, g.nx);
+    const int xc = has1 ? wrap1(x0 + 2, g.nx) : x0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        T *row = P + i * g.qs + (wrap1(z - ez(i), g.nz) * g.ny + wrap1(y - ey(i), g.ny)) * g.pitch;
+        if (ex(i) == 0 && live0 && live1) {
+            put2(row + x0, true, true, f0[i], f1[i]);
+        } else {
+            if (live0) row[ex(i) == 0 ? x0 : (ex(i) > 0 ? xa : xb)] = Rn<T>::of(f0[i]);
+            if (live1) row[ex(i) == 0 ? x0 + 1 : (ex(i) > 0 ? x0 : xc)] = Rn<T>::of(f1[i]);
+        }
+    }
+    if (FLAGS && ((m0 | m1) & 0x7fffeu)) {
+        forget(x0, y, z);
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (!(((k ? m1 : m0) >> i) & 1u)) continue;
+                R v = k ? f1[opp(i)] : f0[opp(i)];
+                // (the gather adds the moving-wall term to a value bounced off a moving wall)
+                if (!bounce_in_solid(S) && d.moving_on && d.flags[push_dst(g, x0 + k, y, z, i)] == 2)
+                    v += wall_term<R>(d, i);
+                P[i * g.qs + c + k] = Rn<T>::of(v);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // get_state: canonical shifted f^n = gather(P), format D; solid cells 0.
 // Bound by HBM (19 values read and 19 written a cell). One cell a thread with
 // 18 flag loads and every value converted over double took 1622 us for the
@@ -1788,15 +1841,28 @@ cudaError_t Ops<S>::fill_solid(const Dev &d, void *lat) {
 }
 
 template <int S>
-cudaError_t Ops<S>::init_eq(const Dev &d, void *lat, const void *rho0, const void *u0) {
+cudaError_t Ops<S>::init_eq(const Dev &d0, void *lat, const void *rho0, const void *u0) {
     typedef typename Stor<S>::T T;
     typedef typename Stor<S>::R R;
-    if (d.flags)
-        k_init_eq<S, true><<<row_grid(d), row_block(d), 0, d.stream>>>(
-            d, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0));
-    else
-        k_init_eq<S, false><<<row_grid(d), row_block(d), 0, d.stream>>>(
-            d, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0));
+    if (d0.flags && !d0.mask) return cudaErrorInvalidValue;
+    if constexpr (is_split(S)) {
+        if (d0.flags)
+            k_init_eq_split<S, true><<<row_grid(d0), row_block(d0), 0, d0.stream>>>(
+                d0, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0));
+        else
+            k_init_eq_split<S, false><<<row_grid(d0), row_block(d0), 0, d0.stream>>>(
+                d0, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0));
+    } else {
+        Dev d = d0;
+        d.PF = all_pairs(d.g);
+        const bool pair = pair_aligned(d.g, u0, sizeof(R)) && (!rho0 || pair_aligned(d.g, rho0, sizeof(R)));
+        if (d.flags)
+            k_init_eq<S, true><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
+                d, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0), pair);
+        else
+            k_init_eq<S, false><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
+                d, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0), pair);
+    }
     return cudaGetLastError();
 }
 
