@@ -80,10 +80,11 @@ __device__ __forceinline__ void pair_check_record(const Dev &d, int c, bool live
 
 // Even step (natural -> swapped): local, every access an aligned pair.
 // FLAT (both AA kernels): the launch of d.PF (pairs in plane order), else of d.P.
-// RED: also add the pair's pre-collision totals to red[4] (pair_add_totals).
+// RED: also hand out the pair's pre-collision totals.
 template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT, bool RED>
 __device__ __forceinline__ void aa_even_pair(const Dev &d, typename Stor<S>::T *__restrict__ A,
-                                             typename Stor<S>::R *__restrict__ tape, double *red) {
+                                             typename Stor<S>::R *__restrict__ tape,
+                                             PairTotals<typename Stor<S>::R> *tot) {
     typedef typename Stor<S>::R R;
     typedef typename Pair2<R>::V V;
     int x0, y, z;
@@ -108,7 +109,7 @@ __device__ __forceinline__ void aa_even_pair(const Dev &d, typename Stor<S>::T *
     Guo2<R> G;
     pair_force<R, FORCE, relax_about_t(S)>(d, c, Fx, Fy, Fz, G);
     const Mom2<R> m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
-    if (RED) pair_add_totals<R>(m, live0, live1, d.incomp, red);
+    if (RED) tot->set(m, live0, live1);
     pair_check_record<R, RECORD>(d, c, live0, live1, m, tape);
     collide2<R, FORCE != 0, relax_about_t(S)>(s, m, DevR<R>::omega(d), DevR<R>::cs(d), Fx, Fy, Fz, G, d.incomp);
     // a solid lane writes its NaN back (its slots stay marked). FP32: a
@@ -141,9 +142,10 @@ __global__ void __launch_bounds__(256, StepBlocks<S>::value)
 template <int S, bool FLAGS, int FORCE, bool FLAT>
 __global__ void __launch_bounds__(256, StepBlocks<S>::value)
     k_aa_even_reduce(const Dev d, typename Stor<S>::T *__restrict__ A, double *__restrict__ partials) {
-    double red[4] = {0.0, 0.0, 0.0, 0.0};
-    aa_even_pair<S, FLAGS, FORCE, false, FLAT, true>(d, A, nullptr, red);
-    block_partials(red, partials);
+    PairTotals<typename Stor<S>::R> tot;
+    tot.clear();
+    aa_even_pair<S, FLAGS, FORCE, false, FLAT, true>(d, A, nullptr, &tot);
+    block_partials(tot, partials, blockIdx.y * gridDim.x + blockIdx.x);
 }
 
 // Resident 256-thread blocks per SM the odd step is compiled for. With flags
@@ -178,7 +180,8 @@ template <int S> __host__ __device__ constexpr bool aa_free_scatter() { return S
 
 template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT, bool RED>
 __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *__restrict__ A,
-                                            typename Stor<S>::R *__restrict__ tape, double *red) {
+                                            typename Stor<S>::R *__restrict__ tape,
+                                             PairTotals<typename Stor<S>::R> *tot) {
     typedef typename Stor<S>::T T;
     typedef typename Stor<S>::R R;
     typedef typename Pair2<R>::V V;
@@ -242,7 +245,7 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
     Guo2<R> G;
     pair_force<R, FORCE, relax_about_t(S)>(d, c, Fx, Fy, Fz, G);
     const Mom2<R> m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
-    if (RED) pair_add_totals<R>(m, live0, live1, d.incomp, red);
+    if (RED) tot->set(m, live0, live1);
     pair_check_record<R, RECORD>(d, c, live0, live1, m, tape);
     collide2<R, FORCE != 0, relax_about_t(S)>(s, m, DevR<R>::omega(d), DevR<R>::cs(d), Fx, Fy, Fz, G, d.incomp);
     // P_i(x) to slot i of x + e_i, or to slot opp(i) of x if x + e_i is solid
@@ -294,9 +297,10 @@ __global__ void __launch_bounds__(256, AaOddBlocks<S, FLAGS>::value)
 template <int S, bool FLAGS, int FORCE, bool FLAT>
 __global__ void __launch_bounds__(256, AaOddBlocks<S, FLAGS>::value)
     k_aa_odd_reduce(const Dev d, typename Stor<S>::T *__restrict__ A, double *__restrict__ partials) {
-    double red[4] = {0.0, 0.0, 0.0, 0.0};
-    aa_odd_pair<S, FLAGS, FORCE, false, FLAT, true>(d, A, nullptr, red);
-    block_partials(red, partials);
+    PairTotals<typename Stor<S>::R> tot;
+    tot.clear();
+    aa_odd_pair<S, FLAGS, FORCE, false, FLAT, true>(d, A, nullptr, &tot);
+    block_partials(tot, partials, blockIdx.y * gridDim.x + blockIdx.x);
 }
 
 template <int S, bool FLAGS, int FORCE, bool FLAT>
@@ -348,8 +352,7 @@ static cudaError_t launch_aa_reduce4(const Dev &d, void *A, int odd, double *par
         k_aa_even_reduce<S, FLAGS, FORCE, FLAT><<<grid, block, 0, d.stream>>>(d, a, partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_reduce_final<<<1, RED_THREADS, 0, d.stream>>>(partials, (int)(grid.x * grid.y), out);
-    return cudaGetLastError();
+    return sum_partials(partials, (int)(grid.x * grid.y), partials + 4 * (size_t)grid.x * grid.y, out, d.stream);
 }
 
 template <int S, bool FLAGS>

@@ -1,5 +1,5 @@
 // Discrete adjoint of the D3Q19 BGK + Guo update (not in the paper; the
-// transpose of the forward kernels in lbm_kernels.cuh), and the final stage
+// transpose of the forward kernels in lbm_kernels.cuh), and the final stages
 // of the FP64 reduction.
 //
 // Forward step n at fluid cell x, in shifted populations s:
@@ -25,32 +25,43 @@
 
 namespace lbm {
 
-__device__ __forceinline__ double warp_sum_final(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Sum RED_BLOCKS x 4 partials in a fixed order (one block).
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double *__restrict__ partials, int nblocks,
+// Block g adds the partials (4 doubles each) 64 g .. 64 g + 63, + 64 gridDim.x,
+// ... in a fixed order, thread t taking quantity t & 3 of the (t >> 2)-th, to
+// out[4 g ..]. (FP64 adds issue at 2 a clock and SM: a thread summing all four
+// quantities spent 20 of them in the block sum alone.)
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double *__restrict__ partials, int n,
                                                              double *__restrict__ out) {
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
+    constexpr int ROWS = RED_THREADS / 4;
+    const int q = threadIdx.x & 3, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double acc = 0.0;
+#pragma unroll 4
+    for (int b = blockIdx.x * ROWS + (threadIdx.x >> 2); b < n; b += gridDim.x * ROWS)
+        acc += partials[4 * (long long)b + q];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] += partials[b * 4 + k];
+    for (int o = 16; o >= 4; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     __shared__ double sm[RED_THREADS / 32][4];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double v = warp_sum_final(acc[k]);
-        if (lane == 0) sm[wid][k] = v;
-    }
+    if (lane < 4) sm[wid][lane] = acc;
     __syncthreads();
     if (threadIdx.x < 4) {
         double t = 0.0;
         for (int w = 0; w < RED_THREADS / 32; ++w) t += sm[w][threadIdx.x];
-        out[threadIdx.x] = t;
+        out[4 * blockIdx.x + threadIdx.x] = t;
     }
+}
+
+// Above 2048 partials, SUM_BLOCKS blocks add them into scratch first: one block
+// took 80 us for the 65536 partials of a 256^3 step.
+cudaError_t sum_partials(double *partials, int n, double *scratch, double *out, cudaStream_t st) {
+    if (scratch && n > 2048) {
+        const int g = n / 512 < SUM_BLOCKS ? n / 512 : SUM_BLOCKS;
+        k_reduce_final<<<g, RED_THREADS, 0, st>>>(partials, n, scratch);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        partials = scratch;
+        n = g;
+    }
+    k_reduce_final<<<1, RED_THREADS, 0, st>>>(partials, n, out);
+    return cudaGetLastError();
 }
 
 // lambda^n of one cell from mu = G^T lambda^{n+1}, the recorded (rho, u) and

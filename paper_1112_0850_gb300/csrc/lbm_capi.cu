@@ -44,7 +44,7 @@ struct lbm_ctx {
     bool lam_valid;
     double *red_partials;  // RED_BLOCKS * 4 doubles
     double *red_out;       // 4 doubles
-    double *step_partials; // 4 doubles per block of the step grid (fused reduction), on first use
+    double *step_partials; // 4 doubles per block of the step grid and SUM_BLOCKS more (fused reduction), on first use
     size_t step_partials_n;
     unsigned *status_d;
     void *staging;         // device buffer for host-side arrays
@@ -772,7 +772,7 @@ static lbm_status ensure_step_partials(lbm_ctx *ctx, const Dev &d) {
     }
     ctx->step_partials = nullptr;
     ctx->step_partials_n = 0;
-    cudaError_t e = cudaMalloc((void **)&ctx->step_partials, nb * 4 * sizeof(double));
+    cudaError_t e = cudaMalloc((void **)&ctx->step_partials, (nb + SUM_BLOCKS) * 4 * sizeof(double));
     if (e != cudaSuccess) {
         cudaGetLastError();
         ctx->step_partials = nullptr;

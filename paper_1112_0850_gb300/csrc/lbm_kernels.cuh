@@ -389,23 +389,55 @@ template <int S> struct SharedRows {
     static __device__ __forceinline__ void ld2(const T *p, R &a, R &b) { Stor<S>::ls2(p, a, b); }
 };
 
-// The pair's mass and momentum j + F/2 (rho u, or u itself in the
-// incompressible model) of the pre-collision state, in FP64, added to red[4].
-template <class R>
-__device__ __forceinline__ void pair_add_totals(const Mom2<R> &m, bool live0, bool live1, bool incomp, double *red) {
-    if (live0) {
-        const double mr = incomp ? 1.0 : (double)m.rho.x;
-        red[0] += (double)m.rho.x;
-        red[1] += mr * (double)m.ux.x;
-        red[2] += mr * (double)m.uy.x;
-        red[3] += mr * (double)m.uz.x;
+// A pair's contribution to the totals: rho - 1 and the momentum j + F/2 of its
+// fluid cells (0 for the others), and how many fluid cells it has.
+template <class R> struct PairTotals {
+    typename Pair2<R>::V v[4];
+    int cells;
+    __device__ __forceinline__ void clear() {
+        v[0] = v[1] = v[2] = v[3] = vsplat(R(0));
+        cells = 0;
     }
-    if (live1) {
-        const double mr = incomp ? 1.0 : (double)m.rho.y;
-        red[0] += (double)m.rho.y;
-        red[1] += mr * (double)m.ux.y;
-        red[2] += mr * (double)m.uy.y;
-        red[3] += mr * (double)m.uz.y;
+    __device__ __forceinline__ void set(const Mom2<R> &m, bool live0, bool live1) {
+        const typename Pair2<R>::V a[4] = {m.rho1, m.jx, m.jy, m.jz};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k].x = live0 ? a[k].x : R(0);
+            v[k].y = live1 ? a[k].y : R(0);
+        }
+        cells = (int)live0 + (int)live1;
+    }
+};
+
+// Totals of FP32 values without FP64 arithmetic, which GB300 executes at 2 a
+// clock and SM (the block sums of a step took longer than the step itself:
+// 256^3 box, BF16, 595 us against 212; 259 with integer sums). A value |v| < 1024 is cut exactly
+// into whole multiples of 2^-12, 2^-35, 2^-58 and 2^-81 (adding and taking off
+// 1.5 2^23 grid steps rounds to a grid), and the multiples are summed as
+// integers: exactly, and in any order. What is dropped is below 2^-82 per
+// value, so the sums carry less rounding than FP64 ones.
+constexpr int TOT_LEVELS = 4;
+__host__ __device__ constexpr int tot_grid(int l) { return -12 - 23 * l; }
+__device__ __forceinline__ constexpr float pow2f(int e) {
+    float r = 1.0f;
+    for (; e < 0; ++e) r *= 0.5f;
+    for (; e > 0; --e) r *= 2.0f;
+    return r;
+}
+__device__ __forceinline__ constexpr double pow2d(int e) {
+    double r = 1.0;
+    for (; e < 0; ++e) r *= 0.5;
+    return r;
+}
+__device__ __forceinline__ bool tot_fits(float v) { return fabsf(v) < 1024.0f; }  // (false for NaN)
+__device__ __forceinline__ void tot_add(int h[TOT_LEVELS], float v) {
+#pragma unroll
+    for (int l = 0; l < TOT_LEVELS; ++l) {
+        constexpr float one = 1.5f * 8388608.0f;
+        const float M = one * pow2f(tot_grid(l));
+        const float t = __fadd_rn(v, M);
+        h[l] += __float_as_int(t) - __float_as_int(M);  // the multiple: |v| / 2^grid <= 2^22
+        v = __fsub_rn(v, __fsub_rn(t, M));
     }
 }
 
@@ -415,10 +447,9 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// The block's sum of every thread's red[4], in a fixed order, to
-// partials[4 b + k] of block b = blockIdx.y * gridDim.x + blockIdx.x. Every
-// thread of the block calls it (blocks of whole warps, at most 256 threads).
-__device__ __forceinline__ void block_partials(const double red[4], double *__restrict__ partials) {
+// The block's sum of every thread's red[4], in a fixed order, to out[k] of
+// thread k < 4. Every thread of the block calls it (whole warps, <= 256 threads).
+__device__ __forceinline__ double block_sum_d(const double red[4]) {
     __shared__ double sm[8][4];
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nwarps = (blockDim.x * blockDim.y) >> 5;
@@ -428,22 +459,80 @@ __device__ __forceinline__ void block_partials(const double red[4], double *__re
         if (lane == 0) sm[wid][k] = v;
     }
     __syncthreads();
+    double t = 0.0;
+    if (tid < 4)
+        for (int w = 0; w < nwarps; ++w) t += sm[w][tid];
+    return t;
+}
+
+// The block's totals (sum rho, sum j) to partials[4 b + k] of block b, from
+// each thread's pair. FP32: integer sums (above); where a value of the block is
+// too large for them (or NaN), FP64 sums in a fixed order.
+__device__ __forceinline__ void block_partials(const PairTotals<double> &p, double *__restrict__ partials, int b) {
+    double red[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) red[k] = p.v[k].x + p.v[k].y;
+    red[0] += (double)p.cells;
+    const double t = block_sum_d(red);
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    if (tid < 4) partials[4 * (long long)b + tid] = t;
+}
+__device__ __forceinline__ void block_partials(const PairTotals<float> &p, double *__restrict__ partials, int b) {
+    __shared__ int smw[8][4 * TOT_LEVELS + 1];
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int nwarps = (blockDim.x * blockDim.y) >> 5;
+    bool fits = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) fits = fits && tot_fits(p.v[k].x) && tot_fits(p.v[k].y);
+    if (__syncthreads_or(!fits)) {
+        double red[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) red[k] = (double)p.v[k].x + (double)p.v[k].y;
+        red[0] += (double)p.cells;
+        const double t = block_sum_d(red);
+        if (tid < 4) partials[4 * (long long)b + tid] = t;
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        int h[TOT_LEVELS] = {0, 0, 0, 0};
+        tot_add(h, p.v[k].x);
+        tot_add(h, p.v[k].y);
+#pragma unroll
+        for (int l = 0; l < TOT_LEVELS; ++l) {
+            const int r = __reduce_add_sync(0xffffffffu, h[l]);  // |r| <= 32 * 2 * 2^22
+            if (lane == 0) smw[wid][k * TOT_LEVELS + l] = r;
+        }
+    }
+    const int n = __reduce_add_sync(0xffffffffu, p.cells);
+    if (lane == 0) smw[wid][4 * TOT_LEVELS] = n;
+    __syncthreads();
     if (tid < 4) {
         double t = 0.0;
-        for (int w = 0; w < nwarps; ++w) t += sm[w][tid];
-        partials[4 * ((long long)blockIdx.y * gridDim.x + blockIdx.x) + tid] = t;
+#pragma unroll
+        for (int l = TOT_LEVELS - 1; l >= 0; --l) {
+            long long h = 0;
+            for (int w = 0; w < nwarps; ++w) h += smw[w][tid * TOT_LEVELS + l];
+            t = fma((double)h, pow2d(tot_grid(l)), t);
+        }
+        if (tid == 0) {
+            int n = 0;
+            for (int w = 0; w < nwarps; ++w) n += smw[w][4 * TOT_LEVELS];
+            t += (double)n;
+        }
+        partials[4 * (long long)b + tid] = t;
     }
 }
 
 // One fused step for the cell pair (x0, x0 + 1) of row (y, z): gather through
 // `rows` (the cell's own opposite populations, for bounce-back, from src),
-// collide, store to dst. RED: also add the pair's mass and momentum j + F/2
-// (of the pre-collision state, in FP64) to red[4]; the pair then never
-// returns early, so that its block can reduce.
+// collide, store to dst. RED: also hand out the pair's totals (of the
+// pre-collision state); the pair then never returns early, so that its block
+// can reduce.
 template <int S, bool FLAGS, int FORCE, bool RECORD, class Rows, bool RED = false, class I = long long>
 __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const typename Stor<S>::T *__restrict__ src,
                                           typename Stor<S>::T *__restrict__ dst, typename Stor<S>::R *__restrict__ tape,
-                                          int x0, int y, int z, double *red = nullptr) {
+                                          int x0, int y, int z, PairTotals<typename Stor<S>::R> *tot = nullptr) {
     typedef typename Stor<S>::T T;
     typedef typename Stor<S>::R R;
     typedef typename Pair2<R>::V V;  // lane x: cell x0, lane y: cell x0 + 1
@@ -559,7 +648,7 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
     const bool bad0 = live0 && !(m.rho.x > R(0) && m.rho.x < R(1e30));
     const bool bad1 = live1 && !(m.rho.y > R(0) && m.rho.y < R(1e30));
     if (bad0 || bad1) atomicOr(d.status, LBM_STATUS_DIVERGED);
-    if (RED) pair_add_totals<R>(m, live0, live1, d.incomp, red);
+    if (RED) tot->set(m, live0, live1);
     if (RECORD) {
         const long long qs = g.qs;
         st2_real(tape + c, m.rho.x, m.rho.y);
@@ -738,7 +827,7 @@ __device__ __forceinline__ void gather_pair_split(const Dev &d, const typename S
 template <int S, bool FLAGS, int FORCE, bool RECORD, bool RED = false, bool ODD = false>
 __device__ __forceinline__ void step_pair_split(const Dev &d, const typename Stor<S>::T *__restrict__ src,
                                                 typename Stor<S>::T *__restrict__ dst, float *__restrict__ tape,
-                                                int x0, int y, int z, double *red = nullptr) {
+                                                int x0, int y, int z, PairTotals<typename Stor<S>::R> *tot = nullptr) {
     typedef typename Stor<S>::T T;
     typedef float R;
     typedef float2 V;  // lane x: cell x0, lane y: cell x0 + 1
@@ -774,7 +863,7 @@ __device__ __forceinline__ void step_pair_split(const Dev &d, const typename Sto
     const bool bad0 = live0 && !(m.rho.x > R(0) && m.rho.x < R(1e30));
     const bool bad1 = live1 && !(m.rho.y > R(0) && m.rho.y < R(1e30));
     if (bad0 || bad1) atomicOr(d.status, LBM_STATUS_DIVERGED);
-    if (RED) pair_add_totals<R>(m, live0, live1, d.incomp, red);
+    if (RED) tot->set(m, live0, live1);
     if (RECORD) {
         const long long qs = g.qs;
         st2_real(tape + c, m.rho.x, m.rho.y);
@@ -875,17 +964,18 @@ __global__ void __launch_bounds__(256, StepBlocks<S>::value)
     k_step_reduce(const Dev d, const typename Stor<S>::T *__restrict__ src, typename Stor<S>::T *__restrict__ dst,
                   double *__restrict__ partials) {
     if (FLAGS && LinkBounce<S>::value) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    double red[4] = {0.0, 0.0, 0.0, 0.0};
+    PairTotals<typename Stor<S>::R> tot;
+    tot.clear();
     int x0, y, z;
     if (pair_cell<FLAT>(d.g, FLAT ? d.PF : d.P, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x,
                         threadIdx.y, x0, y, z)) {
         if constexpr (is_split(S))
-            step_pair_split<S, FLAGS, FORCE, false, true, ODD>(d, src, dst, nullptr, x0, y, z, red);
+            step_pair_split<S, FLAGS, FORCE, false, true, ODD>(d, src, dst, nullptr, x0, y, z, &tot);
         else
             step_pair<S, FLAGS, FORCE, false, GlobalRows<S>, true>(d, GlobalRows<S>{src}, src, dst, nullptr, x0, y,
-                                                                  z, red);
+                                                                  z, &tot);
     }
-    block_partials(red, partials);
+    block_partials(tot, partials, blockIdx.y * gridDim.x + blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1502,59 +1592,91 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
 }
 
 // ---------------------------------------------------------------------------
-// Mass and momentum totals in FP64: fixed grid, each thread walks the cells
-// c = tid, tid + stride, ... in order; blocks combine in a fixed tree; a
-// single block adds the per-block partials in index order. Deterministic.
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
+// Mass and momentum totals of planes z0 <= z < z1: each thread walks the pairs
+// tid, tid + stride, ... in order; every warp adds the integer sums of its
+// pairs (tot_add) to 64-bit ones, one (quantity, level) a lane; warps and
+// blocks combine in a fixed order. Deterministic. Bound by HBM (19 values read
+// a cell). FP64 values, and FP32 ones too large for the integer sums, are
+// added in FP64.
 template <int S, bool FLAGS, bool FORCE>
-__global__ void __launch_bounds__(RED_THREADS)
+__global__ void __launch_bounds__(RED_THREADS, FLAGS || is_split(S) ? 2 : FieldBlocks<S, FLAGS>::value)
     k_reduce(const Dev d, const typename Stor<S>::T *__restrict__ P, int z0, int z1, double *__restrict__ partials) {
     typedef typename Stor<S>::R R;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    // the cells of planes z0 <= z < z1
-    const long long N = (long long)d.g.nx * d.g.ny * (z1 - z0);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long cc = (long long)blockIdx.x * blockDim.x + threadIdx.x; cc < N; cc += stride) {
-        const int x = (int)(cc % d.g.nx);
-        const long long r = cc / d.g.nx;
-        const int y = (int)(r % d.g.ny);
-        const int z = z0 + (int)(r / d.g.ny);
-        const int c = cell_index(d.g, x, y, z);
-        if (FLAGS && d.flags[c]) continue;
-        R s[Q];
-        gather<S, FLAGS>(d, P, x, y, z, c, s);
-        R Fx = R(0), Fy = R(0), Fz = R(0);
-        if (FORCE) force_at<R>(d, c, Fx, Fy, Fz);
-        const Mom<R> m = moments<R>(s, Fx, Fy, Fz, d.incomp);
-        // momentum j + F/2: rho u, or u itself in the incompressible model
-        const double mr = d.incomp ? 1.0 : (double)m.rho;
-        acc[0] += (double)m.rho;
-        acc[1] += mr * (double)m.ux;
-        acc[2] += mr * (double)m.uy;
-        acc[3] += mr * (double)m.uz;
-    }
-    __shared__ double sm[RED_THREADS / 32][4];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    typedef typename Pair2<R>::V V;
+    constexpr bool INT = sizeof(R) == 4;
+    const int W = (d.g.nx + 1) / 2, per = W * d.g.ny, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long pairs = (long long)per * (z1 - z0);
+    double red[4] = {0.0, 0.0, 0.0, 0.0};
+    long long acc = 0, cells = 0;
+    bool in_red = !INT;
+    // (whole warps iterate together: their sums need every lane)
+    for (long long q0 = (long long)blockIdx.x * RED_THREADS + 32 * wid; q0 < pairs;
+         q0 += (long long)gridDim.x * RED_THREADS) {
+        const long long q = q0 + lane;
+        PairTotals<R> tot;
+        tot.clear();
+        if (q < pairs) {
+            const int zz = (int)q / per, r = (int)q - zz * per, y = r / W;  // (pairs < 2^31)
+            const int x0 = 2 * (r - y * W), z = z0 + zz;
+            const bool has1 = x0 + 1 < d.g.nx;
+            const int c = cell_index(d.g, x0, y, z);
+            uint32_t m0, m1;
+            bool live0, live1;
+            pair_masks<FLAGS>(d, c, has1, m0, m1, live0, live1);
+            if (!FLAGS || live0 || live1) {
+                V s[Q], Fx, Fy, Fz;
+                gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
+                pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
+                tot.set(moments2<R, FORCE>(s, Fx, Fy, Fz, d.incomp), live0, live1);
+            }
+        }
+        cells += tot.cells;
+        bool fits = INT;
+        if constexpr (INT) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double v = warp_sum(acc[k]);
-        if (lane == 0) sm[wid][k] = v;
+            for (int k = 0; k < 4; ++k) fits = fits && tot_fits(tot.v[k].x) && tot_fits(tot.v[k].y);
+            fits = __all_sync(0xffffffffu, fits);
+            if (fits) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    int h[TOT_LEVELS] = {0, 0, 0, 0};
+                    tot_add(h, tot.v[k].x);
+                    tot_add(h, tot.v[k].y);
+#pragma unroll
+                    for (int l = 0; l < TOT_LEVELS; ++l) {
+                        const int sum = __reduce_add_sync(0xffffffffu, h[l]);
+                        if (lane == k * TOT_LEVELS + l) acc += sum;
+                    }
+                }
+            }
+        }
+        if (!fits) {
+            in_red = true;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) red[k] += (double)tot.v[k].x + (double)tot.v[k].y;
+        }
     }
-    __syncthreads();
+    __shared__ long long sm[RED_THREADS / 32][4 * TOT_LEVELS + 1];
+    if (lane < 4 * TOT_LEVELS) sm[wid][lane] = acc;
+    for (int o = 16; o > 0; o >>= 1) cells += __shfl_xor_sync(0xffffffffu, cells, o);
+    if (lane == 0) sm[wid][4 * TOT_LEVELS] = cells;
+    double t = 0.0;
+    if (__syncthreads_or(in_red)) t = block_sum_d(red);
     if (threadIdx.x < 4) {
-        double t = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) t += sm[w][threadIdx.x];
+#pragma unroll
+        for (int l = TOT_LEVELS - 1; INT && l >= 0; --l) {
+            long long h = 0;
+            for (int w = 0; w < RED_THREADS / 32; ++w) h += sm[w][threadIdx.x * TOT_LEVELS + l];
+            t = fma((double)h, pow2d(tot_grid(l)), t);
+        }
+        if (threadIdx.x == 0) {
+            long long n = 0;
+            for (int w = 0; w < RED_THREADS / 32; ++w) n += sm[w][4 * TOT_LEVELS];
+            t += (double)n;
+        }
         partials[blockIdx.x * 4 + threadIdx.x] = t;
     }
 }
-
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double *__restrict__ partials, int nblocks,
-                                                             double *__restrict__ out);
 
 // ---------------------------------------------------------------------------
 // Adjoint seed (not in the paper): lambda^T_m = dL/drho + g.(e_m - u)/rho,
@@ -1817,8 +1939,7 @@ cudaError_t Ops<S>::step_reduce(const Dev &d, const void *src, void *dst, double
         k_bounce<S><<<dim3(Q - 1, (d.link_max + per_block - 1) / per_block), 256, 0, d.stream>>>(d, t);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    k_reduce_final<<<1, RED_THREADS, 0, d.stream>>>(partials, (int)(grid.x * grid.y), out);
-    return cudaGetLastError();
+    return sum_partials(partials, (int)(grid.x * grid.y), partials + 4 * (size_t)grid.x * grid.y, out, d.stream);
 }
 
 // NaN marks on every slot of every solid cell (NaN-mark form; no-op otherwise).
@@ -1948,24 +2069,27 @@ cudaError_t Ops<S>::macros(const Dev &d, const void *lat, void *rho, void *u) {
 }
 
 template <int S, bool FLAGS>
-static cudaError_t launch_reduce(const Dev &d, const void *lat, int z0, int z1, double *partials) {
+static cudaError_t launch_reduce(const Dev &d, const void *lat, int z0, int z1, double *partials, int blocks) {
     typedef typename Stor<S>::T T;
+    if (d.flags && !d.mask) return cudaErrorInvalidValue;
     if (d.force_on)
-        k_reduce<S, FLAGS, true><<<RED_BLOCKS, RED_THREADS, 0, d.stream>>>(d, static_cast<const T *>(lat), z0, z1,
-                                                                          partials);
+        k_reduce<S, FLAGS, true><<<blocks, RED_THREADS, 0, d.stream>>>(d, static_cast<const T *>(lat), z0, z1,
+                                                                      partials);
     else
-        k_reduce<S, FLAGS, false><<<RED_BLOCKS, RED_THREADS, 0, d.stream>>>(d, static_cast<const T *>(lat), z0, z1,
-                                                                           partials);
+        k_reduce<S, FLAGS, false><<<blocks, RED_THREADS, 0, d.stream>>>(d, static_cast<const T *>(lat), z0, z1,
+                                                                       partials);
     return cudaGetLastError();
 }
 
 template <int S>
 cudaError_t Ops<S>::reduce(const Dev &d, const void *lat, int z0, int z1, double *partials, double *out) {
-    cudaError_t e = d.flags ? launch_reduce<S, true>(d, lat, z0, z1, partials)
-                            : launch_reduce<S, false>(d, lat, z0, z1, partials);
+    // one pair a thread, at most RED_BLOCKS blocks
+    const long long want = ((long long)(d.g.nx + 1) / 2 * d.g.ny * (z1 - z0) + RED_THREADS - 1) / RED_THREADS;
+    const int blocks = (int)(want < 1 ? 1 : (want < RED_BLOCKS ? want : RED_BLOCKS));
+    cudaError_t e = d.flags ? launch_reduce<S, true>(d, lat, z0, z1, partials, blocks)
+                            : launch_reduce<S, false>(d, lat, z0, z1, partials, blocks);
     if (e != cudaSuccess) return e;
-    k_reduce_final<<<1, RED_THREADS, 0, d.stream>>>(partials, RED_BLOCKS, out);
-    return cudaGetLastError();
+    return sum_partials(partials, blocks, nullptr, out, d.stream);
 }
 
 template <int S, bool FLAGS>

@@ -92,7 +92,8 @@ __host__ __device__ constexpr bool relax_about_t(int s) { return s == LBM_F32; }
 constexpr int BOUNCE_LINKS_PER_BLOCK = 1024;
 constexpr long long BOUNCE_MAX_LINKS = 65535LL * BOUNCE_LINKS_PER_BLOCK;
 
-constexpr int RED_BLOCKS = 152 * 8;  // fixed grid of the reduction: deterministic order
+constexpr int RED_BLOCKS = 152 * 8;  // most blocks of the reduction (a function of its size: deterministic order)
+constexpr int SUM_BLOCKS = 128;      // blocks of the first stage of sum_partials
 constexpr int RED_THREADS = 256;
 
 template <int S> struct Ops {
@@ -116,7 +117,7 @@ template <int S> struct Ops {
     static cudaError_t reduce(const Dev &d, const void *lat, int z0, int z1, double *partials, double *out);
     // One step (as step, no tape) that also sums the totals of reduce for its
     // pre-collision state into out (4 doubles, device); partials: 4 doubles per
-    // block of the step grid.
+    // block of the step grid, and SUM_BLOCKS * 4 more.
     static cudaError_t step_reduce(const Dev &d, const void *src, void *dst, double *partials, double *out);
     // lambda^T from dL/du, dL/drho at the current state; grad_F += explicit term.
     static cudaError_t adj_seed(const Dev &d, const void *lat, const void *dL_du,
@@ -130,11 +131,14 @@ template <int S> struct AaOps {
     // which takes it back. tape as in Ops<S>::step.
     static cudaError_t step(const Dev &d, void *A, int odd, void *tape);
     // The same step, with the mass/momentum totals of the state it starts from
-    // summed by its blocks (partials: 4 doubles per block of the launch) and
-    // finished into out[4] (device), as Ops<S>::step_reduce.
+    // summed by its blocks (partials: 4 doubles per block of the launch and
+    // SUM_BLOCKS * 4 more) and finished into out[4] (device), as Ops<S>::step_reduce.
     static cudaError_t step_reduce(const Dev &d, void *A, int odd, double *partials, double *out);
 };
 
+// The sum of n partials (4 doubles each) in a fixed order, to out[4] (device).
+// scratch: room for SUM_BLOCKS more partials, or null (n is then small).
+cudaError_t sum_partials(double *partials, int n, double *scratch, double *out, cudaStream_t st);
 // Set-up: push masks of every padded cell from the padded flags (device).
 cudaError_t build_push_mask(const Geom &g, const uint8_t *flags, uint32_t *mask, cudaStream_t st);
 // z-slab halo copy between plane z of the lattice and a packed buffer of the

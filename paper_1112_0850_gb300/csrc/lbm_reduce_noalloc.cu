@@ -111,8 +111,7 @@ cudaError_t launch_sum(const void *state, long long N, const uint8_t *flags, con
                                                   F[1], F[2], scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_reduce_final<<<1, RED_THREADS, 0, st>>>(scratch, blocks, out);
-    return cudaGetLastError();
+    return sum_partials(scratch, blocks, nullptr, out, st);
 }
 
 }  // namespace
