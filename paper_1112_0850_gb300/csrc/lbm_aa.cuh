@@ -53,13 +53,13 @@ __device__ __forceinline__ void pair_force(const Dev &d, int c, typename Pair2<R
         Fx = vsplat(DevR<R>::F(d, 0));
         Fy = vsplat(DevR<R>::F(d, 1));
         Fz = vsplat(DevR<R>::F(d, 2));
-        G = uniform_guo<R, TFORM>(d);
+        if constexpr (sizeof(R) == 4) G = uniform_guo<R, TFORM>(d);
     } else if (FORCE == 2) {
         const R *F = static_cast<const R *>(d.Ffield);
         ld2_real(F + c, Fx.x, Fx.y);
         ld2_real(F + d.g.qs + c, Fy.x, Fy.y);
         ld2_real(F + 2 * d.g.qs + c, Fz.x, Fz.y);
-        G = guo2<R>(TFORM ? DevR<R>::cs(d) : R(1) - R(0.5) * DevR<R>::omega(d), Fx, Fy, Fz);
+        if constexpr (sizeof(R) == 4) G = guo2<R>(TFORM ? DevR<R>::cs(d) : R(1) - R(0.5) * DevR<R>::omega(d), Fx, Fy, Fz);
     }
 }
 
@@ -108,10 +108,15 @@ __device__ __forceinline__ void aa_even_pair(const Dev &d, typename Stor<S>::T *
     V Fx, Fy, Fz;
     Guo2<R> G;
     pair_force<R, FORCE, relax_about_t(S)>(d, c, Fx, Fy, Fz, G);
-    const Mom2<R> m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
+    Mom2<R> m;
+    if constexpr (S == LBM_F64)
+        m = pair64<FORCE != 0, true, RECORD || RED>(d, s, Fx, Fy, Fz);
+    else
+        m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
     if (RED) tot->set(m, live0, live1);
     pair_check_record<R, RECORD>(d, c, live0, live1, m, tape);
-    collide2<R, FORCE != 0, relax_about_t(S)>(s, m, DevR<R>::omega(d), DevR<R>::cs(d), Fx, Fy, Fz, G, d.incomp);
+    if constexpr (S != LBM_F64)
+        collide2<R, FORCE != 0, relax_about_t(S)>(s, m, DevR<R>::omega(d), DevR<R>::cs(d), Fx, Fy, Fz, G, d.incomp);
     // a solid lane writes its NaN back (its slots stay marked). FP32: a
     // 32-byte sector whose 8 cells are all solid skips its stores instead (as
     // in the two-grid step: no reader takes a solid slot's value), found by
@@ -244,10 +249,15 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
     V Fx, Fy, Fz;
     Guo2<R> G;
     pair_force<R, FORCE, relax_about_t(S)>(d, c, Fx, Fy, Fz, G);
-    const Mom2<R> m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
+    Mom2<R> m;
+    if constexpr (S == LBM_F64)
+        m = pair64<FORCE != 0, true, RECORD || RED>(d, s, Fx, Fy, Fz);
+    else
+        m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
     if (RED) tot->set(m, live0, live1);
     pair_check_record<R, RECORD>(d, c, live0, live1, m, tape);
-    collide2<R, FORCE != 0, relax_about_t(S)>(s, m, DevR<R>::omega(d), DevR<R>::cs(d), Fx, Fy, Fz, G, d.incomp);
+    if constexpr (S != LBM_F64)
+        collide2<R, FORCE != 0, relax_about_t(S)>(s, m, DevR<R>::omega(d), DevR<R>::cs(d), Fx, Fy, Fz, G, d.incomp);
     // P_i(x) to slot i of x + e_i, or to slot opp(i) of x if x + e_i is solid
 #pragma unroll
     for (int i = 0; i < Q; ++i) {

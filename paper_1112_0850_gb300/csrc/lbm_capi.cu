@@ -125,6 +125,7 @@ Dev make_dev(const lbm_ctx *ctx) {
     d.force_on = ctx->Ffield_d != nullptr || ctx->F[0] != 0.0 || ctx->F[1] != 0.0 || ctx->F[2] != 0.0;
     d.omega = 1.0 / ctx->tau;
     d.cs = ctx->tau - 0.5;
+    d.fk = fixed_k(d.omega);
     d.omega_f = (float)d.omega;
     d.cs_f = (float)d.cs;
     for (int a = 0; a < 3; ++a) d.F_f[a] = (float)d.F[a];
@@ -132,10 +133,8 @@ Dev make_dev(const lbm_ctx *ctx) {
     for (int p = 0; p < NPAIR; ++p) {
         const int i = pair_first(p);
         const double eF = ex(i) * ctx->F[0] + ey(i) * ctx->F[1] + ez(i) * ctx->F[2];
-        d.gA[p] = 9.0 * cF * weight(i) * eF;
-        d.gC[p] = 3.0 * cF * weight(i) * eF;
-        d.gAf[p] = (float)d.gA[p];
-        d.gCf[p] = (float)d.gC[p];
+        d.gAf[p] = (float)(9.0 * cF * weight(i) * eF);
+        d.gCf[p] = (float)(3.0 * cF * weight(i) * eF);
         d.gAtf[p] = (float)(9.0 * d.cs * weight(i) * eF);
         d.gCtf[p] = (float)(3.0 * d.cs * weight(i) * eF);
     }
@@ -764,7 +763,10 @@ lbm_status lbm_reduce(lbm_ctx *ctx, double out[4]) {
 // mapping of the whole step (a plane window's launch has fewer blocks).
 static lbm_status ensure_step_partials(lbm_ctx *ctx, const Dev &d) {
     const size_t nb_rows = (size_t)d.P.nxb * d.P.nyb * d.P.nzr, nb_flat = (size_t)d.PF.nxb * d.PF.nyb * d.PF.nzr;
-    const size_t nb = nb_rows > nb_flat ? nb_rows : nb_flat;
+    size_t nb = nb_rows > nb_flat ? nb_rows : nb_flat;
+    // (the FP64 two-grid step: one cell a thread)
+    const size_t nb_cells = ((size_t)d.P.nyr * d.g.nx + 255) / 256 * d.P.nzr;
+    if (ctx->storage == LBM_F64 && nb_cells > nb) nb = nb_cells;
     if (ctx->step_partials_n >= nb) return LBM_OK;
     if (ctx->step_partials) {
         cudaStreamSynchronize(ctx->stream);

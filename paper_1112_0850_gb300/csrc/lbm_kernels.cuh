@@ -281,11 +281,8 @@ template <int S> __device__ __forceinline__ bool nan_marked(const Dev &d) {
 // cells are all solid, which no one reads). Halfway bounce-back takes one of
 // these forms, chosen per storage format by measurement (Bounce<S>):
 //
-//  - load side (FP64): a 32-bit push mask per cell (bit j: x + e_j is solid)
-//    is loaded first; a population whose source x - e_i is solid (bit opp(i))
-//    loads the opposite population of the cell itself, so each value costs one
-//    load; threads whose two cells are solid skip everything.
-//  - mask-guided reload (FP32): the push mask is loaded first but the gather
+//  - mask-guided reload (FP32 and FP64): a 32-bit push mask per cell (bit j:
+//    x + e_j is solid) is loaded first but the gather
 //    does not wait for it (every load takes the neighbour's address); pairs
 //    with a bounce bit then reload their bounced populations from the cell's
 //    own opposite slots, over the gathered values, before the moments.
@@ -347,16 +344,6 @@ template <> __device__ __forceinline__ Guo2<float> uniform_guo<float, true>(cons
     }
     return t;
 }
-template <> __device__ __forceinline__ Guo2<double> uniform_guo<double, false>(const Dev &d) {
-    Guo2<double> t;
-#pragma unroll
-    for (int p = 0; p < NPAIR; ++p) {
-        t.A[p] = vsplat(d.gA[p]);
-        t.C[p] = vsplat(d.gC[p]);
-    }
-    return t;
-}
-
 // Where the gather finds the row of population i that cell row (y, z) pulls
 // from, (y - e_iy, z - e_iz): in the source lattice in global memory, or in
 // a shared-memory copy of those 19 rows (see k_step_tma).
@@ -441,23 +428,21 @@ __device__ __forceinline__ void tot_add(int h[TOT_LEVELS], float v) {
     }
 }
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // The block's sum of every thread's red[4], in a fixed order, to out[k] of
 // thread k < 4. Every thread of the block calls it (whole warps, <= 256 threads).
 __device__ __forceinline__ double block_sum_d(const double red[4]) {
     __shared__ double sm[8][4];
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nwarps = (blockDim.x * blockDim.y) >> 5;
+    // halves of the warp exchange two of the quantities, quarters one: 6 FP64
+    // adds a thread instead of the 20 of four whole butterflies
+    const bool up = lane & 16, up2 = lane & 8;
+    const double a = (up ? red[2] : red[0]) + __shfl_xor_sync(0xffffffffu, up ? red[0] : red[2], 16);
+    const double b = (up ? red[3] : red[1]) + __shfl_xor_sync(0xffffffffu, up ? red[1] : red[3], 16);
+    double v = (up2 ? b : a) + __shfl_xor_sync(0xffffffffu, up2 ? a : b, 8);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double v = warp_sum_d(red[k]);
-        if (lane == 0) sm[wid][k] = v;
-    }
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 7) == 0) sm[wid][lane >> 3] = v;
     __syncthreads();
     double t = 0.0;
     if (tid < 4)
@@ -524,6 +509,100 @@ __device__ __forceinline__ void block_partials(const PairTotals<float> &p, doubl
     }
 }
 
+// ---------------------------------------------------------------------------
+// One cell in FP64: moments and collision in fixed point (lbm_fixed.cuh), in
+// FP64 arithmetic where the cell is outside its range. Every FP64 kernel takes
+// its cells through here, so they agree bit for bit.
+struct Cell64 {
+    double rho1, rho, jx, jy, jz, ux, uy, uz;  // (j = j + F/2)
+};
+// The FP64 form: s is replaced by its post-collision values if `collide`.
+static __device__ __noinline__ void cell64_fp64(double *s, Cell64 *m, double Fx, double Fy, double Fz, double omega,
+                                                bool incomp, bool collide) {
+    double v[Q];
+    for (int i = 0; i < Q; ++i) v[i] = s[i];
+    const Mom<double> o = moments<double>(v, Fx, Fy, Fz, incomp);
+    m->rho1 = o.rho1;
+    m->rho = o.rho;
+    m->ux = o.ux;
+    m->uy = o.uy;
+    m->uz = o.uz;
+    m->jx = incomp ? o.ux : o.rho * o.ux;
+    m->jy = incomp ? o.uy : o.rho * o.uy;
+    m->jz = incomp ? o.uz : o.rho * o.uz;
+    if (!collide) return;
+    const double rho_e = incomp ? 1.0 : o.rho, c = 1.0 - 0.5 * omega;
+    const double usq = o.ux * o.ux + o.uy * o.uy + o.uz * o.uz, uF = o.ux * Fx + o.uy * Fy + o.uz * Fz;
+    for (int i = 0; i < Q; ++i) {
+        const double w = weight(i), eu = ex(i) * o.ux + ey(i) * o.uy + ez(i) * o.uz;
+        const double eF = ex(i) * Fx + ey(i) * Fy + ez(i) * Fz;
+        s[i] = (1.0 - omega) * v[i] + omega * w * (o.rho1 + rho_e * (3.0 * eu + 4.5 * eu * eu - 1.5 * usq)) +
+               c * w * (3.0 * (eF - uF) + 9.0 * eu * eF);
+    }
+}
+// MOM: m is wanted (otherwise only m.rho, 1 or what a diverging cell has).
+template <bool FORCE, bool COLLIDE, bool MOM>
+__device__ __forceinline__ void cell64(const Dev &d, double s[Q], double Fx, double Fy, double Fz, Cell64 &m) {
+    FixedMom f;
+    m.rho = 1.0;
+    if (fixed_moments<FORCE>(s, Fx, Fy, Fz, f)) {
+        if (MOM) {
+            m.rho1 = fx_out(f.r, f.E);
+            m.rho = 1.0 + m.rho1;
+            m.jx = fx_out(f.jx, f.E);
+            m.jy = fx_out(f.jy, f.E);
+            m.jz = fx_out(f.jz, f.E);
+            const double inv = d.incomp ? 1.0 : rcp_rn(m.rho);
+            m.ux = m.jx * inv;
+            m.uy = m.jy * inv;
+            m.uz = m.jz * inv;
+        }
+        if (COLLIDE) fixed_collide<FORCE>(s, f, d.fk, d.incomp);
+    } else {
+        double t[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) t[i] = s[i];
+        Cell64 o;
+        cell64_fp64(t, &o, Fx, Fy, Fz, d.omega, d.incomp, COLLIDE);
+        m = o;
+#pragma unroll
+        for (int i = 0; COLLIDE && i < Q; ++i) s[i] = t[i];
+    }
+}
+
+// The pair's moments, and its collision (COLLIDE), cell by cell.
+template <bool FORCE, bool COLLIDE, bool MOM>
+__device__ __forceinline__ Mom2<double> pair64(const Dev &d, double2 s[Q], double2 Fx, double2 Fy, double2 Fz) {
+    Mom2<double> m;
+    double t[Q];
+    Cell64 o;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) t[i] = s[i].x;
+    cell64<FORCE, COLLIDE, MOM>(d, t, Fx.x, Fy.x, Fz.x, o);
+#pragma unroll
+    for (int i = 0; COLLIDE && i < Q; ++i) s[i].x = t[i];
+    m.rho.x = o.rho;
+    if (MOM) m.rho1.x = o.rho1, m.jx.x = o.jx, m.jy.x = o.jy, m.jz.x = o.jz, m.ux.x = o.ux, m.uy.x = o.uy, m.uz.x = o.uz;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) t[i] = s[i].y;
+    cell64<FORCE, COLLIDE, MOM>(d, t, Fx.y, Fy.y, Fz.y, o);
+#pragma unroll
+    for (int i = 0; COLLIDE && i < Q; ++i) s[i].y = t[i];
+    m.rho.y = o.rho;
+    if (MOM) m.rho1.y = o.rho1, m.jx.y = o.jx, m.jy.y = o.jy, m.jz.y = o.jz, m.ux.y = o.ux, m.uy.y = o.uy, m.uz.y = o.uz;
+    return m;
+}
+
+// The moments of a pair for the readers.
+template <class R, bool FORCE>
+__device__ __forceinline__ Mom2<R> pair_moments(const Dev &d, typename Pair2<R>::V s[Q], typename Pair2<R>::V Fx,
+                                                typename Pair2<R>::V Fy, typename Pair2<R>::V Fz) {
+    if constexpr (sizeof(R) == 8)
+        return pair64<FORCE, false, true>(d, s, Fx, Fy, Fz);
+    else
+        return moments2<R, FORCE>(s, Fx, Fy, Fz, d.incomp);
+}
+
 // One fused step for the cell pair (x0, x0 + 1) of row (y, z): gather through
 // `rows` (the cell's own opposite populations, for bounce-back, from src),
 // collide, store to dst. RED: also hand out the pair's totals (of the
@@ -537,7 +616,7 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
     typedef typename Stor<S>::R R;
     typedef typename Pair2<R>::V V;  // lane x: cell x0, lane y: cell x0 + 1
     constexpr bool MFIX = Bounce<S>::mode == BB_MFIX;
-    constexpr bool LINKS = Bounce<S>::mode != BB_LOAD && !MFIX;  // flag-free gather (links or NaN marks)
+    constexpr bool LINKS = !MFIX;  // flag-free gather (links or NaN marks)
     constexpr bool NANS = Bounce<S>::mode == BB_NANS;
     const Geom &g = d.g;
     const bool has1 = x0 + 1 < g.nx;
@@ -550,7 +629,6 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
         m1 = mm.y;
         live0 = !(m0 & SOLID_BIT);
         live1 = has1 && !(m1 & SOLID_BIT);
-        if (!MFIX && !RED && !live0 && !live1) return;
     } else if (FLAGS) {
         const uchar2 fl = __ldg(reinterpret_cast<const uchar2 *>(d.flags + c));
         // (no early exit for two solid cells: branching on this load would put
@@ -567,21 +645,7 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const T *Pi = rows.row(g, i, y, z);
-        if (FLAGS && !LINKS && !MFIX && i > 0) {
-            const T *Po = lat_at<I>(src, opp(i), g.qs, c);  // own cell, opposite population
-            const bool b0 = (m0 >> opp(i)) & 1u, b1 = (m1 >> opp(i)) & 1u;
-            if (ex(i) == 0) {
-                if (b0 == b1) {
-                    Stor<S>::ld2(b0 ? Po : Pi + x0, s[i].x, s[i].y);
-                } else {
-                    s[i].x = Stor<S>::ld(b0 ? Po : Pi + x0);
-                    s[i].y = Stor<S>::ld(b1 ? Po + 1 : Pi + x0 + 1);
-                }
-            } else {
-                s[i].x = Stor<S>::ld(b0 ? Po : Pi + (ex(i) > 0 ? xa : xb));
-                s[i].y = Stor<S>::ld(b1 ? Po + 1 : Pi + (ex(i) > 0 ? x0 : xc));
-            }
-        } else if (ex(i) == 0) {
+        if (ex(i) == 0) {
             Rows::ld2(Pi + x0, s[i].x, s[i].y);
         } else {
             s[i].x = Rows::ld(Pi + (ex(i) > 0 ? xa : xb));
@@ -979,6 +1043,84 @@ __global__ void __launch_bounds__(256, StepBlocks<S>::value)
 }
 
 // ---------------------------------------------------------------------------
+// The fused step in FP64 storage, one cell a thread (a warp's 8-byte loads of
+// 32 consecutive cells fill whole lines): gather with the mask-guided reload,
+// moments and collision in fixed point (lbm_fixed.cuh), store whole sectors
+// (a solid cell stores zeros nobody reads). Threads take the cells of the
+// fluid box's rows in order, across row ends. I: 32-bit lattice offsets where
+// they fit. RED: also the totals of the pre-collision state, per block.
+constexpr int STEP64_BLOCKS = 2;
+template <bool FLAGS, int FORCE, bool RECORD, bool RED, class I>
+__global__ void __launch_bounds__(256, STEP64_BLOCKS)
+    k_step64(const Dev d, const double *__restrict__ src, double *__restrict__ dst, double *__restrict__ out) {
+    // (as k_step: a programmatic dependent of the kernel before it)
+    if (STEP_PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (STEP_PDL) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const Geom &g = d.g;
+    const int bz = d.zrev ? (int)gridDim.y - 1 - (int)blockIdx.y : (int)blockIdx.y;
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    const int r = k / g.nx;
+    PairTotals<double> tot;
+    if (RED) tot.clear();
+    if (r < d.P.nyr) {
+        const int x = k - r * g.nx, y = d.P.y0 + r, z = d.P.z0 + bz;
+        const int c = cell_index(g, x, y, z);
+        const uint32_t m = FLAGS ? __ldg(d.mask + c) : 0u;
+        const bool live = !(m & SOLID_BIT);
+        const int xa = wrap1(x - 1, g.nx), xb = wrap1(x + 1, g.nx);
+        double s[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            s[i] = __ldg(GlobalRows<LBM_F64, I>{src}.row(g, i, y, z) + (ex(i) == 0 ? x : (ex(i) > 0 ? xa : xb)));
+        if (FLAGS && live && (m & 0x7fffeu)) {
+            // bounced populations come from the cell's own opposite slots
+#pragma unroll
+            for (int i = 1; i < Q; ++i)
+                if ((m >> opp(i)) & 1u) s[i] = __ldg(lat_at<I>(src, opp(i), g.qs, c));
+            if (d.moving_on && (m & MOVING_BIT)) {
+                int xm = x, ym = y, zm = z;
+                forget(xm, ym, zm);
+#pragma unroll
+                for (int i = 1; i < Q; ++i)
+                    if (((m >> opp(i)) & 1u) && d.flags[pull_src(g, xm, ym, zm, i)] == 2) s[i] += d.wc[i];
+            }
+        }
+        if (!FLAGS || live) {
+            double Fx = 0.0, Fy = 0.0, Fz = 0.0;
+            if (FORCE == 1) {
+                Fx = d.F[0];
+                Fy = d.F[1];
+                Fz = d.F[2];
+            } else if (FORCE == 2) {
+                const double *F = static_cast<const double *>(d.Ffield);
+                Fx = __ldg(F + c);
+                Fy = __ldg(F + g.qs + c);
+                Fz = __ldg(F + 2 * g.qs + c);
+            }
+            Cell64 mo;
+            cell64<FORCE != 0, true, RECORD || RED>(d, s, Fx, Fy, Fz, mo);
+            if (!(mo.rho > 0.0 && mo.rho < 1e30)) atomicOr(d.status, LBM_STATUS_DIVERGED);
+            if (RECORD) {
+                __stcs(out + c, mo.rho);
+                __stcs(out + g.qs + c, mo.ux);
+                __stcs(out + 2 * g.qs + c, mo.uy);
+                __stcs(out + 3 * g.qs + c, mo.uz);
+            }
+            if (RED) {
+                tot.v[0].x = mo.rho1;
+                tot.v[1].x = mo.jx;
+                tot.v[2].x = mo.jy;
+                tot.v[3].x = mo.jz;
+                tot.cells = 1;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < Q; ++i) *lat_at<I>(dst, i, g.qs, c) = !FLAGS || live ? s[i] : 0.0;
+    }
+    if (RED) block_partials(tot, out, blockIdx.y * gridDim.x + blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
 // The step with its source rows staged in shared memory by the Tensor Memory
 // Accelerator (FP32 and 16-bit storage). A cell row (y, z) pulls population
 // i from the one row (y - e_iy, z - e_iz) of array i, shifted by e_ix, so a
@@ -1340,8 +1482,15 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
     get2<RF>(u0 + N + cc, pair, has1, uy[0], uy[1]);
     get2<RF>(u0 + 2 * N + cc, pair, has1, uz[0], uz[1]);
     R f0[Q], f1[Q];
-    feq_all(f0, r[0] - R(1), ux[0], uy[0], uz[0], d.incomp);
-    feq_all(f1, r[1] - R(1), ux[1], uy[1], uz[1], d.incomp);
+    if constexpr (S == LBM_F64) {
+        if (!fixed_equilibrium(f0, r[0] - 1.0, ux[0], uy[0], uz[0], d.incomp))
+            feq_all(f0, r[0] - R(1), ux[0], uy[0], uz[0], d.incomp);
+        if (!fixed_equilibrium(f1, r[1] - 1.0, ux[1], uy[1], uz[1], d.incomp))
+            feq_all(f1, r[1] - R(1), ux[1], uy[1], uz[1], d.incomp);
+    } else {
+        feq_all(f0, r[0] - R(1), ux[0], uy[0], uz[0], d.incomp);
+        feq_all(f1, r[1] - R(1), ux[1], uy[1], uz[1], d.incomp);
+    }
     if (d.layout == LAYOUT_AA_NAT) {  // AA natural layout: f^0_i(x) at the cell itself
         const R nan = quiet_nan<R>();
 #pragma unroll
@@ -1577,7 +1726,7 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
         V s[Q], Fx, Fy, Fz;
         gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
         pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
-        const Mom2<R> m = moments2<R, FORCE>(s, Fx, Fy, Fz, d.incomp);
+        const Mom2<R> m = pair_moments<R, FORCE>(d, s, Fx, Fy, Fz);
         o[0] = m.rho;
         o[1] = m.ux;
         o[2] = m.uy;
@@ -1627,7 +1776,7 @@ __global__ void __launch_bounds__(RED_THREADS, FLAGS || is_split(S) ? 2 : FieldB
                 V s[Q], Fx, Fy, Fz;
                 gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
                 pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
-                tot.set(moments2<R, FORCE>(s, Fx, Fy, Fz, d.incomp), live0, live1);
+                tot.set(pair_moments<R, FORCE>(d, s, Fx, Fy, Fz), live0, live1);
             }
         }
         cells += tot.cells;
@@ -1708,7 +1857,7 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
     if (dL_drho) get2<RF>(dL_drho + cc, pair, has1, dr.x, dr.y);
     gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
     pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
-    const Mom2<R> m = moments2<R, FORCE>(s, Fx, Fy, Fz, d.incomp);
+    const Mom2<R> m = pair_moments<R, FORCE>(d, s, Fx, Fy, Fz);
     const V inv = d.incomp ? vsplat(R(1)) : vrcp(m.rho);
     const V gu = vfma(gz, m.uz, vfma(gy, m.uy, vmul(gx, m.ux)));
     const V base = d.incomp ? dr : vsub(dr, vmul(gu, inv));
@@ -1821,7 +1970,7 @@ template <int S> inline int tma_smem_bytes(const Dev &d) {
 // buffers fit.
 template <int S> inline bool tma_eligible(const Dev &d) {
     const long long rowbytes = (long long)d.g.pitch * sizeof(typename Stor<S>::T);
-    return d.row_staging && Bounce<S>::mode != BB_LOAD && rowbytes % 16 == 0 && tma_smem_bytes<S>(d) <= TMA_SMEM_MAX;
+    return d.row_staging && rowbytes % 16 == 0 && tma_smem_bytes<S>(d) <= TMA_SMEM_MAX;
 }
 
 template <int S, bool FLAGS, int FORCE, bool RECORD>
@@ -1846,14 +1995,44 @@ static cudaError_t launch_step_tma4(const Dev &d, const void *src, void *dst, vo
     return cudaGetLastError();
 }
 
+// FP64: one cell a thread over the box rows; 32-bit offsets where they fit.
+// RED: out is the partials (4 doubles per block), else the tape or null.
+inline dim3 step64_grid(const Dev &d) {
+    return dim3((unsigned)(((long long)d.P.nyr * d.g.nx + 255) / 256), d.P.nzr);
+}
+template <bool FLAGS, int FORCE, bool RECORD, bool RED>
+static cudaError_t launch_step64(const Dev &d, const void *src, void *dst, void *out) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = step64_grid(d);
+    cfg.blockDim = dim3(256);
+    cfg.stream = d.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = STEP_PDL;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const double *a = static_cast<const double *>(src);
+    double *b = static_cast<double *>(dst), *o = static_cast<double *>(out);
+    const cudaError_t e =
+        (long long)Q * d.g.qs < (1LL << 32)
+            ? cudaLaunchKernelEx(&cfg, k_step64<FLAGS, FORCE, RECORD, RED, unsigned>, d, a, b, o)
+            : cudaLaunchKernelEx(&cfg, k_step64<FLAGS, FORCE, RECORD, RED, long long>, d, a, b, o);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <int S, bool FLAGS, int FORCE>
 static cudaError_t launch_step3_any(const Dev &d, const void *src, void *dst, void *tape) {
-    if constexpr (!is_split(S)) {  // (the moment-split formats have no staged form)
-        if (tma_eligible<S>(d))
-            return tape ? launch_step_tma4<S, FLAGS, FORCE, true>(d, src, dst, tape)
-                        : launch_step_tma4<S, FLAGS, FORCE, false>(d, src, dst, tape);
+    if constexpr (S == LBM_F64) {
+        return tape ? launch_step64<FLAGS, FORCE, true, false>(d, src, dst, tape)
+                    : launch_step64<FLAGS, FORCE, false, false>(d, src, dst, nullptr);
+    } else {
+        if constexpr (!is_split(S)) {  // (the moment-split formats have no staged form)
+            if (tma_eligible<S>(d))
+                return tape ? launch_step_tma4<S, FLAGS, FORCE, true>(d, src, dst, tape)
+                            : launch_step_tma4<S, FLAGS, FORCE, false>(d, src, dst, tape);
+        }
+        return launch_step3<S, FLAGS, FORCE>(d, src, dst, tape);
     }
-    return launch_step3<S, FLAGS, FORCE>(d, src, dst, tape);
 }
 
 template <int S, bool FLAGS>
@@ -1916,30 +2095,46 @@ template <int S>
 cudaError_t Ops<S>::step_reduce(const Dev &d, const void *src, void *dst, double *partials, double *out) {
     typedef typename Stor<S>::T T;
     if (d.flags && !d.mask) return cudaErrorInvalidValue;
-    const T *s = static_cast<const T *>(src);
-    T *t = static_cast<T *>(dst);
-    // the launch mapping of the plain step (launch_step3)
-    const bool flat = d.flat_step || (d.flags ? flat_preferred<S, true>() : flat_preferred<S, false>());
-    const RowLaunch &P = flat ? d.PF : d.P;
-    const dim3 grid(P.nxb * P.nyb, P.nzr), block(P.bx_threads, P.by_threads);
-    if constexpr (is_split(S)) {  // (always the flat launch)
-        if (d.g.nx & 1)
-            launch_step_reduce2<S, true, true>(d, grid, block, s, t, partials);
+    if constexpr (S == LBM_F64) {
+        cudaError_t e;
+        if (d.flags)
+            e = d.Ffield ? launch_step64<true, 2, false, true>(d, src, dst, partials)
+                         : (d.force_on ? launch_step64<true, 1, false, true>(d, src, dst, partials)
+                                       : launch_step64<true, 0, false, true>(d, src, dst, partials));
         else
-            launch_step_reduce2<S, true, false>(d, grid, block, s, t, partials);
-    } else if (flat) {
-        launch_step_reduce2<S, true, false>(d, grid, block, s, t, partials);
+            e = d.Ffield ? launch_step64<false, 2, false, true>(d, src, dst, partials)
+                         : (d.force_on ? launch_step64<false, 1, false, true>(d, src, dst, partials)
+                                       : launch_step64<false, 0, false, true>(d, src, dst, partials));
+        if (e != cudaSuccess) return e;
+        const dim3 grid = step64_grid(d);
+        const int n = (int)(grid.x * grid.y);
+        return sum_partials(partials, n, partials + 4 * (size_t)n, out, d.stream);
     } else {
-        launch_step_reduce2<S, false, false>(d, grid, block, s, t, partials);
+        const T *s = static_cast<const T *>(src);
+        T *t = static_cast<T *>(dst);
+        // the launch mapping of the plain step (launch_step3)
+        const bool flat = d.flat_step || (d.flags ? flat_preferred<S, true>() : flat_preferred<S, false>());
+        const RowLaunch &P = flat ? d.PF : d.P;
+        const dim3 grid(P.nxb * P.nyb, P.nzr), block(P.bx_threads, P.by_threads);
+        if constexpr (is_split(S)) {  // (always the flat launch)
+            if (d.g.nx & 1)
+                launch_step_reduce2<S, true, true>(d, grid, block, s, t, partials);
+            else
+                launch_step_reduce2<S, true, false>(d, grid, block, s, t, partials);
+        } else if (flat) {
+            launch_step_reduce2<S, true, false>(d, grid, block, s, t, partials);
+        } else {
+            launch_step_reduce2<S, false, false>(d, grid, block, s, t, partials);
+        }
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (d.flags && LinkBounce<S>::value && d.link_max > 0) {
+            const int per_block = 256 * LINKS_PER_THREAD;
+            k_bounce<S><<<dim3(Q - 1, (d.link_max + per_block - 1) / per_block), 256, 0, d.stream>>>(d, t);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+        return sum_partials(partials, (int)(grid.x * grid.y), partials + 4 * (size_t)grid.x * grid.y, out, d.stream);
     }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (d.flags && LinkBounce<S>::value && d.link_max > 0) {
-        const int per_block = 256 * LINKS_PER_THREAD;
-        k_bounce<S><<<dim3(Q - 1, (d.link_max + per_block - 1) / per_block), 256, 0, d.stream>>>(d, t);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    return sum_partials(partials, (int)(grid.x * grid.y), partials + 4 * (size_t)grid.x * grid.y, out, d.stream);
 }
 
 // NaN marks on every slot of every solid cell (NaN-mark form; no-op otherwise).

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "lbm_device.cuh"
+#include "lbm_fixed.cuh"
 
 namespace lbm {
 
@@ -27,8 +28,7 @@ struct Dev {
     const uint32_t *mask;  // padded [qs] push masks (SOLID_BIT, bounce bits), null iff flags is
     const void *Ffield;    // padded [3][qs] of R, or nullptr
     double F[3];           // uniform force (used when Ffield == nullptr)
-    double gA[9], gC[9];   // Guo constants of the uniform force per opposite pair (see guo2)
-    float gAf[9], gCf[9];  // the same, rounded to float
+    float gAf[9], gCf[9];  // Guo constants of the uniform force per opposite pair (see guo2)
     float gAtf[9], gCtf[9];  // the same over omega, rounded to float (the FP32 form of collide2)
     bool has_moving;       // some cell is a moving wall (flag 2)
     bool moving_on;        // has_moving and the wall velocity is nonzero
@@ -39,6 +39,7 @@ struct Dev {
     int link_max;          // largest per-direction count
     bool force_on;         // Ffield != nullptr or F != 0
     double omega;          // 1 / tau
+    FixedK fk;             // the FP64 collision's constants
     double cs;             // tau - 1/2: the Guo factor 1 - omega/2 over omega
     float omega_f, cs_f;   // the same, and F, rounded to float on the host: a conversion from
     float F_f[3];          // double in every thread costs the narrow FP64 pipe (28% busy in the FP32 step)
@@ -67,14 +68,14 @@ template <> struct DevR<double> {
 };
 
 // Bounce-back form per storage format (see k_step), the measured fastest on
-// the walled channel: FP64 load side, FP32 mask-guided reload, 16-bit link
+// the walled channel: FP64 and FP32 mask-guided reload, 16-bit link
 // kernel (BB_NANS, NaN marks with a rho-gated fix-up, is kept as the
 // measured alternative). The moment-split formats take the mask-guided
 // reload: a bounced value is rebuilt from the cell's own momentum, which a
 // copy into a solid slot could not carry.
-enum { BB_LOAD = 0, BB_LINKS = 1, BB_NANS = 2, BB_MFIX = 3 };
+enum { BB_LINKS = 1, BB_NANS = 2, BB_MFIX = 3 };
 __host__ __device__ constexpr int bounce_mode(int s) {
-    return s == LBM_F64 ? BB_LOAD : ((s == LBM_F32 || is_split(s)) ? BB_MFIX : BB_LINKS);
+    return s == LBM_F64 || s == LBM_F32 || is_split(s) ? BB_MFIX : BB_LINKS;
 }
 // The form in which a solid cell's slot holds the value bounced into it, so
 // the gather needs no flags (links).
