@@ -237,13 +237,15 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
         }
     }
     const bool bounce_st = FLAGS && FREE_ST && ((m0 | m1) & 0x7fffeu);
-    const bool mv = FLAGS && d.moving_on && ((m0 | m1) & MOVING_BIT);
-    if (mv) {
+    const uint2 mv = FLAGS && d.moving_on && ((m0 | m1) & MOVING_BIT)
+                         ? moving_links(d, c, live0 ? m0 : 0u, live1 ? m1 : 0u)
+                         : make_uint2(0u, 0u);
+    if (mv.x | mv.y) {
         // bounced off a moving wall: plus 6 w_i (e_i . u_w)
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
-            if (((m0 >> opp(i)) & 1u) && d.flags[pull_src(g, x0, y, z, i)] == 2) s[i].x += wall_term<R>(d, i);
-            if (((m1 >> opp(i)) & 1u) && d.flags[pull_src(g, x0 + 1, y, z, i)] == 2) s[i].y += wall_term<R>(d, i);
+            if ((mv.x >> opp(i)) & 1u) s[i].x += wall_term<R>(d, i);
+            if ((mv.y >> opp(i)) & 1u) s[i].y += wall_term<R>(d, i);
         }
     }
     V Fx, Fy, Fz;
@@ -282,17 +284,15 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
             if (live1 && ((m1 >> i) & 1u)) Stor<S>::st(Po + 1, s[i].y);
         }
     }
-    if (mv) {
+    if (mv.x | mv.y) {
         // a population bounced back from a moving wall arrives as opp(i) and
         // carries 6 w_opp(i) (e_opp(i) . u_w) = -6 w_i (e_i . u_w): rewrite
         // the own slots just stored (same thread, so this store is the last)
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
             T *Po = A + (long long)opp(i) * qs + c;
-            if (live0 && ((m0 >> i) & 1u) && d.flags[push_dst(g, x0, y, z, i)] == 2)
-                Stor<S>::st(Po, s[i].x - wall_term<R>(d, i));
-            if (live1 && ((m1 >> i) & 1u) && d.flags[push_dst(g, x0 + 1, y, z, i)] == 2)
-                Stor<S>::st(Po + 1, s[i].y - wall_term<R>(d, i));
+            if ((mv.x >> i) & 1u) Stor<S>::st(Po, s[i].x - wall_term<R>(d, i));
+            if ((mv.y >> i) & 1u) Stor<S>::st(Po + 1, s[i].y - wall_term<R>(d, i));
         }
     }
 }

@@ -35,6 +35,7 @@ struct lbm_ctx {
     int box[4];         // y0, rows, z0, planes: the smallest y/z box holding every fluid cell
     uint8_t *flags_d;   // padded [qs], 1 = solid (padding included), or null
     uint32_t *mask_d;   // padded [qs] push masks for the step kernels, or null
+    uint32_t *moving_d; // padded [qs] moving-wall bits (contexts with cells flagged 2), or null
     uint32_t *links_d;  // bounce-back links (fluid cell, solid cell), grouped by direction
     int link_off[20];
     int link_max;
@@ -118,6 +119,7 @@ Dev make_dev(const lbm_ctx *ctx) {
     d.flat_step = rows_leave_lanes_idle(d.P);
     d.flags = ctx->flags_d;
     d.mask = ctx->mask_d;
+    d.moving = ctx->moving_d;
     d.Ffield = ctx->Ffield_d;
     d.F[0] = ctx->F[0];
     d.F[1] = ctx->F[1];
@@ -281,6 +283,7 @@ void free_ctx(lbm_ctx *ctx) {
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     drop_graphs(ctx);
     void *ptrs[] = {ctx->lat[0], ctx->lat[1],  ctx->flags_d,     ctx->mask_d,   ctx->links_d,        ctx->Ffield_d,
+                    ctx->moving_d,
                     ctx->lam[0], ctx->lam[1], ctx->red_partials, ctx->red_out, ctx->step_partials, ctx->status_d,
                     ctx->staging};
     for (void *p : ptrs)
@@ -348,6 +351,7 @@ lbm_status lbm_create(lbm_ctx **out, int nx, int ny, int nz, double tau, const u
     ctx->cur = 0;
     ctx->flags_d = nullptr;
     ctx->mask_d = nullptr;
+    ctx->moving_d = nullptr;
     ctx->links_d = nullptr;
     for (int j = 0; j < 20; ++j) ctx->link_off[j] = 0;
     ctx->link_max = 0;
@@ -442,6 +446,7 @@ lbm_status lbm_create(lbm_ctx **out, int nx, int ny, int nz, double tau, const u
               cudaMalloc((void **)&ctx->status_d, sizeof(unsigned)) == cudaSuccess;
     if (ok && flags) ok = cudaMalloc((void **)&ctx->flags_d, (size_t)qs) == cudaSuccess;
     if (ok && flags) ok = cudaMalloc((void **)&ctx->mask_d, (size_t)qs * sizeof(uint32_t)) == cudaSuccess;
+    if (ok && ctx->has_moving) ok = cudaMalloc((void **)&ctx->moving_d, (size_t)qs * sizeof(uint32_t)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         free_ctx(ctx);
@@ -455,7 +460,7 @@ lbm_status lbm_create(lbm_ctx **out, int nx, int ny, int nz, double tau, const u
         ok = cudaMemcpyAsync(ctx->flags_d, hflags.data(), (size_t)qs, cudaMemcpyHostToDevice, ctx->stream) ==
              cudaSuccess;
     // push masks, built on the device from the padded flags
-    if (ok && flags) ok = build_push_mask(ctx->g, ctx->flags_d, ctx->mask_d, ctx->stream) == cudaSuccess;
+    if (ok && flags) ok = build_push_mask(ctx->g, ctx->flags_d, ctx->mask_d, ctx->moving_d, ctx->stream) == cudaSuccess;
     if (ok && flags) {
         Dev d = make_dev(ctx);
         ok = LBM_DISPATCH(ctx, fill_solid(d, ctx->lat[0])) == cudaSuccess &&
@@ -942,7 +947,7 @@ static lbm_status ensure_lambda(lbm_ctx *ctx) {
             ctx->mask_d = nullptr;
             return fail(ctx, LBM_ERR_OOM, "cannot allocate the push masks");
         }
-        e = build_push_mask(ctx->g, ctx->flags_d, ctx->mask_d, ctx->stream);
+        e = build_push_mask(ctx->g, ctx->flags_d, ctx->mask_d, ctx->moving_d, ctx->stream);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "push mask build");
     }
     const size_t bytes = (size_t)Q * (size_t)ctx->g.qs * real_size(ctx->storage);

@@ -192,9 +192,17 @@ __device__ __forceinline__ void split_store(const Dev &d, typename Stor<S>::T *P
 // The same values, as if newly read: what a rare branch computes from them is
 // not computed ahead of it and kept in registers.
 __device__ __forceinline__ void forget(int &a) { asm volatile("" : "+r"(a)); }
-__device__ __forceinline__ void forget(int &a, int &b, int &c) { asm volatile("" : "+r"(a), "+r"(b), "+r"(c)); }
 
-__device__ __forceinline__ bool is_solid(const uint8_t *flags, int c) { return flags && flags[c]; }
+// The moving-wall bits of the pair at cell c among the bits of m0 and m1. One
+// dependent load: a flag load per bounced link put a chain of them on the
+// threads next to a lid, which the whole step of a small cavity waits for
+// (65x67x63: 9.3 us a step, 6.3 with these words).
+__device__ __forceinline__ uint2 moving_links(const Dev &d, int c, uint32_t m0, uint32_t m1) {
+    uint2 v = ld_resident2(d.moving + c);
+    v.x &= m0;
+    v.y &= m1;
+    return v;
+}
 
 // Moving-wall term of a population bounced into direction i: 6 w_i (e_i . u_w).
 template <class R> __device__ __forceinline__ R wall_term(const Dev &d, int i);
@@ -667,11 +675,12 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
         }
     }
     if (FLAGS && !LINKS && d.moving_on && ((m0 | m1) & MOVING_BIT)) {
-        // load side next to a moving wall: add its term to the bounced values
+        // next to a moving wall: add its term to the bounced values
+        const uint2 mv = moving_links(d, c, m0, m1);
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
-            if (((m0 >> opp(i)) & 1u) && d.flags[pull_src(g, x0, y, z, i)] == 2) s[i].x += wall_term<R>(d, i);
-            if (((m1 >> opp(i)) & 1u) && d.flags[pull_src(g, x0 + 1, y, z, i)] == 2) s[i].y += wall_term<R>(d, i);
+            if ((mv.x >> opp(i)) & 1u) s[i].x += wall_term<R>(d, i);
+            if ((mv.y >> opp(i)) & 1u) s[i].y += wall_term<R>(d, i);
         }
     }
     V Fx = vsplat(R(0)), Fy = vsplat(R(0)), Fz = vsplat(R(0));
@@ -700,11 +709,11 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
             const T *Po = lat_at<I>(src, opp(i), g.qs, c);
             if (live0 && s[i].x != s[i].x) {
                 s[i].x = Stor<S>::ld(Po);
-                if (d.moving_on && d.flags[pull_src(g, x0, y, z, i)] == 2) s[i].x += wall_term<R>(d, i);
+                if (d.moving_on && ((__ldg(d.moving + c) >> opp(i)) & 1u)) s[i].x += wall_term<R>(d, i);
             }
             if (live1 && s[i].y != s[i].y) {
                 s[i].y = Stor<S>::ld(Po + 1);
-                if (d.moving_on && d.flags[pull_src(g, x0 + 1, y, z, i)] == 2) s[i].y += wall_term<R>(d, i);
+                if (d.moving_on && ((__ldg(d.moving + c + 1) >> opp(i)) & 1u)) s[i].y += wall_term<R>(d, i);
             }
         }
         m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
@@ -767,18 +776,15 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
         // Links into a moving wall (not in the link list): slot opp(j) of the
         // wall cell x + e_j gets P_j(x) + 6 w_opp(j) (e_opp(j) . u_w), formed
         // from the unrounded P_j(x) so that it is rounded to storage once.
-        const uint2 mm = ld_resident2(d.mask + c);
-        if ((mm.x | mm.y) & MOVING_BIT) {
+        const uint2 mm = moving_links(d, c, live0 ? ~0u : 0u, live1 ? ~0u : 0u);
+        if (mm.x | mm.y) {
 #pragma unroll
             for (int j = 1; j < Q; ++j) {
-                if (live0 && ((mm.x >> j) & 1u)) {
-                    const int t = push_dst(g, x0, y, z, j);
-                    if (d.flags[t] == 2) Stor<S>::st(lat_at<I>(dst, opp(j), g.qs, t), s[j].x - wall_term<R>(d, j));
-                }
-                if (live1 && ((mm.y >> j) & 1u)) {
-                    const int t = push_dst(g, x0 + 1, y, z, j);
-                    if (d.flags[t] == 2) Stor<S>::st(lat_at<I>(dst, opp(j), g.qs, t), s[j].y - wall_term<R>(d, j));
-                }
+                if ((mm.x >> j) & 1u)
+                    Stor<S>::st(lat_at<I>(dst, opp(j), g.qs, push_dst(g, x0, y, z, j)), s[j].x - wall_term<R>(d, j));
+                if ((mm.y >> j) & 1u)
+                    Stor<S>::st(lat_at<I>(dst, opp(j), g.qs, push_dst(g, x0 + 1, y, z, j)),
+                                s[j].y - wall_term<R>(d, j));
             }
         }
     }
@@ -874,10 +880,11 @@ __device__ __forceinline__ void gather_pair_split(const Dev &d, const typename S
         }
     }
     if (FLAGS && d.moving_on && ((m0 | m1) & MOVING_BIT)) {
+        const uint2 mv = moving_links(d, c, m0, m1);
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
-            if (((m0 >> opp(i)) & 1u) && d.flags[pull_src(g, x0, y, z, i)] == 2) s[i].x += wall_term<R>(d, i);
-            if (((m1 >> opp(i)) & 1u) && d.flags[pull_src(g, x0 + 1, y, z, i)] == 2) s[i].y += wall_term<R>(d, i);
+            if ((mv.x >> opp(i)) & 1u) s[i].x += wall_term<R>(d, i);
+            if ((mv.y >> opp(i)) & 1u) s[i].y += wall_term<R>(d, i);
         }
     }
 }
@@ -1078,11 +1085,10 @@ __global__ void __launch_bounds__(256, STEP64_BLOCKS)
             for (int i = 1; i < Q; ++i)
                 if ((m >> opp(i)) & 1u) s[i] = __ldg(lat_at<I>(src, opp(i), g.qs, c));
             if (d.moving_on && (m & MOVING_BIT)) {
-                int xm = x, ym = y, zm = z;
-                forget(xm, ym, zm);
+                const uint32_t mv = __ldg(d.moving + c);
 #pragma unroll
                 for (int i = 1; i < Q; ++i)
-                    if (((m >> opp(i)) & 1u) && d.flags[pull_src(g, xm, ym, zm, i)] == 2) s[i] += d.wc[i];
+                    if ((mv >> opp(i)) & 1u) s[i] += d.wc[i];
             }
         }
         if (!FLAGS || live) {
@@ -1369,12 +1375,11 @@ __device__ __forceinline__ void gather_pair(const Dev &d, const typename Stor<S>
                 if ((m1 >> opp(i)) & 1u) s[i].y = Stor<S>::ld(Po + 1);
             }
             if (d.moving_on && ((m0 | m1) & MOVING_BIT)) {
-                forget(x0, y, z);
+                const uint2 mv = moving_links(d, c, m0, m1);
 #pragma unroll
                 for (int i = 1; i < Q; ++i) {
-                    if (((m0 >> opp(i)) & 1u) && d.flags[pull_src(g, x0, y, z, i)] == 2) s[i].x += wall_term<R>(d, i);
-                    if (((m1 >> opp(i)) & 1u) && d.flags[pull_src(g, x0 + 1, y, z, i)] == 2)
-                        s[i].y += wall_term<R>(d, i);
+                    if ((mv.x >> opp(i)) & 1u) s[i].x += wall_term<R>(d, i);
+                    if ((mv.y >> opp(i)) & 1u) s[i].y += wall_term<R>(d, i);
                 }
             }
         }
@@ -1442,6 +1447,7 @@ __global__ void __launch_bounds__(256)
     const int c = cell_index(g, x, y, z);
     const uint32_t m = FLAGS ? __ldg(d.mask + c) : 0u;
     if (m & SOLID_BIT) return;
+    const uint32_t mv = FLAGS && d.moving_on && (m & MOVING_BIT) ? __ldg(d.moving + c) : 0u;
     const long long N = d.n_cells, cc = canon_index(g, x, y, z);
     R v[Q];
 #pragma unroll
@@ -1451,7 +1457,7 @@ __global__ void __launch_bounds__(256)
         const R r1 = rho0 ? rho0[ct] - R(1) : R(0);
         v[i] = feq_shifted<R>(i, r1, bounce ? -u0[ct] : u0[ct], bounce ? -u0[N + ct] : u0[N + ct],
                               bounce ? -u0[2 * N + ct] : u0[2 * N + ct], d.incomp);
-        if (bounce && d.moving_on && d.flags[push_dst(g, x, y, z, i)] == 2) v[i] += wall_term<R>(d, i);
+        if (bounce && (mv >> i) & 1u) v[i] += wall_term<R>(d, i);
     }
     split_store<S>(d, P, x, c, v);
 }
@@ -1512,16 +1518,16 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
         }
     }
     if (FLAGS && ((m0 | m1) & 0x7fffeu)) {
-        forget(x0, y, z);
+        // (the gather adds the moving-wall term to a value bounced off a moving wall)
+        const uint2 mv = !bounce_in_solid(S) && d.moving_on && ((m0 | m1) & MOVING_BIT) ? moving_links(d, c, m0, m1)
+                                                                                       : make_uint2(0u, 0u);
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (!(((k ? m1 : m0) >> i) & 1u)) continue;
                 R v = k ? f1[opp(i)] : f0[opp(i)];
-                // (the gather adds the moving-wall term to a value bounced off a moving wall)
-                if (!bounce_in_solid(S) && d.moving_on && d.flags[push_dst(g, x0 + k, y, z, i)] == 2)
-                    v += wall_term<R>(d, i);
+                if (((k ? mv.y : mv.x) >> i) & 1u) v += wall_term<R>(d, i);
                 P[i * g.qs + c + k] = Rn<T>::of(v);
             }
         }
@@ -1628,7 +1634,9 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
             }
         }
     }
-    const bool mv = FLAGS && d.moving_on && d.layout == LAYOUT_PULL && ((m0 | m1) & MOVING_BIT);
+    const uint2 mv = FLAGS && d.has_moving && d.layout == LAYOUT_PULL && ((m0 | m1) & MOVING_BIT)
+                         ? moving_links(d, c, m0, m1)
+                         : make_uint2(0u, 0u);
     if constexpr (is_split(S)) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
@@ -1637,8 +1645,7 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 v[i] = (double)(k ? s1[i] : s0[i]);
-                if (mv && (((k ? m1 : m0) >> i) & 1u) && i > 0 && d.flags[push_dst(g, x0 + k, y, z, i)] == 2)
-                    v[i] += d.wc[i];
+                if (d.moving_on && (((k ? mv.y : mv.x) >> i) & 1u)) v[i] += d.wc[i];
             }
             split_store<S>(d, P, x0 + k, c + k, v);
         }
@@ -1665,17 +1672,15 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
         // cell: the solid slot that the link form pulls f_opp(i)(x) from; in
         // the other forms the gather adds the moving-wall term, taken off here
         // (summed in double, rounded once)
-        if (FLAGS && d.layout == LAYOUT_PULL && ((m0 | m1) & MOVING_BIT) && (mv || bounce_in_solid(S))) {
+        if (FLAGS && (mv.x | mv.y) && (d.moving_on || bounce_in_solid(S))) {
 #pragma unroll
             for (int i = 1; i < Q; ++i) {
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
-                    if (!(((k ? m1 : m0) >> i) & 1u)) continue;
+                    if (!(((k ? mv.y : mv.x) >> i) & 1u)) continue;
                     const V v = k ? s1[i] : s0[i];
-                    const int t = push_dst(g, x0 + k, y, z, i);
-                    if (d.flags[t] != 2) continue;
                     if (bounce_in_solid(S))
-                        P[(long long)opp(i) * g.qs + t] = Rn<T>::of(v);
+                        P[(long long)opp(i) * g.qs + push_dst(g, x0 + k, y, z, i)] = Rn<T>::of(v);
                     else
                         P[i * g.qs + c + k] = Rn<T>::of((double)v + d.wc[i]);
                 }

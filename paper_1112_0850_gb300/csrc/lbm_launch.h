@@ -26,6 +26,7 @@ struct Dev {
     bool flat_step;        // the two-grid step uses PF: whole rows would leave lanes idle
     const uint8_t *flags;  // padded [qs] (1 = solid, also on padding), or nullptr = all fluid
     const uint32_t *mask;  // padded [qs] push masks (SOLID_BIT, bounce bits), null iff flags is
+    const uint32_t *moving; // padded [qs], bit j: x + e_j is a moving wall (flag 2); null without such cells
     const void *Ffield;    // padded [3][qs] of R, or nullptr
     double F[3];           // uniform force (used when Ffield == nullptr)
     float gAf[9], gCf[9];  // Guo constants of the uniform force per opposite pair (see guo2)
@@ -140,8 +141,9 @@ template <int S> struct AaOps {
 // The sum of n partials (4 doubles each) in a fixed order, to out[4] (device).
 // scratch: room for SUM_BLOCKS more partials, or null (n is then small).
 cudaError_t sum_partials(double *partials, int n, double *scratch, double *out, cudaStream_t st);
-// Set-up: push masks of every padded cell from the padded flags (device).
-cudaError_t build_push_mask(const Geom &g, const uint8_t *flags, uint32_t *mask, cudaStream_t st);
+// Set-up: push masks of every padded cell from the padded flags (device), and
+// the moving-wall bits among them where `moving` is not null.
+cudaError_t build_push_mask(const Geom &g, const uint8_t *flags, uint32_t *mask, uint32_t *moving, cudaStream_t st);
 // z-slab halo copy between plane z of the lattice and a packed buffer of the
 // five populations with e_z = dir (lbm_halo.cu); unpack writes fluid cells only.
 cudaError_t launch_halo(const Geom &g, void *lat, int elem_bytes, void *buf, int z, int dir, bool unpack,
