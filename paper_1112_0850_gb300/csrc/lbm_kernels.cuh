@@ -209,67 +209,6 @@ template <class R> __device__ __forceinline__ R wall_term(const Dev &d, int i);
 template <> __device__ __forceinline__ float wall_term<float>(const Dev &d, int i) { return d.wcf[i]; }
 template <> __device__ __forceinline__ double wall_term<double>(const Dev &d, int i) { return d.wc[i]; }
 
-template <class R> __device__ __forceinline__ void force_at(const Dev &d, int c, R &Fx, R &Fy, R &Fz) {
-    if (d.Ffield) {
-        const R *F = static_cast<const R *>(d.Ffield);
-        Fx = F[c];
-        Fy = F[d.g.qs + c];
-        Fz = F[2 * d.g.qs + c];
-    } else {
-        Fx = DevR<R>::F(d, 0);
-        Fy = DevR<R>::F(d, 1);
-        Fz = DevR<R>::F(d, 2);
-    }
-}
-
-// Gather the 19 pre-collision populations of fluid cell (x, y, z) from P in
-// the layout d.layout. In the link form a solid source's slot already holds
-// the bounced value (what the next step will read), so the gather there
-// ignores flags; the AA swapped layout is the pull layout with slot i and
-// slot opp(i) exchanged.
-template <int S, bool FLAGS>
-__device__ __forceinline__ void gather(const Dev &d, const typename Stor<S>::T *P, int x, int y, int z,
-                                       int c, typename Stor<S>::R s[Q]) {
-    const long long qs = d.g.qs;
-    if constexpr (is_split(S)) {
-        // rebuild each value from its source cell's momentum word; a bounced
-        // one is the cell's own opposite value, rebuilt from its own word
-        const uint2 *J = split_words(d, P);
-        s[0] = Stor<S>::ld(P + c);
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            const int src = pull_src(d.g, x, y, z, i);
-            const uint8_t f = FLAGS ? d.flags[src] : 0;
-            if (!f) {
-                s[i] = __fmaf_rn(split_k(i), split_edot<S>(split_first(i), __ldg(J + src)),
-                                 Stor<S>::ld(P + (long long)i * qs + src));
-            } else {
-                s[i] = __fmaf_rn(split_k(opp(i)), split_edot<S>(split_first(i), __ldg(J + c)),
-                                 Stor<S>::ld(P + (long long)opp(i) * qs + c));
-                if (f == 2 && d.moving_on) s[i] += wall_term<typename Stor<S>::R>(d, i);
-            }
-        }
-        return;
-    }
-    if (d.layout == LAYOUT_AA_NAT) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) s[i] = Stor<S>::ld(P + (long long)i * qs + c);
-        return;
-    }
-    const bool mirror = d.layout == LAYOUT_AA_SWAP;
-    const bool flag_free = bounce_in_solid(S) && !mirror;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        int src = pull_src(d.g, x, y, z, i);
-        long long off = (long long)(mirror ? opp(i) : i) * qs + src;
-        uint8_t f = 0;
-        if (FLAGS && i > 0 && !flag_free) f = d.flags[src];
-        if (f) off = (long long)(mirror ? i : opp(i)) * qs + c;
-        s[i] = Stor<S>::ld(P + off);
-        if (f == 2 && d.moving_on) s[i] += wall_term<typename Stor<S>::R>(d, i);
-    }
-}
-
 // NaN marks solid slots in the NaN-mark form and in the AA pattern. (In the
 // AA pattern they are hygiene only: the odd step's mask-free scatter stores
 // into solid slots, and no reader takes a solid slot's value.)
@@ -1331,10 +1270,13 @@ __device__ __forceinline__ void pair_masks(const Dev &d, int c, bool has1, uint3
     }
 }
 
-// gather() for the pair (x0, x0 + 1) of row (y, z), with the push masks in
-// place of the neighbours' flags: every value is loaded from its source, and
-// pairs next to a solid then load their bounced values over it. (One mask word
-// a cell instead of 18 flag bytes, and loads that do not wait for them.)
+// The 19 pre-collision values of the fluid cells of the pair (x0, x0 + 1) of row
+// (y, z), from P in the layout d.layout: every value is loaded from its source,
+// and pairs next to a solid (m0, m1: their push masks) then load their bounced
+// values over it. In the link form a solid source's slot already holds the
+// bounced value (what the next step will read); the AA swapped layout is the
+// pull layout with slot i and slot opp(i) exchanged. (One mask word a cell
+// instead of 18 flag bytes, and loads that do not wait for them.)
 template <int S, bool FLAGS>
 __device__ __forceinline__ void gather_pair(const Dev &d, const typename Stor<S>::T *__restrict__ P, int x0, int y,
                                             int z, int c, bool has1, uint32_t m0, uint32_t m1,
@@ -1405,15 +1347,7 @@ template <int S, bool FLAGS> struct FieldBlocks {
 // the values of its 18 neighbours was bound by their 76 loads and by arithmetic
 // (FP64: its pipe 85% busy). Channel: FP32 165 to 111 us (floor 57), FP16 187 to
 // 86, FP64 2358 to 593; 256^3 box, FP32 435 to 288 us (floor 227).
-template <class R>
-__device__ __forceinline__ R feq_shifted(int i, R rho1, R ux, R uy, R uz, bool incomp) {
-    const R eu = R(ex(i)) * ux + R(ey(i)) * uy + R(ez(i)) * uz;
-    const R usq = ux * ux + uy * uy + uz * uz;
-    const R rho = incomp ? R(1) : R(1) + rho1;  // (He & Luo: velocity terms of the reference density)
-    return R(weight(i)) * (rho1 + rho * (R(3) * eu + R(4.5) * eu * eu - R(1.5) * usq));
-}
-
-// The 19 of a cell at once, opposite directions from their even and odd parts.
+// f_eq - w of one cell, opposite directions from their even and odd parts.
 template <class R> __device__ __forceinline__ void feq_all(R f[Q], R rho1, R ux, R uy, R uz, bool incomp) {
     const R rho = incomp ? R(1) : R(1) + rho1;
     const R usq = R(-1.5) * (ux * ux + uy * uy + uz * uz);
@@ -1429,37 +1363,129 @@ template <class R> __device__ __forceinline__ void feq_all(R f[Q], R rho1, R ux,
     }
 }
 
-__device__ __forceinline__ long long canon_neighbor(const Geom &g, int x, int y, int z, int i) {
-    return canon_index(g, wrap1(x + ex(i), g.nx), wrap1(y + ey(i), g.ny), wrap1(z + ez(i), g.nz));
+// Write the 19 shifted values v of a cell pair to a moment-split lattice:
+// their momentum rounded to the format, then the remainders against it (the
+// tail of step_pair_split, for values that are not a collision's).
+template <int S>
+__device__ __forceinline__ void split_store_pair(const Dev &d, typename Stor<S>::T *__restrict__ P, int x0, int c,
+                                                 bool has1, float2 v[Q]) {
+    const float2 jx = vadd(vadd(vadd(vsub(v[1], v[2]), vsub(v[7], v[10])), vadd(vsub(v[8], v[9]), vsub(v[11], v[14]))),
+                           vsub(v[12], v[13]));
+    const float2 jy = vadd(vadd(vadd(vsub(v[3], v[4]), vsub(v[7], v[10])), vadd(vsub(v[9], v[8]), vsub(v[15], v[18]))),
+                           vsub(v[16], v[17]));
+    const float2 jz = vadd(vadd(vadd(vsub(v[5], v[6]), vsub(v[11], v[14])), vadd(vsub(v[13], v[12]), vsub(v[15], v[18]))),
+                           vsub(v[17], v[16]));
+    const uint2 wa = make_uint2(SplitJ<S>::pack(jx.x, jy.x), SplitJ<S>::pack(jz.x, 0.0f));
+    const uint2 wb = make_uint2(SplitJ<S>::pack(jx.y, jy.y), SplitJ<S>::pack(jz.y, 0.0f));
+    const float2 tx = make_float2(SplitJ<S>::lo(wa.x), SplitJ<S>::lo(wb.x));
+    const float2 ty = make_float2(SplitJ<S>::hi(wa.x), SplitJ<S>::hi(wb.x));
+    const float2 tz = make_float2(SplitJ<S>::lo(wa.y), SplitJ<S>::lo(wb.y));
+#pragma unroll
+    for (int p = 0; p < NPAIR; ++p) {
+        const int i = pair_first(p), io = opp(i);
+        const float2 e = edot_first(i, tx, ty, tz);
+        v[i] = vfma(vsplat(-split_k(i)), e, v[i]);
+        v[io] = vfma(vsplat(-split_k(io)), e, v[io]);
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) Stor<S>::st2(P + i * d.g.qs + c, v[i].x, v[i].y);
+    uint2 *J = split_words(d, P);
+    if (has1)
+        *reinterpret_cast<uint4 *>(J + c) = make_uint4(wa.x, wa.y, wb.x, wb.y);
+    else  // the lone last cell of an odd row: the slot after it holds cell 0's copy
+        J[c] = wa;
+    split_ghost(d, J, x0, c, wa);
 }
 
-// Moment-split storage: the 19 values a cell holds, gathered from its
-// neighbours' fields, written as J and remainders; one cell a thread.
+// f_eq_i - w_i of two cells.
+__device__ __forceinline__ float2 feq_pair(int i, float2 r1, float2 ux, float2 uy, float2 uz, bool incomp) {
+    const float2 rho = incomp ? vsplat(1.0f) : vadd(vsplat(1.0f), r1);
+    const float2 usq = vmul(vsplat(-1.5f), vfma(uz, uz, vfma(uy, uy, vmul(ux, ux))));
+    const float w = i == 0 ? (float)(1.0 / 3.0) : (i <= 6 ? (float)(1.0 / 18.0) : (float)(1.0 / 36.0));
+    if (i == 0) return vmul(vsplat(w), vfma(rho, usq, r1));
+    // (the odd part joins in one rounding, with the momentum-exact 3 w of OddK)
+    const float2 e = edot_first(split_first(i), ux, uy, uz);
+    const float2 even = vmul(vsplat(w), vfma(rho, vfma(vmul(vsplat(4.5f), e), e, usq), r1));
+    return vfma(vmul(vsplat(split_k(i)), rho), e, even);
+}
+
+// Moment-split storage: the 19 values that the cells of a pair hold, formed from
+// their neighbours' fields (row by row: the pair and the cells left and right of
+// it), written as J and remainders. 256^3 box 411 us (floor 152); one cell a
+// thread with 76 field loads took 511.
 template <int S, bool FLAGS>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
     k_init_eq_split(const Dev d, typename Stor<S>::T *__restrict__ P, const float *__restrict__ rho0,
-                    const float *__restrict__ u0) {
-    typedef float R;
+                    const float *__restrict__ u0, bool pair) {
     const Geom &g = d.g;
-    int x, y, z;
-    if (!row_cell(g, d.L.nxb, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x, y, z))
+    int x0, y, z;
+    if (!pair_cell<true>(g, d.PF, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x0, y, z))
         return;
-    const int c = cell_index(g, x, y, z);
-    const uint32_t m = FLAGS ? __ldg(d.mask + c) : 0u;
-    if (m & SOLID_BIT) return;
-    const uint32_t mv = FLAGS && d.moving_on && (m & MOVING_BIT) ? __ldg(d.moving + c) : 0u;
-    const long long N = d.n_cells, cc = canon_index(g, x, y, z);
-    R v[Q];
+    const bool has1 = x0 + 1 < g.nx;
+    const int c = cell_index(g, x0, y, z);
+    uint32_t m0, m1;
+    bool live0, live1;
+    pair_masks<FLAGS>(d, c, has1, m0, m1, live0, live1);
+    if (FLAGS && !live0 && !live1) return;
+    const long long N = d.n_cells;
+    const int xa = wrap1(x0 - 1, g.nx), xb = wrap1(x0 + 1, g.nx), xc = wrap1(xb + 1, g.nx);
+    float2 v[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const bool bounce = FLAGS && i > 0 && ((m >> i) & 1u);
-        const long long ct = bounce ? cc : canon_neighbor(g, x, y, z, i);
-        const R r1 = rho0 ? rho0[ct] - R(1) : R(0);
-        v[i] = feq_shifted<R>(i, r1, bounce ? -u0[ct] : u0[ct], bounce ? -u0[N + ct] : u0[N + ct],
-                              bounce ? -u0[2 * N + ct] : u0[2 * N + ct], d.incomp);
-        if (bounce && (mv >> i) & 1u) v[i] += wall_term<R>(d, i);
+    for (int r = 0; r < 9; ++r) {
+        const int dy = r / 3 - 1, dz = r % 3 - 1;
+        const int row = (wrap1(z + dz, g.nz) * g.ny + wrap1(y + dy, g.ny)) * g.nx;
+        float2 f[4];  // rho - 1, u of cells x0, x0 + 1
+        float fa[4], fc[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            f[k] = vsplat(1.0f);
+            fa[k] = fc[k] = 1.0f;
+            if (k == 0 && !rho0) continue;
+            const float *p = (k ? u0 + (k - 1) * N : rho0) + row;
+            if (pair) {
+                ld2_real(p + x0, f[k].x, f[k].y);
+            } else {
+                f[k].x = __ldg(p + x0);
+                f[k].y = __ldg(p + xb);
+            }
+            if (dy == 0 || dz == 0) {
+                fa[k] = __ldg(p + xa);
+                fc[k] = __ldg(p + xc);
+            }
+        }
+        f[0] = vadd(f[0], vsplat(-1.0f));
+        fa[0] -= 1.0f;
+        fc[0] -= 1.0f;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            if (ey(i) != dy || ez(i) != dz) continue;
+            float2 q[4];  // the fields of x + e_i
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                q[k] = ex(i) == 0 ? f[k] : (ex(i) > 0 ? make_float2(f[k].y, fc[k]) : make_float2(fa[k], f[k].x));
+            v[i] = feq_pair(i, q[0], q[1], q[2], q[3], d.incomp);
+        }
     }
-    split_store<S>(d, P, x, c, v);
+    if (FLAGS && ((m0 | m1) & 0x7fffeu)) {  // next to a solid: the cell's own opposite value
+        const long long cc = canon_index(g, x0, y, z);
+        float2 f[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            f[k] = vsplat(1.0f);
+            if (k || rho0) get2<LBM_F32>((k ? u0 + (k - 1) * N : rho0) + cc, false, has1, f[k].x, f[k].y);
+        }
+        f[0] = vadd(f[0], vsplat(-1.0f));
+        const uint2 mv = d.moving_on && ((m0 | m1) & MOVING_BIT) ? moving_links(d, c, m0, m1) : make_uint2(0u, 0u);
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+            float2 o = feq_pair(opp(i), f[0], f[1], f[2], f[3], d.incomp);
+            if ((mv.x >> i) & 1u) o.x += d.wcf[i];
+            if ((mv.y >> i) & 1u) o.y += d.wcf[i];
+            if ((m0 >> i) & 1u) v[i].x = o.x;
+            if ((m1 >> i) & 1u) v[i].y = o.y;
+        }
+    }
+    split_store_pair<S>(d, P, x0, c, has1, v);
 }
 
 template <int S, bool FLAGS>
@@ -1568,8 +1594,10 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
 
 // set_state: P_i(y) = s_i(y + e_i) if fluid there, else s_{opp(i)}(y). The
 // loads follow the reverse step's gather (sources y + e_i, the pair's own
-// values over them where a mask bit is set). Moment-split storage: the 19
-// values a cell holds, in double, one cell a thread.
+// values over them where a mask bit is set). Moment-split storage collects the
+// 19 values its cells hold, in FP32 unless they come as doubles: the remainders
+// are formed by one rounded multiply-add, as in the step, before their 16-bit
+// rounding (256^3 box from FP32 287 us; in double 3017).
 template <int S, int D, bool FLAGS>
 __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
     k_set_state(const Dev d, typename Stor<S>::T *__restrict__ P, const typename IOFmt<D>::T *__restrict__ in,
@@ -1637,7 +1665,18 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
     const uint2 mv = FLAGS && d.has_moving && d.layout == LAYOUT_PULL && ((m0 | m1) & MOVING_BIT)
                          ? moving_links(d, c, m0, m1)
                          : make_uint2(0u, 0u);
-    if constexpr (is_split(S)) {
+    if constexpr (is_split(S) && sizeof(V) == 4) {
+        if (FLAGS && !live0 && !live1) return;
+        float2 v[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            v[i] = make_float2(s0[i], s1[i]);
+            if (d.moving_on && ((mv.x >> i) & 1u)) v[i].x += d.wcf[i];
+            if (d.moving_on && ((mv.y >> i) & 1u)) v[i].y += d.wcf[i];
+        }
+        split_store_pair<S>(d, P, x0, c, has1, v);
+        return;
+    } else if constexpr (is_split(S)) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             if (!(k ? live1 : live0)) continue;
@@ -2167,12 +2206,15 @@ cudaError_t Ops<S>::init_eq(const Dev &d0, void *lat, const void *rho0, const vo
     typedef typename Stor<S>::R R;
     if (d0.flags && !d0.mask) return cudaErrorInvalidValue;
     if constexpr (is_split(S)) {
-        if (d0.flags)
-            k_init_eq_split<S, true><<<row_grid(d0), row_block(d0), 0, d0.stream>>>(
-                d0, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0));
+        Dev d = d0;
+        d.PF = all_pairs(d.g);
+        const bool pair = pair_aligned(d.g, u0, sizeof(R)) && (!rho0 || pair_aligned(d.g, rho0, sizeof(R)));
+        if (d.flags)
+            k_init_eq_split<S, true><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
+                d, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0), pair);
         else
-            k_init_eq_split<S, false><<<row_grid(d0), row_block(d0), 0, d0.stream>>>(
-                d0, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0));
+            k_init_eq_split<S, false><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(
+                d, static_cast<T *>(lat), static_cast<const R *>(rho0), static_cast<const R *>(u0), pair);
     } else {
         Dev d = d0;
         d.PF = all_pairs(d.g);
