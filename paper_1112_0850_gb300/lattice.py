@@ -60,6 +60,7 @@ class Lattice:
             fl = np.ascontiguousarray(np.asarray(flags.cpu() if torch.is_tensor(flags) else flags), dtype=np.uint8)
             assert fl.shape == self.shape, (fl.shape, self.shape)
         self._flags_host = fl
+        self.has_moving_walls = fl is not None and bool((fl == 2).any())
         F = None if force is None else (ctypes.c_double * 3)(*[float(v) for v in force])
         h = ctypes.c_void_p()
         st = L.lbm_create(ctypes.byref(h), int(nx), int(ny), int(nz), float(tau),
@@ -119,6 +120,10 @@ class Lattice:
     def zeros(self, *lead, dtype=None, device="cuda"):
         return torch.zeros(*lead, *self.shape, dtype=dtype or self.real, device=device)
 
+    def empty(self, *lead, dtype=None, device="cuda"):
+        """For results that a call writes whole (solid cells included)."""
+        return torch.empty(*lead, *self.shape, dtype=dtype or self.real, device=device)
+
     # -- the calls of include/lbm_capi.h ------------------------------------
     def set_uniform_force(self, force):
         F = None if force is None else (ctypes.c_double * 3)(*[float(v) for v in force])
@@ -151,9 +156,9 @@ class Lattice:
 
     def macros(self, rho=None, u=None, with_rho=True):
         if u is None:
-            u = self.zeros(3)
+            u = self.empty(3)
         if rho is None and with_rho:
-            rho = self.zeros()
+            rho = self.empty()
         self._call("lbm_macros", self._ptr(rho, self.real, self.shape), self._ptr(u, self.real, (3,) + self.shape))
         return rho, u
 
@@ -268,9 +273,9 @@ class Lattice:
 
     def adjoint_init_grad(self, u0, rho0=None, grad_u0=None, grad_rho0=None, with_rho=False):
         if grad_u0 is None:
-            grad_u0 = self.zeros(3)
+            grad_u0 = self.empty(3)
         if grad_rho0 is None and with_rho:
-            grad_rho0 = self.zeros()
+            grad_rho0 = self.empty()
         self._call("lbm_adjoint_init_grad", self._ptr(rho0, self.real, self.shape),
                    self._ptr(u0, self.real, (3,) + self.shape), self._ptr(grad_u0, self.real, (3,) + self.shape),
                    self._ptr(grad_rho0, self.real, self.shape))

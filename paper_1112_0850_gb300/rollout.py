@@ -10,12 +10,23 @@ state every `ckpt_every` steps (in format `ckpt_fmt`), the backward pass
 restores each checkpoint, recomputes its segment while recording the moments
 the adjoint needs (lbm_step_record), and then runs the segment's adjoint
 steps in reverse. Memory: one checkpoint per segment plus one segment's tape.
+Where the checkpoints hold the lattice's values exactly, the last segment's
+recomputation ends on the final state itself, and no copy of that is kept.
 Checkpoints default to the lattice's own storage format; a moment-split
 lattice (whose canonical state has no exact 16-bit form) keeps FP32 ones.
 """
 import torch
 
 from . import capi
+
+
+def _replays_exactly(lat, own, fmt):
+    """Whether a run restored from a checkpoint in format fmt repeats bit for
+    bit: the format holds the lattice's values, and no wall moves (values bounced
+    off one are stored without its term, rounded again)."""
+    if lat.storage in (capi.LBM_F16M, capi.LBM_BF16M) or lat.has_moving_walls:
+        return False
+    return fmt == own or fmt == capi.LBM_F64 or (fmt == capi.LBM_F32 and own != capi.LBM_F64)
 
 
 class LBMRollout(torch.autograd.Function):
@@ -36,7 +47,7 @@ class LBMRollout(torch.autograd.Function):
             ckpts.append((lat.get_state(fmt), n))
             lat.step(n)
             done += n
-        final = lat.get_state(own)
+        final = None if ckpts and _replays_exactly(lat, own, fmt) else lat.get_state(own)
         _, u = lat.macros(with_rho=False)
         ctx.lat = lat
         ctx.ckpts = ckpts
@@ -50,13 +61,17 @@ class LBMRollout(torch.autograd.Function):
         lat = ctx.lat
         u0, F = ctx.saved_tensors
         lat.set_force_field(F)
-        lat.set_state(ctx.final)
         grad_F = torch.zeros_like(F)
-        lat.adjoint_seed(grad_u.contiguous().to(lat.real), None, grad_F)
+        dL_du = grad_u.contiguous().to(lat.real)
+        if ctx.final is not None:
+            lat.set_state(ctx.final)
+            lat.adjoint_seed(dL_du, None, grad_F)
         tape = lat.new_tape(ctx.K)
-        for state, n in reversed(ctx.ckpts):
+        for k, (state, n) in enumerate(reversed(ctx.ckpts)):
             lat.set_state(state)
             lat.step_record(n, tape)
+            if k == 0 and ctx.final is None:
+                lat.adjoint_seed(dL_du, None, grad_F)
             lat.adjoint_step(n, tape, grad_F)
         grad_u0, _ = lat.adjoint_init_grad(u0)
         return grad_u0, grad_F, None, None, None, None
