@@ -372,21 +372,22 @@ static cudaError_t launch_adj_step(const Dev &d, const void *li, void *lo, const
 // FP32: one cell per thread over the cells of the fluid box's rows.
 template <bool FLAGS>
 static cudaError_t launch_adj_step1(const Dev &d, const void *li, void *lo, const void *tape, void *gF) {
-    const dim3 grid((unsigned)(((long long)d.P.nyr * d.g.nx + 255) / 256), d.P.nzr);
+    const int t = small_lattice(d.P) ? 64 : 256;
+    const dim3 grid((unsigned)(((long long)d.P.nyr * d.g.nx + t - 1) / t), d.P.nzr);
     const float *a = static_cast<const float *>(li);
-    const float *t = static_cast<const float *>(tape);
+    const float *tp = static_cast<const float *>(tape);
     float *b = static_cast<float *>(lo), *G = static_cast<float *>(gF);
     const bool small = (long long)Q * d.g.qs < (1LL << 31) && 3 * d.n_cells < (1LL << 31);
     if (small) {
         if (d.force_on)
-            k_adj_step1<FLAGS, true, int><<<grid, 256, 0, d.stream>>>(d, a, b, t, G);
+            k_adj_step1<FLAGS, true, int><<<grid, t, 0, d.stream>>>(d, a, b, tp, G);
         else
-            k_adj_step1<FLAGS, false, int><<<grid, 256, 0, d.stream>>>(d, a, b, t, G);
+            k_adj_step1<FLAGS, false, int><<<grid, t, 0, d.stream>>>(d, a, b, tp, G);
     } else {
         if (d.force_on)
-            k_adj_step1<FLAGS, true, long long><<<grid, 256, 0, d.stream>>>(d, a, b, t, G);
+            k_adj_step1<FLAGS, true, long long><<<grid, t, 0, d.stream>>>(d, a, b, tp, G);
         else
-            k_adj_step1<FLAGS, false, long long><<<grid, 256, 0, d.stream>>>(d, a, b, t, G);
+            k_adj_step1<FLAGS, false, long long><<<grid, t, 0, d.stream>>>(d, a, b, tp, G);
     }
     return cudaGetLastError();
 }

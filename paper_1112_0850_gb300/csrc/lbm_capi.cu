@@ -115,8 +115,8 @@ Dev make_dev(const lbm_ctx *ctx) {
     d.g = ctx->g;
     d.L = ctx->L;
     d.P = pair_launch(ctx->g, ctx->box[0], ctx->box[1], ctx->box[2], ctx->box[3]);
-    d.PF = flat_launch(d.P);
-    d.flat_step = rows_leave_lanes_idle(d.P);
+    d.PF = flat_launch(d.P, flat_threads(d.P));
+    d.flat_step = rows_leave_lanes_idle(d.P) || small_lattice(d.P);
     d.flags = ctx->flags_d;
     d.mask = ctx->mask_d;
     d.moving = ctx->moving_d;
@@ -770,7 +770,7 @@ static lbm_status ensure_step_partials(lbm_ctx *ctx, const Dev &d) {
     const size_t nb_rows = (size_t)d.P.nxb * d.P.nyb * d.P.nzr, nb_flat = (size_t)d.PF.nxb * d.PF.nyb * d.PF.nzr;
     size_t nb = nb_rows > nb_flat ? nb_rows : nb_flat;
     // (the FP64 two-grid step: one cell a thread)
-    const size_t nb_cells = ((size_t)d.P.nyr * d.g.nx + 255) / 256 * d.P.nzr;
+    const size_t nb_cells = ((size_t)d.P.nyr * d.g.nx + 63) / 64 * d.P.nzr;
     if (ctx->storage == LBM_F64 && nb_cells > nb) nb = nb_cells;
     if (ctx->step_partials_n >= nb) return LBM_OK;
     if (ctx->step_partials) {
@@ -1143,7 +1143,8 @@ int64_t lbm_check_launch_indices(int nx, int ny, int nz, lbm_storage fmt, int ro
     if (visited2 != N) ++bad;
     };
     walk_pairs(Prows, false);
-    walk_pairs(flat_launch(Prows), true);  // the two-grid step's launch when rows leave lanes idle
+    walk_pairs(flat_launch(Prows, 128), true);  // the two-grid step's launch when rows leave lanes idle
+    walk_pairs(flat_launch(Prows, 64), true);  // and of small lattices
     // the FP32 reverse step, one cell per thread over the box rows in order
     {
         long long visited1 = 0;

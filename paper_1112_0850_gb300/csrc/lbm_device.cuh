@@ -323,10 +323,9 @@ inline RowLaunch pair_launch(const Geom &g, int y0 = 0, int nyr = -1, int z0 = 0
 // pairs are not a multiple of 32 (n = 200: 28 of 128 threads). The flat launch
 // gives consecutive threads consecutive pairs of a plane's rows, across row
 // ends (with rows padded only to pairs, consecutive rows are adjacent in
-// memory, so such warps still load contiguous runs): blocks of threads x 1
-// (256 unless a kernel is compiled for another block size).
+// memory, so such warps still load contiguous runs): blocks of threads x 1.
 inline bool rows_leave_lanes_idle(const RowLaunch &P) { return P.nxb * P.bx_threads != P.W; }
-inline RowLaunch flat_launch(const RowLaunch &rows, int threads = 256) {
+inline RowLaunch flat_launch(const RowLaunch &rows, int threads) {
     RowLaunch L = rows;
     L.nxb = 1;
     L.bx_threads = threads;
@@ -334,6 +333,17 @@ inline RowLaunch flat_launch(const RowLaunch &rows, int threads = 256) {
     L.nyb = (int)(((long long)L.nyr * L.W + threads - 1) / threads);
     return L;
 }
+
+// Threads of a flat launch's blocks: 128, and 64 for small lattices, whose few
+// hundred blocks of 256 leave SMs idle or start a second wave for a handful of
+// them, so that a step is as long as one block's chain of loads. Us a step with
+// 256 / 128 / 64 threads: FP32 boxes 24^3 2.70 / 2.06 / 1.93, 32^3 2.70 / 2.06 /
+// 2.12, 48^3 4.71 / 2.89 / 3.02, 64^3 5.84 / 5.45 / 5.20, 80^3 8.95 / 8.65 / 8.56,
+// 96^3 17.4 / 17.2 / 17.2, 256^3 358.9 / 358.9 / 360.4; BF16 split 384^3 999 / 960 /
+// 955; FP16 256^3 208.2 / 205.3 / 205.7.
+constexpr long long SMALL_PAIRS = 300000;
+inline bool small_lattice(const RowLaunch &rows) { return (long long)rows.nyr * rows.nzr * rows.W <= SMALL_PAIRS; }
+inline int flat_threads(const RowLaunch &rows) { return small_lattice(rows) ? 64 : 128; }
 
 template <bool FLAT = false>
 LBM_HD bool pair_cell(const Geom &g, const RowLaunch &P, int bdx, int bdy, int bx, int bz, int tx, int ty, int &x0,

@@ -925,17 +925,20 @@ constexpr int STEP_PDL = 1;
 // Block shape of the step kernel: the flat FP32 step with 32-bit offsets runs
 // 7 blocks of 128 threads per SM (72 registers, no spills: 28 warps) instead
 // of 3 of 256 (80 registers: 24 warps), +1.1% on the walled channel; 4 blocks
-// of 256 (64 registers) spilled 48 bytes and lost 4%.
+// of 256 (64 registers) spilled 48 bytes and lost 4%. A force per cell needs more
+// registers: 6 blocks of 128 (80) for FP32, and 3 of 256 (80) instead of 4 for
+// 16-bit storage (384x256x256 porous channel, recorded step 484 to 428 us).
 template <int S, bool FLAT, bool U32> constexpr int step_threads() { return U32 && FLAT ? 128 : 256; }
-template <int S, bool FLAT, bool U32> constexpr int step_min_blocks() {
-    return U32 && FLAT ? 7 : StepBlocks<S>::value;
+template <int S, int FORCE, bool FLAT, bool U32> constexpr int step_min_blocks() {
+    if (U32 && FLAT) return FORCE == 2 ? 6 : 7;
+    return FORCE == 2 && StepBlocks<S>::value == 4 ? 3 : StepBlocks<S>::value;
 }
 
 // FLAT: the launch of d.PF (pairs in plane order), else of d.P (whole rows).
 // ODD (moment-split formats only): rows of odd length, whose last cell is
 // alone in its pair (see split_ghost). U32: 32-bit lattice offsets (lat_at).
 template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT = false, bool ODD = false, bool U32 = false>
-__global__ void __launch_bounds__(step_threads<S, FLAT, U32>(), step_min_blocks<S, FLAT, U32>())
+__global__ void __launch_bounds__(step_threads<S, FLAT, U32>(), step_min_blocks<S, FORCE, FLAT, U32>())
     k_step(const Dev d, const typename Stor<S>::T *__restrict__ src, typename Stor<S>::T *__restrict__ dst,
            typename Stor<S>::R *__restrict__ tape) {
     // launched as a programmatic dependent: wait for the kernel before it (the
@@ -970,7 +973,7 @@ __global__ void __launch_bounds__(step_threads<S, FLAT, U32>(), step_min_blocks<
 // the lattice or not, reaches the block reduction; partials[4 b + k] of block
 // b = blockIdx.y * gridDim.x + blockIdx.x, summed in a fixed order.
 template <int S, bool FLAGS, int FORCE, bool FLAT, bool ODD = false>
-__global__ void __launch_bounds__(256, StepBlocks<S>::value)
+__global__ void __launch_bounds__(256, step_min_blocks<S, FORCE, FLAT, false>())
     k_step_reduce(const Dev d, const typename Stor<S>::T *__restrict__ src, typename Stor<S>::T *__restrict__ dst,
                   double *__restrict__ partials) {
     if (FLAGS && LinkBounce<S>::value) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -994,17 +997,18 @@ __global__ void __launch_bounds__(256, StepBlocks<S>::value)
 // moments and collision in fixed point (lbm_fixed.cuh), store whole sectors
 // (a solid cell stores zeros nobody reads). Threads take the cells of the
 // fluid box's rows in order, across row ends. I: 32-bit lattice offsets where
-// they fit. RED: also the totals of the pre-collision state, per block.
-constexpr int STEP64_BLOCKS = 2;
+// they fit. RED: also the totals of the pre-collision state, per block. 5 blocks
+// of 128 threads per SM (<= 102 registers): channel 312 us a step, against 332
+// with 2 of 256 (125 registers) and 322 with 4 of 128.
 template <bool FLAGS, int FORCE, bool RECORD, bool RED, class I>
-__global__ void __launch_bounds__(256, STEP64_BLOCKS)
+__global__ void __launch_bounds__(128, 5)
     k_step64(const Dev d, const double *__restrict__ src, double *__restrict__ dst, double *__restrict__ out) {
     // (as k_step: a programmatic dependent of the kernel before it)
     if (STEP_PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (STEP_PDL) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const Geom &g = d.g;
     const int bz = d.zrev ? (int)gridDim.y - 1 - (int)blockIdx.y : (int)blockIdx.y;
-    const int k = blockIdx.x * 256 + threadIdx.x;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int r = k / g.nx;
     PairTotals<double> tot;
     if (RED) tot.clear();
@@ -1250,7 +1254,10 @@ __global__ void __launch_bounds__(256) k_bounce(const Dev d, typename Stor<S>::T
 // ---------------------------------------------------------------------------
 // Readers and writers of the whole lattice run on the flat paired launch over
 // all rows (solid ones too): two x-adjacent cells per thread, d.PF.
-inline RowLaunch all_pairs(const Geom &g) { return flat_launch(pair_launch(g)); }
+inline RowLaunch all_pairs(const Geom &g) {
+    const RowLaunch rows = pair_launch(g);
+    return flat_launch(rows, flat_threads(rows));
+}
 inline dim3 pairs_grid(const RowLaunch &P) { return dim3(P.nyb, P.nzr); }
 
 // The push masks of the pair at cell c, 0 for a cell that is solid or past the
@@ -1947,14 +1954,8 @@ static cudaError_t launch_step3f(const Dev &d, const void *src, void *dst, void 
     typedef typename Stor<S>::T T;
     typedef typename Stor<S>::R R;
     if constexpr (!U32 && S == LBM_F32 && FLAGS) {
-        if (step_u32<S, FLAGS>(d)) {
-            if constexpr (FLAT && step_threads<S, true, true>() != 256) {
-                Dev d2 = d;  // the same pairs in blocks of the kernel's size
-                d2.PF = flat_launch(d.P, step_threads<S, true, true>());
-                return launch_step3f<S, FLAGS, FORCE, FLAT, ODD, true>(d2, src, dst, tape);
-            }
-            return launch_step3f<S, FLAGS, FORCE, FLAT, ODD, true>(d, src, dst, tape);
-        }
+        // (the flat launch's blocks hold at most 128 threads, step_threads)
+        if (step_u32<S, FLAGS>(d)) return launch_step3f<S, FLAGS, FORCE, FLAT, ODD, true>(d, src, dst, tape);
     }
     const RowLaunch &P = FLAT ? d.PF : d.P;
     const dim3 grid(P.nxb * P.nyb, P.nzr), block(P.bx_threads, P.by_threads);
@@ -2041,14 +2042,16 @@ static cudaError_t launch_step_tma4(const Dev &d, const void *src, void *dst, vo
 
 // FP64: one cell a thread over the box rows; 32-bit offsets where they fit.
 // RED: out is the partials (4 doubles per block), else the tape or null.
+inline int step64_threads(const Dev &d) { return small_lattice(d.P) ? 64 : 128; }
 inline dim3 step64_grid(const Dev &d) {
-    return dim3((unsigned)(((long long)d.P.nyr * d.g.nx + 255) / 256), d.P.nzr);
+    const int t = step64_threads(d);
+    return dim3((unsigned)(((long long)d.P.nyr * d.g.nx + t - 1) / t), d.P.nzr);
 }
 template <bool FLAGS, int FORCE, bool RECORD, bool RED>
 static cudaError_t launch_step64(const Dev &d, const void *src, void *dst, void *out) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = step64_grid(d);
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3(step64_threads(d));
     cfg.stream = d.stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -45,7 +45,7 @@ def test_fp64_step_against_extended_precision(pattern, kind, force, incomp):
     rng = np.random.default_rng(7)
     shape = (19, nz, ny, nx)
     s = rng.standard_normal(shape) * np.asarray(w)[:, None, None, None]
-    scale = {"small": 0.03, "edge": 0.0, "beyond": 3.0, "tiny": 1e-200, "mixed": 0.0}[kind]
+    scale = {"small": 0.03, "edge": 0.0, "beyond": 0.5, "tiny": 1e-200, "mixed": 0.0}[kind]
     if kind == "edge":  # cells on either side of each limit
         s *= rng.uniform(0.1, 0.8, (1, nz, ny, nx))
         s[3][s[3] > 0.05] = 0.25
@@ -54,6 +54,8 @@ def test_fp64_step_against_extended_precision(pattern, kind, force, incomp):
         s *= 10.0 ** rng.uniform(-300, -2, shape)
     else:
         s *= scale
+        if kind == "beyond":  # a density near 3/2, all of it above rest in the rest population
+            s[0] += 0.5
     s[:, 0, 0, :9] = 0.0
     F = force * max(scale, 1e-200 if kind == "tiny" else 0.1) * np.array([1.0, -0.5, 0.25])
     lat = Lattice(nx, ny, nz, tau, force=F if force else None, storage="f64", pattern=pattern,
