@@ -23,10 +23,9 @@
 // opp(j) of the push mask, i.e. x + e_opp(j) is solid too) population j is
 // read from slot j of x itself, and population opp(j) is written back there.
 // Solid cells' values are never used; the even step stores their lanes with
-// the rest of the pair (whole 32-byte sectors). The odd step's two forms
-// (aa_odd_pair) either leave solid cells alone or let a solid lane load
-// values it discards (slots a neighbour may be rewriting) and let fluid
-// cells store into solid slots that only they read.
+// the rest of the pair (whole 32-byte sectors). The odd step (aa_odd_pair) lets
+// every lane load values it discards (a solid lane slots that a neighbour may be
+// rewriting) and lets fluid cells store into solid slots that no one reads.
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -78,10 +77,19 @@ __device__ __forceinline__ void pair_check_record(const Dev &d, int c, bool live
     }
 }
 
-// Even step (natural -> swapped): local, every access an aligned pair.
-// FLAT (both AA kernels): the launch of d.PF (pairs in plane order), else of d.P.
+// The AA kernels are launched as programmatic dependents of the step before them
+// (see k_step): wait for it to complete, then let the next one be scheduled.
+__device__ __forceinline__ void aa_dependent() {
+    if (STEP_PDL) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+}
+
+// Even step (natural -> swapped): local, every access an aligned pair; the flat
+// launch (whole rows: FP16 channel 76.9 us, mean with the odd step, against 75.6).
 // RED: also hand out the pair's pre-collision totals.
-template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT, bool RED>
+template <int S, bool FLAGS, int FORCE, bool RECORD, bool RED>
 __device__ __forceinline__ void aa_even_pair(const Dev &d, typename Stor<S>::T *__restrict__ A,
                                              typename Stor<S>::R *__restrict__ tape,
                                              PairTotals<typename Stor<S>::R> *tot) {
@@ -92,8 +100,7 @@ __device__ __forceinline__ void aa_even_pair(const Dev &d, typename Stor<S>::T *
     // flags the 16-bit forms spill 16 more bytes at 64 registers for it (the
     // 512^3 box lost 2.4%, and a lattice that size keeps no plane in L2)
     const int bz = FLAGS && d.zrev ? (int)gridDim.y - 1 - (int)blockIdx.y : (int)blockIdx.y;
-    if (!pair_cell<FLAT>(d.g, FLAT ? d.PF : d.P, blockDim.x, blockDim.y, blockIdx.x, bz, threadIdx.x, threadIdx.y,
-                         x0, y, z))
+    if (!pair_cell<true>(d.g, d.PF, blockDim.x, blockDim.y, blockIdx.x, bz, threadIdx.x, threadIdx.y, x0, y, z))
         return;
     const long long qs = d.g.qs;
     const int c = cell_index(d.g, x0, y, z);
@@ -136,68 +143,61 @@ __device__ __forceinline__ void aa_even_pair(const Dev &d, typename Stor<S>::T *
     }
 }
 
-template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT>
-__global__ void __launch_bounds__(256, StepBlocks<S>::value)
+template <int S, bool FLAGS, int FORCE, bool RECORD>
+__global__ void __launch_bounds__(128, 2 * StepBlocks<S>::value)
     k_aa_even(const Dev d, typename Stor<S>::T *__restrict__ A, typename Stor<S>::R *__restrict__ tape) {
-    aa_even_pair<S, FLAGS, FORCE, RECORD, FLAT, false>(d, A, tape, nullptr);
+    aa_dependent();
+    aa_even_pair<S, FLAGS, FORCE, RECORD, false>(d, A, tape, nullptr);
 }
 
 // The even step with the totals of its pre-collision state summed per block
 // (every thread, in the lattice or not, reaches the block sum).
-template <int S, bool FLAGS, int FORCE, bool FLAT>
-__global__ void __launch_bounds__(256, StepBlocks<S>::value)
+template <int S, bool FLAGS, int FORCE>
+__global__ void __launch_bounds__(128, 2 * StepBlocks<S>::value)
     k_aa_even_reduce(const Dev d, typename Stor<S>::T *__restrict__ A, double *__restrict__ partials) {
+    aa_dependent();
     PairTotals<typename Stor<S>::R> tot;
     tot.clear();
-    aa_even_pair<S, FLAGS, FORCE, false, FLAT, true>(d, A, nullptr, &tot);
+    aa_even_pair<S, FLAGS, FORCE, false, true>(d, A, nullptr, &tot);
     block_partials(tot, partials, blockIdx.y * gridDim.x + blockIdx.x);
 }
 
-// Resident 256-thread blocks per SM the odd step is compiled for. With flags
-// both of its forms (aa_odd_pair) need more registers: 2 blocks (128
-// registers) ran the walled channel at 33.2 vs 26.7 GFLUPS in FP16 with
-// selected addresses, and at 32.8 vs 32.1 in FP32 with the mask-free gather
-// (3 blocks spill about 110 bytes there).
-template <int S, bool FLAGS> struct AaOddBlocks {
-    static constexpr int value = S == LBM_F64 ? 1 : (FLAGS ? 2 : StepBlocks<S>::value);
-};
-
 // Odd step (swapped -> natural): gather from the neighbours, scatter to them.
 // Halfway bounce-back (push mask bit j: x + e_j is solid):
-//  - loads: population i comes from slot i of x itself when bit opp(i) is set,
-//    from slot opp(i) of x - e_i otherwise; every load address is a select,
-//    so the gather is one branch-free sequence that waits for the mask.
-//  - stores, in one of two forms per storage format: selected (FP64), P_i(x)
-//    to slot opp(i) of x itself when bit i is set, else to slot i of x + e_i;
-//    or the mask-free scatter (FP32, 16-bit storage): every population of a
-//    live cell is stored to its neighbour's slot, a solid neighbour's
-//    included (slot i of a solid x + e_i is written by x alone and read by no
-//    one: x itself reads its own slot there), and the bounced ones are then
-//    stored to the cell's own slots.
-// Walled channel, GFLUPS, FP32 / FP16: selected stores 31.1 / 35.0, the
-// mask-free scatter 33.1 / 38.0. Also measured: a mask-free gather (every
-// population loaded from its neighbour without waiting for the mask, the
-// bounced ones reloaded from the own slots after) with the mask-free scatter
-// 32.8 / 32.1, with selected stores 30.9 / 33.2; a NaN-driven fix-up with
-// separate store paths twice as slow (its code size and divergence made it
-// instruction-bound).
-template <int S> __host__ __device__ constexpr bool aa_free_scatter() { return S != LBM_F64; }
+//  - loads: every population from slot opp(i) of x - e_i without waiting for the
+//    mask; a pair with a bounce bit then loads its bounced ones (bit opp(i)) from
+//    slot i of x itself over them.
+//  - stores: every population of a live cell to its neighbour's slot, a solid
+//    neighbour's included (slot i of a solid x + e_i is written by x alone and
+//    read by no one: x itself reads its own slot there), and the bounced ones
+//    then to the cell's own slots.
+// Always the flat launch, blocks of 128 threads, with 32-bit lattice offsets
+// where they fit (I). Walled channel, mean of an even and an odd step, us, FP32 /
+// FP16: 91.6 / 77.9 with 6 / 7 blocks per SM (80 / 72 registers; FP32 with a force
+// per cell 5: 108.1 against 110.9); 64-bit offsets 99.4 / 88.3; loads that select
+// their address by the mask instead 97.2 / 82.7, which with 64-bit offsets in 2
+// blocks of 256 (128 registers) were the former 103.4 / 92.5. Without flags, FP16
+// 256^3: 7 blocks 223.7, 8 226.4, 6 227.3 (a force per cell, 256x128x128: 73.2,
+// 76.1, 71.6).
+template <int S, bool FLAGS, int FORCE> constexpr int aa_odd_blocks() {
+    if (S == LBM_F64) return 2;
+    if (S == LBM_F32) return FLAGS && FORCE == 2 ? 5 : 6;
+    return FORCE == 2 && !FLAGS ? 6 : 7;
+}
 
-template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT, bool RED>
+template <int S, bool FLAGS, int FORCE, bool RECORD, bool RED, class I>
 __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *__restrict__ A,
                                             typename Stor<S>::R *__restrict__ tape,
                                              PairTotals<typename Stor<S>::R> *tot) {
     typedef typename Stor<S>::T T;
     typedef typename Stor<S>::R R;
     typedef typename Pair2<R>::V V;
-    constexpr bool FREE_ST = aa_free_scatter<S>();
     int x0, y, z;
     // alternating plane order (see k_step) on walled lattices only: without
     // flags the 16-bit forms spill 16 more bytes at 64 registers for it (the
     // 512^3 box lost 2.4%, and a lattice that size keeps no plane in L2)
     const int bz = FLAGS && d.zrev ? (int)gridDim.y - 1 - (int)blockIdx.y : (int)blockIdx.y;
-    if (!pair_cell<FLAT>(d.g, FLAT ? d.PF : d.P, blockDim.x, blockDim.y, blockIdx.x, bz, threadIdx.x, threadIdx.y,
-                         x0, y, z))
+    if (!pair_cell<true>(d.g, d.PF, blockDim.x, blockDim.y, blockIdx.x, bz, threadIdx.x, threadIdx.y, x0, y, z))
         return;
     const Geom &g = d.g;
     const long long qs = g.qs;
@@ -210,7 +210,6 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
         m1 |= mm.y;
     }
     const bool live0 = !(m0 & SOLID_BIT), live1 = !(m1 & SOLID_BIT);
-    if (!live0 && !live1) return;  // (the selected gather waits for the mask anyway)
     // neighbour columns: x0 - 1, x0 + 1, x0 + 2 (the last only for a full pair)
     const int xa = wrap1(x0 - 1, g.nx);
     const int xb = wrap1(x0 + 1, g.nx);
@@ -218,27 +217,27 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
     V s[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        // f_i(x) = slot opp(i) of x - e_i, or slot i of x if x - e_i is solid
-        const int row = (wrap1(z - ez(i), g.nz) * g.ny + wrap1(y - ey(i), g.ny)) * g.pitch;
-        const T *Pn = A + (long long)opp(i) * qs + row;
-        const T *Po = A + (long long)i * qs + c;
-        const bool b0 = FLAGS && i > 0 && ((m0 >> opp(i)) & 1u);
-        const bool b1 = FLAGS && i > 0 && ((m1 >> opp(i)) & 1u);
+        const T *Pn = lat_at<I>(A, opp(i), qs, (wrap1(z - ez(i), g.nz) * g.ny + wrap1(y - ey(i), g.ny)) * g.pitch);
         if (ex(i) == 0) {
-            if (b0 == b1) {
-                Stor<S>::ld2(b0 ? Po : Pn + x0, s[i].x, s[i].y);
-            } else {
-                s[i].x = Stor<S>::ld(b0 ? Po : Pn + x0);
-                s[i].y = Stor<S>::ld(b1 ? Po + 1 : Pn + x0 + 1);
-            }
+            Stor<S>::ld2(Pn + x0, s[i].x, s[i].y);
         } else {
-            s[i].x = Stor<S>::ld(b0 ? Po : Pn + (ex(i) > 0 ? xa : xb));
-            s[i].y = Stor<S>::ld(b1 ? Po + 1 : Pn + (ex(i) > 0 ? x0 : xc));
+            s[i].x = Stor<S>::ld(Pn + (ex(i) > 0 ? xa : xb));
+            s[i].y = Stor<S>::ld(Pn + (ex(i) > 0 ? x0 : xc));
         }
     }
-    const bool bounce_st = FLAGS && FREE_ST && ((m0 | m1) & 0x7fffeu);
-    const uint2 mv = FLAGS && d.moving_on && ((m0 | m1) & MOVING_BIT)
-                         ? moving_links(d, c, live0 ? m0 : 0u, live1 ? m1 : 0u)
+    const uint32_t r0 = live0 ? m0 : 0u, r1 = live1 ? m1 : 0u;
+    const bool bounce = FLAGS && ((r0 | r1) & 0x7fffeu);
+    if (bounce) {
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+            const T *Po = lat_at<I>(A, i, qs, c);
+            if ((r0 >> opp(i)) & 1u) s[i].x = Stor<S>::ld(Po);
+            if ((r1 >> opp(i)) & 1u) s[i].y = Stor<S>::ld(Po + 1);
+        }
+    }
+    if (FLAGS && !live0 && !live1) return;
+    const uint2 mv = FLAGS && d.moving_on && ((r0 | r1) & MOVING_BIT)
+                         ? moving_links(d, c, r0, r1)
                          : make_uint2(0u, 0u);
     if (mv.x | mv.y) {
         // bounced off a moving wall: plus 6 w_i (e_i . u_w)
@@ -260,28 +259,24 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
     pair_check_record<R, RECORD>(d, c, live0, live1, m, tape);
     if constexpr (S != LBM_F64)
         collide2<R, FORCE != 0, relax_about_t(S)>(s, m, DevR<R>::omega(d), DevR<R>::cs(d), Fx, Fy, Fz, G, d.incomp);
-    // P_i(x) to slot i of x + e_i, or to slot opp(i) of x if x + e_i is solid
+    // P_i(x) to slot i of x + e_i
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const int row = (wrap1(z + ez(i), g.nz) * g.ny + wrap1(y + ey(i), g.ny)) * g.pitch;
-        T *Pn = A + (long long)i * qs + row;
-        T *Po = A + (long long)opp(i) * qs + c;
-        const bool b0 = FLAGS && !FREE_ST && i > 0 && ((m0 >> i) & 1u);
-        const bool b1 = FLAGS && !FREE_ST && i > 0 && ((m1 >> i) & 1u);
-        if (ex(i) == 0 && b0 == b1 && live0 && live1) {
-            Stor<S>::st2(b0 ? Po : Pn + x0, s[i].x, s[i].y);
+        T *Pn = lat_at<I>(A, i, qs, (wrap1(z + ez(i), g.nz) * g.ny + wrap1(y + ey(i), g.ny)) * g.pitch);
+        if (ex(i) == 0 && live0 && live1) {
+            Stor<S>::st2(Pn + x0, s[i].x, s[i].y);
         } else {
-            if (live0) Stor<S>::st(b0 ? Po : Pn + (ex(i) > 0 ? xb : (ex(i) < 0 ? xa : x0)), s[i].x);
-            if (live1) Stor<S>::st(b1 ? Po + 1 : Pn + (ex(i) > 0 ? xc : (ex(i) < 0 ? x0 : x0 + 1)), s[i].y);
+            if (live0) Stor<S>::st(Pn + (ex(i) > 0 ? xb : (ex(i) < 0 ? xa : x0)), s[i].x);
+            if (live1) Stor<S>::st(Pn + (ex(i) > 0 ? xc : (ex(i) < 0 ? x0 : x0 + 1)), s[i].y);
         }
     }
-    if (bounce_st) {
-        // the mask-free scatter's bounced values, to the own slots
+    if (bounce) {
+        // the bounced values, to the own slots
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
-            T *Po = A + (long long)opp(i) * qs + c;
-            if (live0 && ((m0 >> i) & 1u)) Stor<S>::st(Po, s[i].x);
-            if (live1 && ((m1 >> i) & 1u)) Stor<S>::st(Po + 1, s[i].y);
+            T *Po = lat_at<I>(A, opp(i), qs, c);
+            if ((r0 >> i) & 1u) Stor<S>::st(Po, s[i].x);
+            if ((r1 >> i) & 1u) Stor<S>::st(Po + 1, s[i].y);
         }
     }
     if (mv.x | mv.y) {
@@ -297,84 +292,69 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
     }
 }
 
-template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT>
-__global__ void __launch_bounds__(256, AaOddBlocks<S, FLAGS>::value)
+template <int S, bool FLAGS, int FORCE, bool RECORD, class I>
+__global__ void __launch_bounds__(128, aa_odd_blocks<S, FLAGS, FORCE>())
     k_aa_odd(const Dev d, typename Stor<S>::T *__restrict__ A, typename Stor<S>::R *__restrict__ tape) {
-    aa_odd_pair<S, FLAGS, FORCE, RECORD, FLAT, false>(d, A, tape, nullptr);
+    aa_dependent();
+    aa_odd_pair<S, FLAGS, FORCE, RECORD, false, I>(d, A, tape, nullptr);
 }
 
 // The odd step with the totals of its pre-collision state summed per block.
-template <int S, bool FLAGS, int FORCE, bool FLAT>
-__global__ void __launch_bounds__(256, AaOddBlocks<S, FLAGS>::value)
+template <int S, bool FLAGS, int FORCE, class I>
+__global__ void __launch_bounds__(128, S == LBM_F64 ? 2 : 5)
     k_aa_odd_reduce(const Dev d, typename Stor<S>::T *__restrict__ A, double *__restrict__ partials) {
+    aa_dependent();
     PairTotals<typename Stor<S>::R> tot;
     tot.clear();
-    aa_odd_pair<S, FLAGS, FORCE, false, FLAT, true>(d, A, nullptr, &tot);
+    aa_odd_pair<S, FLAGS, FORCE, false, true, I>(d, A, nullptr, &tot);
     block_partials(tot, partials, blockIdx.y * gridDim.x + blockIdx.x);
 }
 
-template <int S, bool FLAGS, int FORCE, bool FLAT>
-static cudaError_t launch_aa4(const Dev &d, void *A, int odd, void *tape) {
-    typedef typename Stor<S>::T T;
-    typedef typename Stor<S>::R R;
-    T *a = static_cast<T *>(A);
-    R *t = static_cast<R *>(tape);
-    const RowLaunch &P = FLAT ? d.PF : d.P;
-    const dim3 grid(P.nxb * P.nyb, P.nzr), block(P.bx_threads, P.by_threads);
-    if (odd) {
-        if (tape)
-            k_aa_odd<S, FLAGS, FORCE, true, FLAT><<<grid, block, 0, d.stream>>>(d, a, t);
-        else
-            k_aa_odd<S, FLAGS, FORCE, false, FLAT><<<grid, block, 0, d.stream>>>(d, a, nullptr);
-    } else {
-        if (tape)
-            k_aa_even<S, FLAGS, FORCE, true, FLAT><<<grid, block, 0, d.stream>>>(d, a, t);
-        else
-            k_aa_even<S, FLAGS, FORCE, false, FLAT><<<grid, block, 0, d.stream>>>(d, a, nullptr);
-    }
-    return cudaGetLastError();
+// Both steps run on the flat launch; the odd one with 32-bit offsets where all 19
+// arrays fit them.
+inline bool aa_narrow(const Dev &d) { return (long long)Q * d.g.qs < (1LL << 32); }
+inline dim3 aa_grid(const Dev &d) { return dim3(d.PF.nyb, d.PF.nzr); }
+
+template <int S, bool FLAGS, int FORCE, bool RECORD>
+static cudaError_t launch_aa3(const Dev &d, void *A, int odd, void *tape) {
+    auto k = !odd ? k_aa_even<S, FLAGS, FORCE, RECORD>
+                  : (aa_narrow(d) ? k_aa_odd<S, FLAGS, FORCE, RECORD, unsigned>
+                                  : k_aa_odd<S, FLAGS, FORCE, RECORD, long long>);
+    return launch_dependent(k, aa_grid(d), dim3(d.PF.bx_threads), d.stream, d, static_cast<typename Stor<S>::T *>(A),
+                            static_cast<typename Stor<S>::R *>(tape));
 }
 
-// The AA kernels run flat only where whole rows would leave lanes idle (with
-// whole-warp rows their flat forms compile to no fewer spills).
 template <int S, bool FLAGS, int FORCE>
-static cudaError_t launch_aa3(const Dev &d, void *A, int odd, void *tape) {
-    return d.flat_step ? launch_aa4<S, FLAGS, FORCE, true>(d, A, odd, tape)
-                       : launch_aa4<S, FLAGS, FORCE, false>(d, A, odd, tape);
+static cudaError_t launch_aa_tape(const Dev &d, void *A, int odd, void *tape) {
+    return tape ? launch_aa3<S, FLAGS, FORCE, true>(d, A, odd, tape)
+                : launch_aa3<S, FLAGS, FORCE, false>(d, A, odd, nullptr);
 }
 
 template <int S, bool FLAGS>
 static cudaError_t launch_aa2(const Dev &d, void *A, int odd, void *tape) {
-    if (d.Ffield) return launch_aa3<S, FLAGS, 2>(d, A, odd, tape);
-    if (d.force_on) return launch_aa3<S, FLAGS, 1>(d, A, odd, tape);
-    return launch_aa3<S, FLAGS, 0>(d, A, odd, tape);
+    if (d.Ffield) return launch_aa_tape<S, FLAGS, 2>(d, A, odd, tape);
+    if (d.force_on) return launch_aa_tape<S, FLAGS, 1>(d, A, odd, tape);
+    return launch_aa_tape<S, FLAGS, 0>(d, A, odd, tape);
 }
 
-template <int S, bool FLAGS, int FORCE, bool FLAT>
-static cudaError_t launch_aa_reduce4(const Dev &d, void *A, int odd, double *partials, double *out) {
-    typedef typename Stor<S>::T T;
-    T *a = static_cast<T *>(A);
-    const RowLaunch &P = FLAT ? d.PF : d.P;
-    const dim3 grid(P.nxb * P.nyb, P.nzr), block(P.bx_threads, P.by_threads);
-    if (odd)
-        k_aa_odd_reduce<S, FLAGS, FORCE, FLAT><<<grid, block, 0, d.stream>>>(d, a, partials);
-    else
-        k_aa_even_reduce<S, FLAGS, FORCE, FLAT><<<grid, block, 0, d.stream>>>(d, a, partials);
-    cudaError_t e = cudaGetLastError();
+template <int S, bool FLAGS, int FORCE>
+static cudaError_t launch_aa_reduce3(const Dev &d, void *A, int odd, double *partials, double *out) {
+    auto k = !odd ? k_aa_even_reduce<S, FLAGS, FORCE>
+                  : (aa_narrow(d) ? k_aa_odd_reduce<S, FLAGS, FORCE, unsigned>
+                                  : k_aa_odd_reduce<S, FLAGS, FORCE, long long>);
+    const dim3 grid = aa_grid(d);
+    const cudaError_t e = launch_dependent(k, grid, dim3(d.PF.bx_threads), d.stream, d,
+                                           static_cast<typename Stor<S>::T *>(A), partials);
     if (e != cudaSuccess) return e;
-    return sum_partials(partials, (int)(grid.x * grid.y), partials + 4 * (size_t)grid.x * grid.y, out, d.stream);
+    const int n = (int)(grid.x * grid.y);
+    return sum_partials(partials, n, partials + 4 * (size_t)n, out, d.stream);
 }
 
 template <int S, bool FLAGS>
 static cudaError_t launch_aa_reduce2(const Dev &d, void *A, int odd, double *partials, double *out) {
-    if (d.Ffield)
-        return d.flat_step ? launch_aa_reduce4<S, FLAGS, 2, true>(d, A, odd, partials, out)
-                           : launch_aa_reduce4<S, FLAGS, 2, false>(d, A, odd, partials, out);
-    if (d.force_on)
-        return d.flat_step ? launch_aa_reduce4<S, FLAGS, 1, true>(d, A, odd, partials, out)
-                           : launch_aa_reduce4<S, FLAGS, 1, false>(d, A, odd, partials, out);
-    return d.flat_step ? launch_aa_reduce4<S, FLAGS, 0, true>(d, A, odd, partials, out)
-                       : launch_aa_reduce4<S, FLAGS, 0, false>(d, A, odd, partials, out);
+    if (d.Ffield) return launch_aa_reduce3<S, FLAGS, 2>(d, A, odd, partials, out);
+    if (d.force_on) return launch_aa_reduce3<S, FLAGS, 1>(d, A, odd, partials, out);
+    return launch_aa_reduce3<S, FLAGS, 0>(d, A, odd, partials, out);
 }
 
 template <int S>

@@ -1977,6 +1977,22 @@ template <int S, bool FLAGS> inline bool step_u32(const Dev &d) {
     return S == LBM_F32 && FLAGS && (long long)Q * d.g.qs < (1LL << 32);
 }
 
+// Launch k as a programmatic dependent of the kernel before it on the stream.
+template <class... P, class... A>
+static cudaError_t launch_dependent(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = STEP_PDL;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <int S, bool FLAGS, int FORCE, bool FLAT, bool ODD = false, bool U32 = false>
 static cudaError_t launch_step3f(const Dev &d, const void *src, void *dst, void *tape) {
     typedef typename Stor<S>::T T;
@@ -1987,31 +2003,9 @@ static cudaError_t launch_step3f(const Dev &d, const void *src, void *dst, void 
     }
     const RowLaunch &P = FLAT ? d.PF : d.P;
     const dim3 grid(P.nxb * P.nyb, P.nzr), block(P.bx_threads, P.by_threads);
-    if (STEP_PDL) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = grid;
-        cfg.blockDim = block;
-        cfg.stream = d.stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        cudaError_t e = tape ? cudaLaunchKernelEx(&cfg, k_step<S, FLAGS, FORCE, true, FLAT, ODD, U32>, d,
-                                                  static_cast<const T *>(src), static_cast<T *>(dst),
-                                                  static_cast<R *>(tape))
-                             : cudaLaunchKernelEx(&cfg, k_step<S, FLAGS, FORCE, false, FLAT, ODD, U32>, d,
-                                                  static_cast<const T *>(src), static_cast<T *>(dst), (R *)nullptr);
-        if (e != cudaSuccess) return e;
-        return cudaGetLastError();
-    }
-    if (tape)
-        k_step<S, FLAGS, FORCE, true, FLAT, ODD, U32><<<grid, block, 0, d.stream>>>(
-            d, static_cast<const T *>(src), static_cast<T *>(dst), static_cast<R *>(tape));
-    else
-        k_step<S, FLAGS, FORCE, false, FLAT, ODD, U32><<<grid, block, 0, d.stream>>>(
-            d, static_cast<const T *>(src), static_cast<T *>(dst), nullptr);
-    return cudaGetLastError();
+    return launch_dependent(tape ? k_step<S, FLAGS, FORCE, true, FLAT, ODD, U32> : k_step<S, FLAGS, FORCE, false, FLAT, ODD, U32>,
+                            grid, block, d.stream, d, static_cast<const T *>(src), static_cast<T *>(dst),
+                            static_cast<R *>(tape));
 }
 
 // The flat launch where whole rows would leave lanes idle, and also where it
@@ -2077,22 +2071,10 @@ inline dim3 step64_grid(const Dev &d) {
 }
 template <bool FLAGS, int FORCE, bool RECORD, bool RED>
 static cudaError_t launch_step64(const Dev &d, const void *src, void *dst, void *out) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = step64_grid(d);
-    cfg.blockDim = dim3(step64_threads(d));
-    cfg.stream = d.stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = STEP_PDL;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const double *a = static_cast<const double *>(src);
-    double *b = static_cast<double *>(dst), *o = static_cast<double *>(out);
-    const cudaError_t e =
-        (long long)Q * d.g.qs < (1LL << 32)
-            ? cudaLaunchKernelEx(&cfg, k_step64<FLAGS, FORCE, RECORD, RED, unsigned>, d, a, b, o)
-            : cudaLaunchKernelEx(&cfg, k_step64<FLAGS, FORCE, RECORD, RED, long long>, d, a, b, o);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    const bool narrow = (long long)Q * d.g.qs < (1LL << 32);
+    return launch_dependent(narrow ? k_step64<FLAGS, FORCE, RECORD, RED, unsigned> : k_step64<FLAGS, FORCE, RECORD, RED, long long>,
+                            step64_grid(d), dim3(step64_threads(d)), d.stream, d, static_cast<const double *>(src),
+                            static_cast<double *>(dst), static_cast<double *>(out));
 }
 
 template <int S, bool FLAGS, int FORCE>
