@@ -72,6 +72,7 @@ def kernel_source_hash():
     csrc = os.path.join(ROOT, "paper_1112_0850_gb300", "csrc")
     files = [os.path.join(csrc, n) for n in ("lbm_device.cuh", "lbm_launch.h", "lbm_kernels.cuh", "lbm_capi.cu",
                                               "lbm_setup.cu")]
+    files += glob.glob(os.path.join(csrc, "lbm_fixed.cuh"))  # (the FP64 collision)
     files += sorted(glob.glob(os.path.join(csrc, "lbm_ops_*.cu")))
     files.append(os.path.join(ROOT, "include", "lbm_capi.h"))
     h = hashlib.sha256()

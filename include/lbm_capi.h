@@ -233,8 +233,9 @@ lbm_status lbm_step_timed(lbm_ctx *ctx, int n, float *ms);
  * u: real [3][nz][ny][nx]. Solid cells read 0. */
 lbm_status lbm_macros(lbm_ctx *ctx, void *rho, void *u);
 
-/* Totals over fluid cells of the current state, accumulated in FP64 in a
- * fixed order (deterministic): out = {sum rho, sum rho u_x, sum rho u_y,
+/* Totals over fluid cells of the current state, deterministic: values of FP32
+ * arithmetic are summed exactly, as multiples of 2^-81 (those of 1024 or more,
+ * and FP64 values, in FP64 in a fixed order): out = {sum rho, sum rho u_x, sum rho u_y,
  * sum rho u_z} with rho u = j + F/2. out is a host array; synchronizes.
  * Returns LBM_ERR_DIVERGED (out still written) if the status word's
  * divergence bit is set. */

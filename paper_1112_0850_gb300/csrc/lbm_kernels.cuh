@@ -763,7 +763,8 @@ __device__ __forceinline__ void gather_pair_split(const Dev &d, const typename S
     }
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const T *Pi = src + (long long)i * g.qs + (wrap1(z - ez(i), g.nz) * g.ny + wrap1(y - ey(i), g.ny)) * g.pitch;
+        const T *Pi =
+            lat_at<long long>(src, i, g.qs, (wrap1(z - ez(i), g.nz) * g.ny + wrap1(y - ey(i), g.ny)) * g.pitch);
         V gi;
         if (ex(i) == 0) {
             Stor<S>::ld2(Pi + x0, gi.x, gi.y);
@@ -808,8 +809,8 @@ __device__ __forceinline__ void gather_pair_split(const Dev &d, const typename S
             const int i = pair_first(p), io = opp(i);
             const V e = edot_first(i, ox, oy, oz);
             V gi, gio;
-            Stor<S>::ld2(src + (long long)i * g.qs + c, gi.x, gi.y);
-            Stor<S>::ld2(src + (long long)io * g.qs + c, gio.x, gio.y);
+            Stor<S>::ld2(lat_at<long long>(src, i, g.qs, c), gi.x, gi.y);
+            Stor<S>::ld2(lat_at<long long>(src, io, g.qs, c), gio.x, gio.y);
             const V ri = vfma(vsplat(split_k(io)), e, gio);
             const V rio = vfma(vsplat(split_k(i)), e, gi);
             s[i].x = ((m0 >> io) & 1u) ? ri.x : s[i].x;
@@ -906,7 +907,7 @@ __device__ __forceinline__ void step_pair_split(const Dev &d, const typename Sto
     // read: the mask-guided reload rebuilds bounced values from the fluid
     // cell's own slots), so 32-byte sectors are written complete.
 #pragma unroll
-    for (int i = 0; i < Q; ++i) Stor<S>::st2(dst + (long long)i * g.qs + c, s[i].x, s[i].y);
+    for (int i = 0; i < Q; ++i) Stor<S>::st2(lat_at<long long>(dst, i, g.qs, c), s[i].x, s[i].y);
     uint2 *Jd = split_words(d, dst);
     if (!ODD || has1)
         *reinterpret_cast<uint4 *>(Jd + c) = make_uint4(w0x, w0y, w1x, w1y);
@@ -922,23 +923,28 @@ __device__ __forceinline__ void step_pair_split(const Dev &d, const typename Sto
 // +0.5% when launched one by one (short runs), +0.2% in replayed graphs.
 constexpr int STEP_PDL = 1;
 
-// Block shape of the step kernel: the flat FP32 step with 32-bit offsets runs
-// 7 blocks of 128 threads per SM (72 registers, no spills: 28 warps) instead
-// of 3 of 256 (80 registers: 24 warps), +1.1% on the walled channel; 4 blocks
-// of 256 (64 registers) spilled 48 bytes and lost 4%. A force per cell needs more
-// registers: 6 blocks of 128 (80) for FP32, and 3 of 256 (80) instead of 4 for
-// 16-bit storage (384x256x256 porous channel, recorded step 484 to 428 us).
-template <int S, bool FLAT, bool U32> constexpr int step_threads() { return U32 && FLAT ? 128 : 256; }
-template <int S, int FORCE, bool FLAT, bool U32> constexpr int step_min_blocks() {
-    if (U32 && FLAT) return FORCE == 2 ? 6 : 7;
-    return FORCE == 2 && StepBlocks<S>::value == 4 ? 3 : StepBlocks<S>::value;
+// Block shape of the step kernel: the flat launch's blocks hold 128 threads at
+// most, whole rows 256. Blocks of 128 per SM, and what was measured (us a step):
+//  - FP32 with flags (32-bit offsets): 7 (72 registers, no spills: 28 warps)
+//    +1.1% on the walled channel over 3 of 256 (80 registers); 4 of 256 (64)
+//    spilled 48 bytes and lost 4%. A force per cell: 6 (80), channel 97.2 to 94.2.
+//  - moment split with flags: 7, BF16 channel 90.4 against 100.7 with 6; without
+//    flags 6, BF16 384^3 960 against 1030.
+//  - 16-bit: 8 (64); with a force per cell 6 (80), 200^3 FP16 117.5 against 125.4,
+//    porous channel (whole rows, 3 of 256), recorded, 430 against 484.
+template <bool FLAT> constexpr int step_threads() { return FLAT ? 128 : 256; }
+template <int S, bool FLAGS, int FORCE, bool FLAT, bool U32, bool RED = false> constexpr int step_min_blocks() {
+    const int rows = FORCE == 2 && StepBlocks<S>::value == 4 ? 3 : StepBlocks<S>::value;
+    if (!FLAT) return rows;
+    if (U32 || (is_split(S) && FLAGS && !RED)) return FORCE == 2 ? 6 : 7;
+    return 2 * rows;
 }
 
 // FLAT: the launch of d.PF (pairs in plane order), else of d.P (whole rows).
 // ODD (moment-split formats only): rows of odd length, whose last cell is
 // alone in its pair (see split_ghost). U32: 32-bit lattice offsets (lat_at).
 template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT = false, bool ODD = false, bool U32 = false>
-__global__ void __launch_bounds__(step_threads<S, FLAT, U32>(), step_min_blocks<S, FORCE, FLAT, U32>())
+__global__ void __launch_bounds__(step_threads<FLAT>(), step_min_blocks<S, FLAGS, FORCE, FLAT, U32>())
     k_step(const Dev d, const typename Stor<S>::T *__restrict__ src, typename Stor<S>::T *__restrict__ dst,
            typename Stor<S>::R *__restrict__ tape) {
     // launched as a programmatic dependent: wait for the kernel before it (the
@@ -973,7 +979,7 @@ __global__ void __launch_bounds__(step_threads<S, FLAT, U32>(), step_min_blocks<
 // the lattice or not, reaches the block reduction; partials[4 b + k] of block
 // b = blockIdx.y * gridDim.x + blockIdx.x, summed in a fixed order.
 template <int S, bool FLAGS, int FORCE, bool FLAT, bool ODD = false>
-__global__ void __launch_bounds__(256, step_min_blocks<S, FORCE, FLAT, false>())
+__global__ void __launch_bounds__(step_threads<FLAT>(), step_min_blocks<S, FLAGS, FORCE, FLAT, false, true>())
     k_step_reduce(const Dev d, const typename Stor<S>::T *__restrict__ src, typename Stor<S>::T *__restrict__ dst,
                   double *__restrict__ partials) {
     if (FLAGS && LinkBounce<S>::value) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
