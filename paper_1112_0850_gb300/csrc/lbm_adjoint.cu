@@ -230,21 +230,27 @@ __global__ void __launch_bounds__(256, AdjBlocks<R>::value)
 
 // The FP32 reverse step with one cell per thread: a warp's 4-byte loads of 32
 // consecutive cells already fill whole 128-byte lines, so FP32 needs no cell
-// pairs, and one cell's 19 adjoint populations, tape and gradient fit in 64
-// registers, so 4 blocks of 256 threads are resident per SM (the paired
-// kernel holds 2 at 128 registers, and its long-scoreboard waits were the
-// top stall). Threads take the cells of a plane's box rows in order, across
+// pairs, and one cell's 19 adjoint populations, tape and gradient fit in 56
+// registers, so 1152 threads are resident per SM (the paired kernel holds 512
+// at 128 registers, and its long-scoreboard waits were the top stall). Threads take the cells of a plane's box rows in order, across
 // row ends. A solid cell stores zeros (its slots are never read), so that
 // every 32-byte sector of a lattice row is written whole.
 // I: the index type of the lattice, tape and gradient offsets; int where
 // every offset fits (19 qs and 3 nx ny nz below 2^31), so that each address is
 // one 32-bit index and one wide multiply-add.
-constexpr int ADJ1_BLOCKS = 4;
+// Blocks of 128 threads per SM: 9 (56 registers) 871 us on the 384x256x256 porous
+// channel and 61.6 on a 128^3 box; 8 884 / 61.9, 7 881 / 61.7, 4 of 256 892 / 62.9.
+constexpr int ADJ1_THREADS = 128, ADJ1_BLOCKS = 9;
 
 template <bool FLAGS, bool FORCE, class I>
-__global__ void __launch_bounds__(256, ADJ1_BLOCKS)
+__global__ void __launch_bounds__(ADJ1_THREADS, ADJ1_BLOCKS)
     k_adj_step1(const Dev d, const float *__restrict__ lam_in, float *__restrict__ lam_out,
                 const float *__restrict__ tape, float *__restrict__ grad_F) {
+    // launched as a programmatic dependent of the kernel before it (the reverse
+    // step before, the seed, a recorded step): its blocks are scheduled as that
+    // one drains and wait here for it to complete (128^3: +1.1% of a gradient)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const Geom &g = d.g;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int r = k / g.nx;
@@ -372,24 +378,22 @@ static cudaError_t launch_adj_step(const Dev &d, const void *li, void *lo, const
 // FP32: one cell per thread over the cells of the fluid box's rows.
 template <bool FLAGS>
 static cudaError_t launch_adj_step1(const Dev &d, const void *li, void *lo, const void *tape, void *gF) {
-    const int t = small_lattice(d.P) ? 64 : 256;
-    const dim3 grid((unsigned)(((long long)d.P.nyr * d.g.nx + t - 1) / t), d.P.nzr);
-    const float *a = static_cast<const float *>(li);
-    const float *tp = static_cast<const float *>(tape);
-    float *b = static_cast<float *>(lo), *G = static_cast<float *>(gF);
     const bool small = (long long)Q * d.g.qs < (1LL << 31) && 3 * d.n_cells < (1LL << 31);
-    if (small) {
-        if (d.force_on)
-            k_adj_step1<FLAGS, true, int><<<grid, t, 0, d.stream>>>(d, a, b, tp, G);
-        else
-            k_adj_step1<FLAGS, false, int><<<grid, t, 0, d.stream>>>(d, a, b, tp, G);
-    } else {
-        if (d.force_on)
-            k_adj_step1<FLAGS, true, long long><<<grid, t, 0, d.stream>>>(d, a, b, tp, G);
-        else
-            k_adj_step1<FLAGS, false, long long><<<grid, t, 0, d.stream>>>(d, a, b, tp, G);
-    }
-    return cudaGetLastError();
+    auto k = small ? (d.force_on ? k_adj_step1<FLAGS, true, int> : k_adj_step1<FLAGS, false, int>)
+                   : (d.force_on ? k_adj_step1<FLAGS, true, long long> : k_adj_step1<FLAGS, false, long long>);
+    const int t = small_lattice(d.P) ? 64 : ADJ1_THREADS;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((long long)d.P.nyr * d.g.nx + t - 1) / t), d.P.nzr);
+    cfg.blockDim = dim3(t);
+    cfg.stream = d.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, d, static_cast<const float *>(li), static_cast<float *>(lo),
+                                             static_cast<const float *>(tape), static_cast<float *>(gF));
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <class R>
