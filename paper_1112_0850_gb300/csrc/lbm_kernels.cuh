@@ -1342,10 +1342,11 @@ __device__ __forceinline__ void gather_pair(const Dev &d, const typename Stor<S>
     }
 }
 
-// Resident 256-thread blocks per SM of the readers and writers, the measured
-// best of 2 and 3: FP64 2 (3 spilled: get_state of the channel 210 against 343
-// us), moment-split storage with flags 2 (macros 101 against 148 us), else 3
-// (FP16 channel, macros 65 against 75 us, set_state 95 against 133).
+// Resident pairs of 128-thread blocks per SM of the readers and writers, the
+// measured best of 2 and 3: FP64 2 (3 spilled: get_state of the channel 210
+// against 343 us), moment-split storage with flags 2 (macros 101 against 148
+// us), else 3 (FP16 channel, macros 65 against 75 us, set_state 95 against
+// 133); set_state with flags takes 7 single blocks (82.4 against 91).
 template <int S, bool FLAGS> struct FieldBlocks {
     static constexpr int value = S == LBM_F64 ? 2 : (FLAGS && is_split(S) ? 2 : 3);
 };
@@ -1425,10 +1426,11 @@ __device__ __forceinline__ float2 feq_pair(int i, float2 r1, float2 ux, float2 u
 
 // Moment-split storage: the 19 values that the cells of a pair hold, formed from
 // their neighbours' fields (row by row: the pair and the cells left and right of
-// it), written as J and remainders. 256^3 box 411 us (floor 152); one cell a
-// thread with 76 field loads took 511.
+// it), written as J and remainders. 256^3 box 378 us (floor 152), 399 with 6
+// blocks per SM; one cell a thread with 76 field loads took 511. Walled channel
+// with 5 blocks 137 us, 155 with 4.
 template <int S, bool FLAGS>
-__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
+__global__ void __launch_bounds__(128, FLAGS ? 5 : 7)
     k_init_eq_split(const Dev d, typename Stor<S>::T *__restrict__ P, const float *__restrict__ rho0,
                     const float *__restrict__ u0, bool pair) {
     const Geom &g = d.g;
@@ -1503,7 +1505,7 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
 }
 
 template <int S, bool FLAGS>
-__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
+__global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
     k_init_eq(const Dev d, typename Stor<S>::T *__restrict__ P, const typename Stor<S>::R *__restrict__ rho0,
               const typename Stor<S>::R *__restrict__ u0, bool pair) {
     typedef typename Stor<S>::R R;
@@ -1607,7 +1609,7 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
 // 18 flag loads and every value converted over double took 1622 us for the
 // 384x256x256 porous channel (FP16 to BF16: 1.9 GB, 0.17 of copy bandwidth).
 template <int S, int D, bool FLAGS>
-__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
+__global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
     k_get_state(const Dev d, const typename Stor<S>::T *__restrict__ P, typename IOFmt<D>::T *__restrict__ out,
                 bool pair) {
     typedef typename Stor<S>::R R;
@@ -1640,7 +1642,7 @@ __global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
 // are formed by one rounded multiply-add, as in the step, before their 16-bit
 // rounding (256^3 box from FP32 287 us; in double 3017).
 template <int S, int D, bool FLAGS>
-__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
+__global__ void __launch_bounds__(128, FLAGS && !is_split(S) && S != LBM_F64 ? 7 : 2 * FieldBlocks<S, FLAGS>::value)
     k_set_state(const Dev d, typename Stor<S>::T *__restrict__ P, const typename IOFmt<D>::T *__restrict__ in,
                 bool pair) {
     typedef typename Stor<S>::T T;
@@ -1791,7 +1793,7 @@ __device__ __forceinline__ void pair_force_at(const Dev &d, int c, typename Pair
 // Macroscopic fields (Sec. 2 step 1): rho and u = (j + F/2)/rho; solid 0.
 // Bound by HBM (19 values read, 4 reals written a cell).
 template <int S, bool FLAGS, bool FORCE>
-__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
+__global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
     k_macros(const Dev d, const typename Stor<S>::T *__restrict__ P, typename Stor<S>::R *__restrict__ rho,
              typename Stor<S>::R *__restrict__ u, bool pair) {
     typedef typename Stor<S>::R R;
@@ -1917,7 +1919,7 @@ __global__ void __launch_bounds__(RED_THREADS, FLAGS || is_split(S) ? 2 : FieldB
 // g = dL/du, at the gathered state; grad_F += g / (2 rho) (u contains F/2).
 // Incompressible model (u = j + F/2): lambda^T_m = dL/drho + g.e_m, grad_F += g/2.
 template <int S, bool FLAGS, bool FORCE>
-__global__ void __launch_bounds__(256, FieldBlocks<S, FLAGS>::value)
+__global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
     k_adj_seed(const Dev d, const typename Stor<S>::T *__restrict__ P, const typename Stor<S>::R *__restrict__ dL_du,
                const typename Stor<S>::R *__restrict__ dL_drho, typename Stor<S>::R *__restrict__ lam,
                typename Stor<S>::R *__restrict__ grad_F, bool pair) {
