@@ -35,7 +35,7 @@ struct lbm_ctx {
     int box[4];         // y0, rows, z0, planes: the smallest y/z box holding every fluid cell
     uint8_t *flags_d;   // padded [qs], 1 = solid (padding included), or null
     uint32_t *mask_d;   // padded [qs] push masks for the step kernels, or null
-    uint32_t *moving_d; // padded [qs] moving-wall bits (contexts with cells flagged 2), or null
+    uint32_t *moving_d; // padded [qs] moving-wall bits behind mask_d (contexts with cells flagged 2), or null
     uint32_t *links_d;  // bounce-back links (fluid cell, solid cell), grouped by direction
     int link_off[20];
     int link_max;
@@ -283,7 +283,6 @@ void free_ctx(lbm_ctx *ctx) {
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     drop_graphs(ctx);
     void *ptrs[] = {ctx->lat[0], ctx->lat[1],  ctx->flags_d,     ctx->mask_d,   ctx->links_d,        ctx->Ffield_d,
-                    ctx->moving_d,
                     ctx->lam[0], ctx->lam[1], ctx->red_partials, ctx->red_out, ctx->step_partials, ctx->status_d,
                     ctx->staging};
     for (void *p : ptrs)
@@ -445,8 +444,9 @@ lbm_status lbm_create(lbm_ctx **out, int nx, int ny, int nz, double tau, const u
               cudaMalloc((void **)&ctx->red_out, 4 * sizeof(double)) == cudaSuccess &&
               cudaMalloc((void **)&ctx->status_d, sizeof(unsigned)) == cudaSuccess;
     if (ok && flags) ok = cudaMalloc((void **)&ctx->flags_d, (size_t)qs) == cudaSuccess;
-    if (ok && flags) ok = cudaMalloc((void **)&ctx->mask_d, (size_t)qs * sizeof(uint32_t)) == cudaSuccess;
-    if (ok && ctx->has_moving) ok = cudaMalloc((void **)&ctx->moving_d, (size_t)qs * sizeof(uint32_t)) == cudaSuccess;
+    if (ok && flags)
+        ok = cudaMalloc((void **)&ctx->mask_d, (size_t)qs * (ctx->has_moving ? 2 : 1) * sizeof(uint32_t)) == cudaSuccess;
+    if (ok && ctx->has_moving) ctx->moving_d = ctx->mask_d + qs;
     if (!ok) {
         cudaGetLastError();
         free_ctx(ctx);
