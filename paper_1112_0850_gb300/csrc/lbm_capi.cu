@@ -115,7 +115,7 @@ Dev make_dev(const lbm_ctx *ctx) {
     d.g = ctx->g;
     d.L = ctx->L;
     d.P = pair_launch(ctx->g, ctx->box[0], ctx->box[1], ctx->box[2], ctx->box[3]);
-    d.PF = flat_launch(d.P, flat_threads(d.P));
+    d.PF = flat_launch(d.P, step_flat_threads(d.P, ctx->storage, ctx->flags_d, ctx->pattern == LBM_PATTERN_AA));
     d.flat_step = rows_leave_lanes_idle(d.P) || small_lattice(d.P);
     d.flags = ctx->flags_d;
     d.mask = ctx->mask_d;

@@ -345,6 +345,19 @@ constexpr long long SMALL_PAIRS = 300000;
 inline bool small_lattice(const RowLaunch &rows) { return (long long)rows.nyr * rows.nzr * rows.W <= SMALL_PAIRS; }
 inline int flat_threads(const RowLaunch &rows) { return small_lattice(rows) ? 64 : 128; }
 
+// The two-grid step without flags in FP32 and 16-bit shifted storage keeps
+// blocks of 256 where they tile every row (nx = 512, 1024, ..). Us a step with
+// 256 / 128 threads: 512^3 FP16 1683 / 1702, BF16 1670 / 1698, FP32 2900 / 2907;
+// 512x256x256 FP16 419 / 415, FP32 727.3 / 728.2; other rows, FP16: 496^3 1551 /
+// 1542, 528^3 1837 / 1814, 256^3 209.3 / 206.8.
+constexpr bool wide_blocks_fit(int storage, bool flags) {
+    return !flags && (storage == LBM_F32 || storage == LBM_F16S || storage == LBM_BF16S);
+}
+inline int step_flat_threads(const RowLaunch &rows, int storage, bool flags, bool aa) {
+    const int t = flat_threads(rows);
+    return !aa && wide_blocks_fit(storage, flags) && t == 128 && rows.W % 256 == 0 ? 256 : t;
+}
+
 template <bool FLAT = false>
 LBM_HD bool pair_cell(const Geom &g, const RowLaunch &P, int bdx, int bdy, int bx, int bz, int tx, int ty, int &x0,
                       int &y, int &z) {

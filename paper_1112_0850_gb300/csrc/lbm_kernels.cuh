@@ -924,7 +924,7 @@ __device__ __forceinline__ void step_pair_split(const Dev &d, const typename Sto
 constexpr int STEP_PDL = 1;
 
 // Block shape of the step kernel: the flat launch's blocks hold 128 threads at
-// most, whole rows 256. Blocks of 128 per SM, and what was measured (us a step):
+// most (256 where wide_blocks_fit), whole rows 256. Blocks of 128 per SM, and what was measured (us a step):
 //  - FP32 with flags (32-bit offsets): 7 (72 registers, no spills: 28 warps)
 //    +1.1% on the walled channel over 3 of 256 (80 registers); 4 of 256 (64)
 //    spilled 48 bytes and lost 4%. A force per cell: 6 (80), channel 97.2 to 94.2.
@@ -932,10 +932,12 @@ constexpr int STEP_PDL = 1;
 //    flags 6, BF16 384^3 960 against 1030.
 //  - 16-bit: 8 (64); with a force per cell 6 (80), 200^3 FP16 117.5 against 125.4,
 //    porous channel (whole rows, 3 of 256), recorded, 430 against 484.
-template <bool FLAT> constexpr int step_threads() { return FLAT ? 128 : 256; }
+template <bool FLAT, int S, bool FLAGS> constexpr int step_threads() {
+    return FLAT && !wide_blocks_fit(S, FLAGS) ? 128 : 256;
+}
 template <int S, bool FLAGS, int FORCE, bool FLAT, bool U32, bool RED = false> constexpr int step_min_blocks() {
     const int rows = FORCE == 2 && StepBlocks<S>::value == 4 ? 3 : StepBlocks<S>::value;
-    if (!FLAT) return rows;
+    if (!FLAT || wide_blocks_fit(S, FLAGS)) return rows;
     if (U32 || (is_split(S) && FLAGS && !RED)) return FORCE == 2 ? 6 : 7;
     return 2 * rows;
 }
@@ -944,7 +946,7 @@ template <int S, bool FLAGS, int FORCE, bool FLAT, bool U32, bool RED = false> c
 // ODD (moment-split formats only): rows of odd length, whose last cell is
 // alone in its pair (see split_ghost). U32: 32-bit lattice offsets (lat_at).
 template <int S, bool FLAGS, int FORCE, bool RECORD, bool FLAT = false, bool ODD = false, bool U32 = false>
-__global__ void __launch_bounds__(step_threads<FLAT>(), step_min_blocks<S, FLAGS, FORCE, FLAT, U32>())
+__global__ void __launch_bounds__(step_threads<FLAT, S, FLAGS>(), step_min_blocks<S, FLAGS, FORCE, FLAT, U32>())
     k_step(const Dev d, const typename Stor<S>::T *__restrict__ src, typename Stor<S>::T *__restrict__ dst,
            typename Stor<S>::R *__restrict__ tape) {
     // launched as a programmatic dependent: wait for the kernel before it (the
@@ -979,7 +981,7 @@ __global__ void __launch_bounds__(step_threads<FLAT>(), step_min_blocks<S, FLAGS
 // the lattice or not, reaches the block reduction; partials[4 b + k] of block
 // b = blockIdx.y * gridDim.x + blockIdx.x, summed in a fixed order.
 template <int S, bool FLAGS, int FORCE, bool FLAT, bool ODD = false>
-__global__ void __launch_bounds__(step_threads<FLAT>(), step_min_blocks<S, FLAGS, FORCE, FLAT, false, true>())
+__global__ void __launch_bounds__(step_threads<FLAT, S, FLAGS>(), step_min_blocks<S, FLAGS, FORCE, FLAT, false, true>())
     k_step_reduce(const Dev d, const typename Stor<S>::T *__restrict__ src, typename Stor<S>::T *__restrict__ dst,
                   double *__restrict__ partials) {
     if (FLAGS && LinkBounce<S>::value) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -2006,7 +2008,7 @@ static cudaError_t launch_step3f(const Dev &d, const void *src, void *dst, void 
     typedef typename Stor<S>::T T;
     typedef typename Stor<S>::R R;
     if constexpr (!U32 && S == LBM_F32 && FLAGS) {
-        // (the flat launch's blocks hold at most 128 threads, step_threads)
+        // (with flags the flat launch's blocks hold at most 128 threads, step_threads)
         if (step_u32<S, FLAGS>(d)) return launch_step3f<S, FLAGS, FORCE, FLAT, ODD, true>(d, src, dst, tape);
     }
     const RowLaunch &P = FLAT ? d.PF : d.P;
