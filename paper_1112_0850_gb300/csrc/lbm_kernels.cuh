@@ -1364,19 +1364,37 @@ template <int S, bool FLAGS> struct FieldBlocks {
 // the values of its 18 neighbours was bound by their 76 loads and by arithmetic
 // (FP64: its pipe 85% busy). Channel: FP32 165 to 111 us (floor 57), FP16 187 to
 // 86, FP64 2358 to 593; 256^3 box, FP32 435 to 288 us (floor 227).
-// f_eq - w of one cell, opposite directions from their even and odd parts.
-template <class R> __device__ __forceinline__ void feq_all(R f[Q], R rho1, R ux, R uy, R uz, bool incomp) {
-    const R rho = incomp ? R(1) : R(1) + rho1;
-    const R usq = R(-1.5) * (ux * ux + uy * uy + uz * uz);
-    f[0] = R(1.0 / 3.0) * (rho1 + rho * usq);
+// f_eq - w of the two cells of a pair: per direction one expression,
+// w (rho1 + rho (3 e.u + 9/2 (e.u)^2 - 3/2 u.u)), its roundings in this order. (The even
+// and odd parts of opposite directions formed once take 8 operations a pair of them
+// instead of 11 and are as accurate, but differ in the last FP32 bit, which the 16-bit
+// formats turn into a whole storage step of the initial state. On packed cells this
+// order costs no time: 256^3 box FP32 260 to 250 us, FP16 219 to 216, channel FP16
+// 99 to 94, FP32 127 to 132.)
+__device__ __forceinline__ void feq2(float2 f[Q], float2 rho1, float2 ux, float2 uy, float2 uz, bool incomp) {
+    const float2 rho = incomp ? vsplat(1.0f) : vadd(vsplat(1.0f), rho1);
+    const float2 usq = vfma(uz, uz, vfma(ux, ux, vmul(uy, uy)));
+    f[0] = vmul(vsplat((float)(1.0 / 3.0)), vfma(rho, vmul(vsplat(-1.5f), usq), rho1));
 #pragma unroll
     for (int p = 0; p < NPAIR; ++p) {
         const int i = pair_first(p);
-        const R w = i <= 6 ? R(1.0 / 18.0) : R(1.0 / 36.0);
-        const R eu = R(ex(i)) * ux + R(ey(i)) * uy + R(ez(i)) * uz;
-        const R even = w * (rho1 + rho * (R(4.5) * eu * eu + usq)), odd = (R(3) * w * rho) * eu;
-        f[i] = even + odd;
-        f[opp(i)] = even - odd;
+        const float2 w = vsplat(i <= 6 ? (float)(1.0 / 18.0) : (float)(1.0 / 36.0));
+        const float2 eu = edot_first(i, ux, uy, uz), sq = vmul(vmul(vsplat(4.5f), eu), eu);
+        f[i] = vmul(w, vfma(rho, vfma(vsplat(-1.5f), usq, vfma(vsplat(3.0f), eu, sq)), rho1));
+        f[opp(i)] = vmul(w, vfma(rho, vfma(vsplat(-1.5f), usq, vfma(vsplat(-3.0f), eu, sq)), rho1));
+    }
+}
+
+// The same of one cell in FP64.
+__device__ __forceinline__ void feq64(double f[Q], double rho1, double ux, double uy, double uz, bool incomp) {
+    const double rho = incomp ? 1.0 : 1.0 + rho1, usq = fma(uz, uz, fma(ux, ux, uy * uy));
+    f[0] = (1.0 / 3.0) * fma(rho, -1.5 * usq, rho1);
+#pragma unroll
+    for (int p = 0; p < NPAIR; ++p) {
+        const int i = pair_first(p);
+        const double w = i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0, eu = ex(i) * ux + ey(i) * uy + ez(i) * uz, sq = 4.5 * eu * eu;
+        f[i] = w * fma(rho, fma(-1.5, usq, fma(3.0, eu, sq)), rho1);
+        f[opp(i)] = w * fma(rho, fma(-1.5, usq, fma(-3.0, eu, sq)), rho1);
     }
 }
 
@@ -1533,22 +1551,26 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
             get2<RF>(u0 + 2 * N + cc, pair, has1, uz[0], uz[1]);
         }
     }
-    R f0[Q], f1[Q];
+    typedef typename Pair2<R>::V V;
+    V f[Q];
     if constexpr (S == LBM_F64) {
+        double f0[Q], f1[Q];
         if (!fixed_equilibrium(f0, r[0] - 1.0, ux[0], uy[0], uz[0], d.incomp))
-            feq_all(f0, r[0] - R(1), ux[0], uy[0], uz[0], d.incomp);
+            feq64(f0, r[0] - 1.0, ux[0], uy[0], uz[0], d.incomp);
         if (!fixed_equilibrium(f1, r[1] - 1.0, ux[1], uy[1], uz[1], d.incomp))
-            feq_all(f1, r[1] - R(1), ux[1], uy[1], uz[1], d.incomp);
+            feq64(f1, r[1] - 1.0, ux[1], uy[1], uz[1], d.incomp);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) f[i] = make_double2(f0[i], f1[i]);
     } else {
-        feq_all(f0, r[0] - R(1), ux[0], uy[0], uz[0], d.incomp);
-        feq_all(f1, r[1] - R(1), ux[1], uy[1], uz[1], d.incomp);
+        feq2(f, make_float2(r[0] - 1.0f, r[1] - 1.0f), make_float2(ux[0], ux[1]), make_float2(uy[0], uy[1]),
+             make_float2(uz[0], uz[1]), d.incomp);
     }
     if (d.layout == LAYOUT_AA_NAT) {  // AA natural layout: f^0_i(x) at the cell itself
         const R nan = quiet_nan<R>();
         if (!in) return;
 #pragma unroll
         for (int i = 0; i < Q; ++i)
-            put2(P + i * g.qs + c, true, true, !FLAGS || live0 ? f0[i] : nan, !FLAGS || live1 ? f1[i] : nan);
+            put2(P + i * g.qs + c, true, true, !FLAGS || live0 ? f[i].x : nan, !FLAGS || live1 ? f[i].y : nan);
         return;
     }
     // Cells x0 and x0 + 1 to columns x0 - e_x and x0 + 1 - e_x. Where e_x = +-1
@@ -1571,21 +1593,21 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
         T *row = P + i * g.qs + (wrap1(z - ez(i), g.nz) * g.ny + wrap1(y - ey(i), g.ny)) * g.pitch;
         if (ex(i) == 0) {
             if (live0 && live1) {
-                put2(row + x0, true, true, f0[i], f1[i]);
+                put2(row + x0, true, true, f[i].x, f[i].y);
             } else {
-                if (live0) row[x0] = Rn<T>::of(f0[i]);
-                if (live1) row[x0 + 1] = Rn<T>::of(f1[i]);
+                if (live0) row[x0] = Rn<T>::of(f[i].x);
+                if (live1) row[x0 + 1] = Rn<T>::of(f[i].y);
             }
         } else if (ex(i) > 0) {
-            const R v = __shfl_down_sync(0xffffffffu, f0[i], 1);
-            if (next) put2(row + x0, true, true, f1[i], v);
-            else if (live1) row[x0] = Rn<T>::of(f1[i]);
-            if (live0 && !prev) row[xa] = Rn<T>::of(f0[i]);
+            const R v = __shfl_down_sync(0xffffffffu, f[i].x, 1);
+            if (next) put2(row + x0, true, true, f[i].y, v);
+            else if (live1) row[x0] = Rn<T>::of(f[i].y);
+            if (live0 && !prev) row[xa] = Rn<T>::of(f[i].x);
         } else {
-            const R v = __shfl_up_sync(0xffffffffu, f1[i], 1);
-            if (prev1) put2(row + x0, true, true, v, f0[i]);
-            else if (live0) row[xb] = Rn<T>::of(f0[i]);
-            if (live1 && !next1) row[xc] = Rn<T>::of(f1[i]);
+            const R v = __shfl_up_sync(0xffffffffu, f[i].y, 1);
+            if (prev1) put2(row + x0, true, true, v, f[i].x);
+            else if (live0) row[xb] = Rn<T>::of(f[i].x);
+            if (live1 && !next1) row[xc] = Rn<T>::of(f[i].y);
         }
     }
     if (FLAGS && ((m0 | m1) & 0x7fffeu)) {
@@ -1597,7 +1619,7 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (!(((k ? m1 : m0) >> i) & 1u)) continue;
-                R v = k ? f1[opp(i)] : f0[opp(i)];
+                R v = k ? f[opp(i)].y : f[opp(i)].x;
                 if (((k ? mv.y : mv.x) >> i) & 1u) v += wall_term<R>(d, i);
                 P[i * g.qs + c + k] = Rn<T>::of(v);
             }
