@@ -117,7 +117,7 @@ __device__ __forceinline__ void aa_even_pair(const Dev &d, typename Stor<S>::T *
     pair_force<R, FORCE, relax_about_t(S)>(d, c, Fx, Fy, Fz, G);
     Mom2<R> m;
     if constexpr (S == LBM_F64)
-        m = pair64<FORCE != 0, true, RECORD || RED>(d, s, Fx, Fy, Fz);
+        m = pair64<FORCE != 0, true, RECORD || RED>(d, s, Fx, Fy, Fz, live0, live1);
     else
         m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
     if (RED) tot->set(m, live0, live1);
@@ -252,7 +252,7 @@ __device__ __forceinline__ void aa_odd_pair(const Dev &d, typename Stor<S>::T *_
     pair_force<R, FORCE, relax_about_t(S)>(d, c, Fx, Fy, Fz, G);
     Mom2<R> m;
     if constexpr (S == LBM_F64)
-        m = pair64<FORCE != 0, true, RECORD || RED>(d, s, Fx, Fy, Fz);
+        m = pair64<FORCE != 0, true, RECORD || RED>(d, s, Fx, Fy, Fz, live0, live1);
     else
         m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
     if (RED) tot->set(m, live0, live1);

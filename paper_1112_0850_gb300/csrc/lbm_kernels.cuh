@@ -517,35 +517,51 @@ __device__ __forceinline__ void cell64(const Dev &d, double s[Q], double Fx, dou
     }
 }
 
-// The pair's moments, and its collision (COLLIDE), cell by cell.
+// The pair's moments, and its collision (COLLIDE), cell by cell; a cell that is
+// not live is left alone, with rho = 1. (The solid slots of an AA lattice hold
+// NaN, which is outside the fixed-point range: one such lane sent its whole warp
+// through cell64_fp64, and 65% of the warps of the 256x128x128 channel hold one:
+// mean AA step 1871 us, 418 without them; in FP64 arithmetic throughout 1383.)
 template <bool FORCE, bool COLLIDE, bool MOM>
-__device__ __forceinline__ Mom2<double> pair64(const Dev &d, double2 s[Q], double2 Fx, double2 Fy, double2 Fz) {
+__device__ __forceinline__ Mom2<double> pair64(const Dev &d, double2 s[Q], double2 Fx, double2 Fy, double2 Fz,
+                                               bool live0, bool live1) {
     Mom2<double> m;
-    double t[Q];
-    Cell64 o;
+    m.rho = vsplat(1.0);
+    if (MOM) m.rho1 = m.jx = m.jy = m.jz = m.ux = m.uy = m.uz = vsplat(0.0);
+    if (live0) {
+        double t[Q];
+        Cell64 o;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) t[i] = s[i].x;
-    cell64<FORCE, COLLIDE, MOM>(d, t, Fx.x, Fy.x, Fz.x, o);
+        for (int i = 0; i < Q; ++i) t[i] = s[i].x;
+        cell64<FORCE, COLLIDE, MOM>(d, t, Fx.x, Fy.x, Fz.x, o);
 #pragma unroll
-    for (int i = 0; COLLIDE && i < Q; ++i) s[i].x = t[i];
-    m.rho.x = o.rho;
-    if (MOM) m.rho1.x = o.rho1, m.jx.x = o.jx, m.jy.x = o.jy, m.jz.x = o.jz, m.ux.x = o.ux, m.uy.x = o.uy, m.uz.x = o.uz;
+        for (int i = 0; COLLIDE && i < Q; ++i) s[i].x = t[i];
+        m.rho.x = o.rho;
+        if (MOM)
+            m.rho1.x = o.rho1, m.jx.x = o.jx, m.jy.x = o.jy, m.jz.x = o.jz, m.ux.x = o.ux, m.uy.x = o.uy, m.uz.x = o.uz;
+    }
+    if (live1) {
+        double t[Q];
+        Cell64 o;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) t[i] = s[i].y;
-    cell64<FORCE, COLLIDE, MOM>(d, t, Fx.y, Fy.y, Fz.y, o);
+        for (int i = 0; i < Q; ++i) t[i] = s[i].y;
+        cell64<FORCE, COLLIDE, MOM>(d, t, Fx.y, Fy.y, Fz.y, o);
 #pragma unroll
-    for (int i = 0; COLLIDE && i < Q; ++i) s[i].y = t[i];
-    m.rho.y = o.rho;
-    if (MOM) m.rho1.y = o.rho1, m.jx.y = o.jx, m.jy.y = o.jy, m.jz.y = o.jz, m.ux.y = o.ux, m.uy.y = o.uy, m.uz.y = o.uz;
+        for (int i = 0; COLLIDE && i < Q; ++i) s[i].y = t[i];
+        m.rho.y = o.rho;
+        if (MOM)
+            m.rho1.y = o.rho1, m.jx.y = o.jx, m.jy.y = o.jy, m.jz.y = o.jz, m.ux.y = o.ux, m.uy.y = o.uy, m.uz.y = o.uz;
+    }
     return m;
 }
 
 // The moments of a pair for the readers.
 template <class R, bool FORCE>
 __device__ __forceinline__ Mom2<R> pair_moments(const Dev &d, typename Pair2<R>::V s[Q], typename Pair2<R>::V Fx,
-                                                typename Pair2<R>::V Fy, typename Pair2<R>::V Fz) {
+                                                typename Pair2<R>::V Fy, typename Pair2<R>::V Fz, bool live0,
+                                                bool live1) {
     if constexpr (sizeof(R) == 8)
-        return pair64<FORCE, false, true>(d, s, Fx, Fy, Fz);
+        return pair64<FORCE, false, true>(d, s, Fx, Fy, Fz, live0, live1);
     else
         return moments2<R, FORCE>(s, Fx, Fy, Fz, d.incomp);
 }
@@ -1837,7 +1853,7 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
         V s[Q], Fx, Fy, Fz;
         gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
         pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
-        const Mom2<R> m = pair_moments<R, FORCE>(d, s, Fx, Fy, Fz);
+        const Mom2<R> m = pair_moments<R, FORCE>(d, s, Fx, Fy, Fz, live0, live1);
         o[0] = m.rho;
         o[1] = m.ux;
         o[2] = m.uy;
@@ -1887,7 +1903,7 @@ __global__ void __launch_bounds__(RED_THREADS, FLAGS || is_split(S) ? 2 : FieldB
                 V s[Q], Fx, Fy, Fz;
                 gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
                 pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
-                tot.set(pair_moments<R, FORCE>(d, s, Fx, Fy, Fz), live0, live1);
+                tot.set(pair_moments<R, FORCE>(d, s, Fx, Fy, Fz, live0, live1), live0, live1);
             }
         }
         cells += tot.cells;
@@ -1968,7 +1984,7 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
     if (dL_drho) get2<RF>(dL_drho + cc, pair, has1, dr.x, dr.y);
     gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
     pair_force_at<R, FORCE>(d, c, Fx, Fy, Fz);
-    const Mom2<R> m = pair_moments<R, FORCE>(d, s, Fx, Fy, Fz);
+    const Mom2<R> m = pair_moments<R, FORCE>(d, s, Fx, Fy, Fz, live0, live1);
     const V inv = d.incomp ? vsplat(R(1)) : vrcp(m.rho);
     const V gu = vfma(gz, m.uz, vfma(gy, m.uy, vmul(gx, m.ux)));
     const V base = d.incomp ? dr : vsub(dr, vmul(gu, inv));
