@@ -2,17 +2,23 @@
 //
 // GB300 executes FP64 arithmetic at 2 operations a clock and SM, and integer
 // arithmetic at 64 to 128: an update's 164 FP64 operations held the FP64 step
-// at 0.12 of copy bandwidth (1383 us on the 256x128x128 channel; 266 us in this
-// form). Here a cell's 19 deviations s_i (and its force)
+// at 0.12 of copy bandwidth (1383 us on the 256x128x128 channel; 280 us in this
+// form). Here a cell's 19 deviations s_i (and half its force)
 // are aligned to one exponent, that of the largest of them, as 64-bit integers
-// with the largest in [2^56, 2^57): 4 bits finer than its FP64 spacing. Sums
-// of them are exact. Products keep 62 bits. What is added to (1 - omega) s_i
-// comes back as a double, correctly rounded, and one FP64 multiply-add per
-// population is left. Against 113-bit arithmetic, over tau from 0.5005 to 5 and
-// values from 1e-200 to 0.3, the post-collision values are off by 0.4 to 0.95
-// times what the FP64 form is (rms, relative to the cell's largest: 4e-17 to
-// 6e-17 against 4.5e-17 to 2e-16), the moments by half, and the mass balance by
-// 1e-17, as the FP64 form's.
+// with the largest in [2^57, 2^58): 5 bits finer than its FP64 spacing. Sums
+// of them are exact. Products are rounded to nearest and keep 3 more bits. What is
+// added to (1 - omega) s_i comes back as a double, correctly rounded, and one FP64
+// multiply-add per population is left.
+//
+// Against extended precision, relative to the cell's largest value, the
+// post-collision values are off (rms) by 0.2 to 1.0 times what the FP64 form is, the
+// momentum they carry by 0.1 to 1.02 times, with no mean in it: for tau from 0.5005
+// to 50, flows of 1e-9 to 0.2 with density deviations up to 0.2, noise, and forces
+// from none to the largest value of the cell (tests/test_fixed64_cpu.py). Equilibria
+// and moments are off by 0.4 to 0.7 times. (With inputs cut at 2^-56, products rounded
+// to that unit and a fixed offset for their dropped low parts, the momentum was off
+// by up to 2.8 times and had a mean of a few 1e-17 of either sign, by tau: a body
+// force. The step took 272 us.)
 //
 // With j' = j + F/2, u = j'/rho (u = j' in the incompressible model) and
 // c = 1 - omega/2, collide2's E and P (omega folded in) are, in
@@ -30,18 +36,20 @@
 
 namespace lbm {
 
-// Constants of the collision as 62-bit fractions (value 2^62, rounded).
+// Constants of the collision as 62-bit fractions (value 2^62, rounded). omega is
+// taken as 1 - (1 - omega), so that it and the rounded 1 - omega add up to 1: else
+// every step would scale mass and momentum by the rounding (tau = 5: 1 + 5.6e-17).
 struct FixedK {
-    long long w94, w12, c12;  // 4/9 omega, omega/12, (1 - omega/2)/12
-    double omc;               // 1 - omega
+    long long w29, w12, c6;  // 2/9 omega, omega/12, (1 - omega/2)/6
+    double omc;              // 1 - omega
 };
 inline FixedK fixed_k(double omega) {
     FixedK k;
-    const long long w = (long long)ldexp(omega, 61);  // omega < 2
-    k.w94 = w / 9 * 8 + (w % 9 * 8 + 4) / 9;
-    k.w12 = (w + 3) / 6;
-    k.c12 = ((1LL << 62) - w + 6) / 12;  // (2^62 - omega 2^61) / 12
     k.omc = 1.0 - omega;
+    const long long w = (long long)ldexp(1.0 - k.omc, 61);  // omega < 2
+    k.w29 = w / 9 * 4 + (w % 9 * 4 + 4) / 9;
+    k.w12 = (w + 3) / 6;
+    k.c6 = ((1LL << 62) - w + 3) / 6;  // (2^62 - omega 2^61) / 6
     return k;
 }
 
@@ -105,15 +113,15 @@ LBM_HD uint64_t fx_shr(uint64_t a, int n) {
 #endif
 }
 
-// a 2^(56 - (E - 1023)), E >= the exponent field of a; towards zero.
+// a 2^(57 - (E - 1023)), E >= the exponent field of a; towards zero.
 LBM_HD long long fx_in(double a, int E) {
     const uint32_t h = fx_hi(a);
-    const int sh = E + 6 - (int)((h >> 20) & 0x7ffu);
+    const int sh = E + 5 - (int)((h >> 20) & 0x7ffu);
     const uint64_t q = ((((uint64_t)((h & 0xfffffu) | 0x100000u)) << 32) | fx_lo(a)) << 10;
     return fx_neg_if((long long)fx_shr(q, sh), (int)h);
 }
 
-// q 2^((E - 1023) - 56), |q| < 2^62, rounded to nearest (ties away from zero).
+// q 2^((E - 1023) - 57), |q| < 2^63, rounded to nearest (ties away from zero).
 LBM_HD double fx_out(long long q, int E) {
     const int qh = (int)(q >> 32);
     const uint64_t a = (uint64_t)fx_neg_if(q, qh);
@@ -121,7 +129,7 @@ LBM_HD double fx_out(long long q, int E) {
     // the leading one to bit 62, half a unit of the 53 bits kept added (the
     // leading bit adds the last 1 of the exponent field, a carry one more)
     const uint64_t r = ((a << (62 - p)) + (1u << 9)) >> 10;
-    uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)(E + p - 57) << 20);
+    uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)(E + p - 58) << 20);
     hi = (hi & 0x7fffffffu) | ((uint32_t)qh & 0x80000000u);
     return fx_double(p < 0 ? 0u : hi, (uint32_t)r);
 }
@@ -132,21 +140,31 @@ struct L31 {
     int h, l;
 };
 LBM_HD L31 limbs(long long a) { return L31{(int)(a >> 31), (int)((uint32_t)a & 0x7fffffffu)}; }
-// a b / 2^62 to within 1; the 0.75 makes up for the dropped a.l b.l and the floor.
-LBM_HD long long mul62(L31 a, L31 b) {
-    const long long mid = (long long)a.h * b.l + ((long long)a.l * b.h + (3LL << 29));
-    return (long long)a.h * b.h + (mid >> 31);
+LBM_HD uint32_t fx_mulhi(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+#endif
+}
+// a b / 2^(62 - K), rounded to nearest (to within 2^(K - 31)); |the result| < 2^63.
+// (b, the factor that several products share or a constant, is the one shifted.)
+template <int K> LBM_HD long long mulk(L31 a, L31 b) {
+    const uint32_t ll = fx_mulhi((uint32_t)a.l, (uint32_t)b.l << 1);
+    const long long mid = (long long)a.h * b.l + ((long long)a.l * b.h + (long long)(ll + (1u << (30 - K))));
+    return (long long)((unsigned long long)((long long)a.h * b.h) << K) + (mid >> (31 - K));
 }
 
-// The moments of a cell: rho - 1 and j' in units of 2^((E - 1023) - 56).
+// The moments of a cell: rho - 1, j' and F/2 in units of 2^((E - 1023) - 57).
 struct FixedMom {
     int E;
-    long long r, jx, jy, jz, fx, fy, fz;  // (f: F in the same units)
+    long long r, jx, jy, jz, fx, fy, fz;
 };
 
 // False where the cell is outside the range of the fixed-point collision
-// (|s_i| or |F| >= 1/4, |rho - 1| or |j'| >= 1/2, not finite): the caller then
-// takes FP64 arithmetic.
+// (|s_i| or |F| >= 1/4, |rho - 1| or |j'| >= 1/2 or 8 to 16 times the largest of the
+// s_i and F, not finite): the caller then takes FP64 arithmetic. (A flow near
+// equilibrium has |rho - 1| < 4 and |j'| < 6 times its largest s_i.)
 template <bool FORCE>
 LBM_HD bool fixed_moments(const double s[Q], double Fx, double Fy, double Fz, FixedMom &m) {
     uint32_t top = 128u << 20;  // (values below 2^-895 count as zero; keeps every result a normal number)
@@ -176,26 +194,27 @@ LBM_HD bool fixed_moments(const double s[Q], double Fx, double Fy, double Fz, Fi
     m.jz = (q[5] - q[6]) + (q[11] - q[14]) + (q[13] - q[12]) + (q[15] - q[18]) + (q[17] - q[16]);
     m.fx = m.fy = m.fz = 0;
     if (FORCE) {
-        m.fx = fx_in(Fx, E);
-        m.fy = fx_in(Fy, E);
-        m.fz = fx_in(Fz, E);
-        m.jx += m.fx >> 1;
-        m.jy += m.fy >> 1;
-        m.jz += m.fz >> 1;
+        m.fx = fx_in(Fx, E + 1);
+        m.fy = fx_in(Fy, E + 1);
+        m.fz = fx_in(Fz, E + 1);
+        m.jx += m.fx;
+        m.jy += m.fy;
+        m.jz += m.fz;
     }
-    const int n = 1023 - E;  // >= 3: the unit is 2^-(56 + n)
-    if (n >= 8) return true;  // |s|, |F| < 2^-7: |rho - 1| <= 19/128, |j'| < 11/128
-    const long long half = 1LL << (55 + n);
-    return m.r < half && m.r > -half && m.jx < half && m.jx > -half && m.jy < half && m.jy > -half && m.jz < half &&
-           m.jz > -half;
+    // |r|, |j| < 2^61 units and 1/2 (compared in the high halves)
+    const int n = 1023 - E;  // >= 3: the unit is 2^-(57 + n)
+    const int rh = (int)(m.r >> 32), xh = (int)(m.jx >> 32), yh = (int)(m.jy >> 32), zh = (int)(m.jz >> 32);
+    const int o = (rh ^ (rh >> 31)) | (xh ^ (xh >> 31)) | (yh ^ (yh >> 31)) | (zh ^ (zh >> 31));
+    return (o >> (n < 5 ? 24 + n : 29)) == 0;
 }
-
 // s <- (1 - omega) s + E +- P (see the head of this file), or with EQ
-// s <- E +- P: at omega = 1 and no force that is the equilibrium.
+// s <- E +- P: at omega = 1 and no force that is the equilibrium. g, h, X and B are
+// held in eighths of m's unit, so that 2 (B + X) +- 2 g and 12 B are whole in
+// quarters and halves of it.
 template <bool FORCE, bool EQ = false>
 LBM_HD void fixed_collide(double s[Q], const FixedMom &m, const FixedK &k, bool incomp) {
     const int n = 1023 - m.E;  // >= 3
-    const int n2 = n - 2 < 63 ? n - 2 : 63, n0 = n < 63 ? n : 63;
+    const int n2 = n - 1 < 63 ? n - 1 : 63, n0 = n + 1 < 63 ? n + 1 : 63;
     // j' and 3/2 / rho as 58- and 60-bit fractions
     const L31 j58x = limbs(m.jx >> n2), j58y = limbs(m.jy >> n2), j58z = limbs(m.jz >> n2);
     long long inv15 = 3LL << 59;
@@ -220,11 +239,11 @@ LBM_HD void fixed_collide(double s[Q], const FixedMom &m, const FixedK &k, bool 
     }
     const L31 iv = limbs(inv15);
     const L31 w12 = limbs(k.w12);
-    long long gx = mul62(limbs(m.jx), w12), gy = mul62(limbs(m.jy), w12), gz = mul62(limbs(m.jz), w12);
+    long long gx = mulk<3>(limbs(m.jx), w12), gy = mulk<3>(limbs(m.jy), w12), gz = mulk<3>(limbs(m.jz), w12);
     long long hx = gx, hy = gy, hz = gz;
     if (FORCE) {
-        const L31 c12 = limbs(k.c12);
-        const long long cx = mul62(limbs(m.fx), c12), cy = mul62(limbs(m.fy), c12), cz = mul62(limbs(m.fz), c12);
+        const L31 c6 = limbs(k.c6);
+        const long long cx = mulk<3>(limbs(m.fx), c6), cy = mulk<3>(limbs(m.fy), c6), cz = mulk<3>(limbs(m.fz), c6);
         gx += cx;
         gy += cy;
         gz += cz;
@@ -232,32 +251,30 @@ LBM_HD void fixed_collide(double s[Q], const FixedMom &m, const FixedK &k, bool 
         hy = gy + cy;
         hz = gz + cz;
     }
-    // v (56-bit fractions, |v| < 4) and h, both 8 times: their product / 2^62
-    const L31 vx = limbs(mul62(j58x, iv) << 3), vy = limbs(mul62(j58y, iv) << 3), vz = limbs(mul62(j58z, iv) << 3);
-    const L31 lx = limbs(hx << 3), ly = limbs(hy << 3), lz = limbs(hz << 3);
-    const long long X = mul62(vx, lx), Y = mul62(vy, ly), Z = mul62(vz, lz);
-    const long long XY = FORCE ? mul62(vx, ly) + mul62(vy, lx) : mul62(vx, ly) << 1;
-    const long long XZ = FORCE ? mul62(vx, lz) + mul62(vz, lx) : mul62(vx, lz) << 1;
-    const long long YZ = FORCE ? mul62(vy, lz) + mul62(vz, ly) : mul62(vy, lz) << 1;
-    // 16 B: it enters the 19 populations 36 times, so its rounding would be the
-    // mass balance's (4/9 omega < 8/9; 16/3 S = 2 (4 S 2/3))
-    constexpr long long two3 = 3074457345618258603LL;  // 2^63 / 3
-    const long long B16 = mul62(limbs(m.r), limbs(k.w94)) - 2 * mul62(limbs((X + Y + Z) << 2), limbs(two3));
-    const long long B0 = (3 * B16 + 2) >> 2, B1 = (B16 + 4) >> 3, B2 = (B16 + 8) >> 4;
+    // v as 60-bit fractions (|v| < 3/2)
+    const L31 vx = limbs(mulk<4>(j58x, iv)), vy = limbs(mulk<4>(j58y, iv)), vz = limbs(mulk<4>(j58z, iv));
+    const L31 lx = limbs(hx), ly = limbs(hy), lz = limbs(hz);
+    const long long X = mulk<2>(vx, lx), Y = mulk<2>(vy, ly), Z = mulk<2>(vz, lz);
+    const long long XY = FORCE ? mulk<2>(vx, ly) + mulk<2>(vy, lx) : mulk<2>(vx, ly) << 1;
+    const long long XZ = FORCE ? mulk<2>(vx, lz) + mulk<2>(vz, lx) : mulk<2>(vx, lz) << 1;
+    const long long YZ = FORCE ? mulk<2>(vy, lz) + mulk<2>(vz, ly) : mulk<2>(vy, lz) << 1;
+    constexpr long long third = 1537228672809129301LL;  // 2^62 / 3
+    const long long B = mulk<0>(limbs(m.r), limbs(k.w29)) - mulk<0>(limbs(X + Y + Z), limbs(third));
     const int E = m.E;
-    s[0] = EQ ? fx_out(B0, E) : fma(k.omc, s[0], fx_out(B0, E));
+    s[0] = EQ ? fx_out(3 * B, E - 1) : fma(k.omc, s[0], fx_out(3 * B, E - 1));
 #pragma unroll
     for (int p = 0; p < NPAIR; ++p) {
         const int i = pair_first(p);
+        const int Ep = p < 3 ? E - 2 : E - 3;
         long long e, o;
-        if (p == 0) { e = B1 + 2 * X; o = 2 * gx; }
-        else if (p == 1) { e = B1 + 2 * Y; o = 2 * gy; }
-        else if (p == 2) { e = B1 + 2 * Z; o = 2 * gz; }
-        else if (ez(i) == 0) { e = B2 + X + Y + (ey(i) > 0 ? XY : -XY); o = ey(i) > 0 ? gx + gy : gx - gy; }
-        else if (ey(i) == 0) { e = B2 + X + Z + (ez(i) > 0 ? XZ : -XZ); o = ez(i) > 0 ? gx + gz : gx - gz; }
-        else { e = B2 + Y + Z + (ez(i) > 0 ? YZ : -YZ); o = ez(i) > 0 ? gy + gz : gy - gz; }
-        s[i] = EQ ? fx_out(e + o, E) : fma(k.omc, s[i], fx_out(e + o, E));
-        s[opp(i)] = EQ ? fx_out(e - o, E) : fma(k.omc, s[opp(i)], fx_out(e - o, E));
+        if (p == 0) { e = B + X; o = gx; }
+        else if (p == 1) { e = B + Y; o = gy; }
+        else if (p == 2) { e = B + Z; o = gz; }
+        else if (ez(i) == 0) { e = B + X + Y + (ey(i) > 0 ? XY : -XY); o = ey(i) > 0 ? gx + gy : gx - gy; }
+        else if (ey(i) == 0) { e = B + X + Z + (ez(i) > 0 ? XZ : -XZ); o = ez(i) > 0 ? gx + gz : gx - gz; }
+        else { e = B + Y + Z + (ez(i) > 0 ? YZ : -YZ); o = ez(i) > 0 ? gy + gz : gy - gz; }
+        s[i] = EQ ? fx_out(e + o, Ep) : fma(k.omc, s[i], fx_out(e + o, Ep));
+        s[opp(i)] = EQ ? fx_out(e - o, Ep) : fma(k.omc, s[opp(i)], fx_out(e - o, Ep));
     }
 }
 
@@ -280,13 +297,13 @@ LBM_HD bool fixed_equilibrium(double f[Q], double rho1, double ux, double uy, do
     m.jz = fx_in(uz, E);
     m.fx = m.fy = m.fz = 0;
     if (!incomp) {  // j = u + rho1 u (rho1 as a 61-bit fraction)
-        const int n = 1023 - E - 5;
-        const L31 r = n >= 0 ? limbs(m.r >> (n < 63 ? n : 63)) : limbs(m.r << -n);
-        m.jx += mul62(r, limbs(m.jx)) << 1;
-        m.jy += mul62(r, limbs(m.jy)) << 1;
-        m.jz += mul62(r, limbs(m.jz)) << 1;
+        const int n = 1023 - E - 4;  // >= 2
+        const L31 r = limbs(m.r >> (n < 63 ? n : 63));
+        m.jx += mulk<1>(r, limbs(m.jx));
+        m.jy += mulk<1>(r, limbs(m.jy));
+        m.jz += mulk<1>(r, limbs(m.jz));
     }
-    fixed_collide<false, true>(f, m, FixedK{0x1c71c71c71c71c72LL, 0x0555555555555555LL, 0, 0.0}, incomp);
+    fixed_collide<false, true>(f, m, FixedK{0x0e38e38e38e38e39LL, 0x0555555555555555LL, 0, 0.0}, incomp);
     return true;
 }
 

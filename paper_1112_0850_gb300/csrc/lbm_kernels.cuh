@@ -1023,8 +1023,8 @@ __global__ void __launch_bounds__(step_threads<FLAT, S, FLAGS>(), step_min_block
 // fluid box's rows in order, across row ends. I: 32-bit lattice offsets where
 // they fit. RED: also the totals of the pre-collision state, per block. 5 blocks
 // of 128 threads per SM (<= 102 registers): channel 312 us a step, against 332
-// with 2 of 256 (125 registers) and 322 with 4 of 128 (266 since lbm_fixed.cuh
-// took fewer integer instructions).
+// with 2 of 256 (125 registers) and 322 with 4 of 128 (280 now, with the integer
+// instructions of lbm_fixed.cuh as they are).
 template <bool FLAGS, int FORCE, bool RECORD, bool RED, class I>
 __global__ void __launch_bounds__(128, 5)
     k_step64(const Dev d, const double *__restrict__ src, double *__restrict__ dst, double *__restrict__ out) {
