@@ -1414,6 +1414,20 @@ __device__ __forceinline__ void feq64(double f[Q], double rho1, double ux, doubl
     }
 }
 
+// Store the remainders g of a cell pair and its momentum words wa, wb.
+template <int S>
+__device__ __forceinline__ void split_put_pair(const Dev &d, typename Stor<S>::T *__restrict__ P, int x0, int c,
+                                               bool has1, const float2 g[Q], uint2 wa, uint2 wb) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) Stor<S>::st2(P + i * d.g.qs + c, g[i].x, g[i].y);
+    uint2 *J = split_words(d, P);
+    if (has1)
+        *reinterpret_cast<uint4 *>(J + c) = make_uint4(wa.x, wa.y, wb.x, wb.y);
+    else  // the lone last cell of an odd row: the slot after it holds cell 0's copy
+        J[c] = wa;
+    split_ghost(d, J, x0, c, wa);
+}
+
 // Write the 19 shifted values v of a cell pair to a moment-split lattice:
 // their momentum rounded to the format, then the remainders against it (the
 // tail of step_pair_split, for values that are not a collision's).
@@ -1438,14 +1452,66 @@ __device__ __forceinline__ void split_store_pair(const Dev &d, typename Stor<S>:
         v[i] = vfma(vsplat(-split_k(i)), e, v[i]);
         v[io] = vfma(vsplat(-split_k(io)), e, v[io]);
     }
+    split_put_pair<S>(d, P, x0, c, has1, v, wa, wb);
+}
+
+// a + b rounded to odd: exact if a float holds the sum, else the neighbour with an odd
+// last bit. Rounding that to 16 bits gives the sum rounded once.
+__device__ __forceinline__ float odd_of(float down, float up) { return __float_as_uint(down) & 1u ? down : up; }
+__device__ __forceinline__ float2 odd_add(float2 a, float2 b) {
+    return make_float2(odd_of(__fadd_rd(a.x, b.x), __fadd_ru(a.x, b.x)), odd_of(__fadd_rd(a.y, b.y), __fadd_ru(a.y, b.y)));
+}
+__device__ __forceinline__ float2 odd_fma(float k, float2 a, float2 b) {
+    return make_float2(odd_of(__fmaf_rd(k, a.x, b.x), __fmaf_ru(k, a.x, b.x)),
+                       odd_of(__fmaf_rd(k, a.y, b.y), __fmaf_ru(k, a.y, b.y)));
+}
+// A sum of floats and the sum of its roundings.
+struct Sum2 {
+    float2 s, e;
+    // (Knuth's two-sum: b's part of the rounded sum, then what both lost)
+    __device__ __forceinline__ void add(float2 b) {
+        const float2 t = vadd(s, b), v = vsub(t, s);
+        e = vadd(e, vadd(vsub(s, vsub(t, v)), vsub(b, v)));
+        s = t;
+    }
+};
+__device__ __forceinline__ Sum2 operator-(float2 a, float2 b) {
+    Sum2 r = {a, vsplat(0.0f)};
+    r.add(vmul(b, vsplat(-1.0f)));
+    return r;
+}
+__device__ __forceinline__ Sum2 operator+(Sum2 a, Sum2 b) {
+    a.add(b.s);
+    a.e = vadd(a.e, b.e);
+    return a;
+}
+__device__ __forceinline__ Sum2 operator-(Sum2 a) { return Sum2{vmul(a.s, vsplat(-1.0f)), vmul(a.e, vsplat(-1.0f))}; }
+
+// The same from values of a canonical state, which is exchanged unrounded: the
+// momentum and the remainders are each rounded once, to 16 bits, as split_store
+// rounds them from double (in FP32, twice). FP64 adds would take 2.5 ms for a 256^3
+// box, which moves in 0.3.
+template <int S>
+__device__ __forceinline__ void split_store_pair_once(const Dev &d, typename Stor<S>::T *__restrict__ P, int x0, int c,
+                                                      bool has1, float2 v[Q]) {
+    const Sum2 a = v[7] - v[10], b = v[8] - v[9], e = v[11] - v[14], f = v[12] - v[13], g = v[15] - v[18],
+               h = v[16] - v[17];
+    const Sum2 jx = (v[1] - v[2]) + a + b + e + f, jy = (v[3] - v[4]) + a + -b + g + h,
+               jz = (v[5] - v[6]) + e + -f + g + -h;
+    const float2 ox = odd_add(jx.s, jx.e), oy = odd_add(jy.s, jy.e), oz = odd_add(jz.s, jz.e);
+    const uint2 wa = make_uint2(SplitJ<S>::pack(ox.x, oy.x), SplitJ<S>::pack(oz.x, 0.0f));
+    const uint2 wb = make_uint2(SplitJ<S>::pack(ox.y, oy.y), SplitJ<S>::pack(oz.y, 0.0f));
+    const float2 tx = make_float2(SplitJ<S>::lo(wa.x), SplitJ<S>::lo(wb.x));
+    const float2 ty = make_float2(SplitJ<S>::hi(wa.x), SplitJ<S>::hi(wb.x));
+    const float2 tz = make_float2(SplitJ<S>::lo(wa.y), SplitJ<S>::lo(wb.y));
 #pragma unroll
-    for (int i = 0; i < Q; ++i) Stor<S>::st2(P + i * d.g.qs + c, v[i].x, v[i].y);
-    uint2 *J = split_words(d, P);
-    if (has1)
-        *reinterpret_cast<uint4 *>(J + c) = make_uint4(wa.x, wa.y, wb.x, wb.y);
-    else  // the lone last cell of an odd row: the slot after it holds cell 0's copy
-        J[c] = wa;
-    split_ghost(d, J, x0, c, wa);
+    for (int p = 0; p < NPAIR; ++p) {
+        const int i = pair_first(p), io = opp(i);
+        const float2 w = edot_first(i, tx, ty, tz);
+        v[i] = odd_fma(-split_k(i), w, v[i]);
+        v[io] = odd_fma(-split_k(io), w, v[io]);
+    }
+    split_put_pair<S>(d, P, x0, c, has1, v, wa, wb);
 }
 
 // f_eq_i - w_i of two cells.
@@ -1643,6 +1709,17 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
     }
 }
 
+// The values v of a cell, each with its moving-wall term where bit i of mv is set, to
+// a moment-split lattice.
+template <int S>
+static __device__ __noinline__ void split_store_moving(const Dev &d, typename Stor<S>::T *P, int x, int c, uint32_t mv,
+                                                       const float *v) {
+    double t[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) t[i] = (double)v[i] + ((mv >> i) & 1u ? d.wc[i] : 0.0);
+    split_store<S>(d, P, x, c, t);
+}
+
 // ---------------------------------------------------------------------------
 // get_state: canonical shifted f^n = gather(P), format D; solid cells 0.
 // Bound by HBM (19 values read and 19 written a cell). One cell a thread with
@@ -1678,9 +1755,8 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
 // set_state: P_i(y) = s_i(y + e_i) if fluid there, else s_{opp(i)}(y). The
 // loads follow the reverse step's gather (sources y + e_i, the pair's own
 // values over them where a mask bit is set). Moment-split storage collects the
-// 19 values its cells hold, in FP32 unless they come as doubles: the remainders
-// are formed by one rounded multiply-add, as in the step, before their 16-bit
-// rounding (256^3 box from FP32 287 us; in double 3017).
+// 19 values its cells hold and rounds momentum and remainders once, whatever format
+// they come in (256^3 box from FP32 301 us; in double 3017).
 template <int S, int D, bool FLAGS>
 __global__ void __launch_bounds__(128, FLAGS && !is_split(S) && S != LBM_F64 ? 7 : 2 * FieldBlocks<S, FLAGS>::value)
     k_set_state(const Dev d, typename Stor<S>::T *__restrict__ P, const typename IOFmt<D>::T *__restrict__ in,
@@ -1750,14 +1826,21 @@ __global__ void __launch_bounds__(128, FLAGS && !is_split(S) && S != LBM_F64 ? 7
                          : make_uint2(0u, 0u);
     if constexpr (is_split(S) && sizeof(V) == 4) {
         if (FLAGS && !live0 && !live1) return;
+        if (d.moving_on && (mv.x | mv.y)) {  // rare: with the walls' terms, in double
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (!(k ? live1 : live0)) continue;
+                float t[Q];
+#pragma unroll
+                for (int i = 0; i < Q; ++i) t[i] = k ? s1[i] : s0[i];
+                split_store_moving<S>(d, P, x0 + k, c + k, k ? mv.y : mv.x, t);
+            }
+            return;
+        }
         float2 v[Q];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            v[i] = make_float2(s0[i], s1[i]);
-            if (d.moving_on && ((mv.x >> i) & 1u)) v[i].x += d.wcf[i];
-            if (d.moving_on && ((mv.y >> i) & 1u)) v[i].y += d.wcf[i];
-        }
-        split_store_pair<S>(d, P, x0, c, has1, v);
+        for (int i = 0; i < Q; ++i) v[i] = make_float2(s0[i], s1[i]);
+        split_store_pair_once<S>(d, P, x0, c, has1, v);
         return;
     } else if constexpr (is_split(S)) {
 #pragma unroll
