@@ -182,6 +182,9 @@ void lbm_destroy(lbm_ctx *ctx);
 
 lbm_status lbm_get_info(const lbm_ctx *ctx, lbm_info *info);
 
+/* Whether some cell is flagged 2 (counted at creation): 1 or 0. */
+int lbm_has_moving_walls(const lbm_ctx *ctx);
+
 /* Replace the uniform body force (host array of 3 doubles; NULL = zero). */
 lbm_status lbm_set_uniform_force(lbm_ctx *ctx, const double force[3]);
 

@@ -52,6 +52,7 @@ PROTOTYPES = {
     "lbm_create": (_st, [ctypes.POINTER(_vp), _i, _i, _i, ctypes.c_double, _vp, _vp, ctypes.POINTER(lbm_options)]),
     "lbm_destroy": (None, [_vp]),
     "lbm_get_info": (_st, [_vp, ctypes.POINTER(lbm_info)]),
+    "lbm_has_moving_walls": (_i, [_vp]),
     "lbm_set_uniform_force": (_st, [_vp, _vp]),
     "lbm_set_wall_velocity": (_st, [_vp, _vp]),
     "lbm_set_force_field": (_st, [_vp, _vp]),

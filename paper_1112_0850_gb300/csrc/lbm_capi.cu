@@ -537,6 +537,8 @@ lbm_status lbm_get_info(const lbm_ctx *ctx, lbm_info *info) {
     return LBM_OK;
 }
 
+int lbm_has_moving_walls(const lbm_ctx *ctx) { return ctx && ctx->has_moving ? 1 : 0; }
+
 lbm_status lbm_set_uniform_force(lbm_ctx *ctx, const double force[3]) {
     if (check_ctx(ctx)) return LBM_ERR_ARG;
     cudaStreamSynchronize(ctx->stream);

@@ -60,7 +60,6 @@ class Lattice:
             fl = np.ascontiguousarray(np.asarray(flags.cpu() if torch.is_tensor(flags) else flags), dtype=np.uint8)
             assert fl.shape == self.shape, (fl.shape, self.shape)
         self._flags_host = fl
-        self.has_moving_walls = bool(fl is not None and fl.max(initial=0) >= 2 and (fl == 2).any())
         F = None if force is None else (ctypes.c_double * 3)(*[float(v) for v in force])
         h = ctypes.c_void_p()
         st = L.lbm_create(ctypes.byref(h), int(nx), int(ny), int(nz), float(tau),
@@ -116,6 +115,10 @@ class Lattice:
     @property
     def n_fluid(self):
         return self.info.n_fluid
+
+    @property
+    def has_moving_walls(self):
+        return bool(capi.lib().lbm_has_moving_walls(self.handle))
 
     def zeros(self, *lead, dtype=None, device="cuda"):
         return torch.zeros(*lead, *self.shape, dtype=dtype or self.real, device=device)
