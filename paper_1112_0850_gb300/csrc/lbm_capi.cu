@@ -101,6 +101,13 @@ int pitch_for(int nx, lbm_storage s, int row_align = 0) {
     return (nx + per - 1) / per * per;
 }
 
+// Device bytes that lbm_create allocates: lattices, reduction scratch, and with
+// flags these and the push masks (and the moving-wall words behind them).
+size_t create_bytes(lbm_storage s, long long qs, bool aa, bool flags, bool moving) {
+    return (aa ? 1 : 2) * lattice_bytes_of(s, qs) + (flags ? (moving ? 9 : 5) * (size_t)qs : 0) +
+           ((size_t)RED_BLOCKS * 4 + 8) * sizeof(double);
+}
+
 bool is_device_ptr(const void *p) {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
@@ -382,10 +389,7 @@ lbm_status lbm_create(lbm_ctx **out, int nx, int ny, int nz, double tau, const u
         delete ctx;
         return LBM_ERR_CUDA;
     }
-    // lattices, flags and push masks, reduction scratch
-    const size_t need = (aa ? 1 : 2) * lat_bytes + (flags ? 5 * (size_t)qs : 0) +
-                        ((size_t)RED_BLOCKS * 4 + 8) * sizeof(double);
-    if (need > free_b) {
+    if (create_bytes(o.storage, qs, aa, flags != nullptr, false) > free_b) {
         delete ctx;
         return LBM_ERR_OOM;
     }
@@ -438,6 +442,10 @@ lbm_status lbm_create(lbm_ctx **out, int nx, int ny, int nz, double tau, const u
         }
     }
     ctx->n_fluid = n_fluid;
+    if (create_bytes(o.storage, qs, aa, flags != nullptr, ctx->has_moving) > free_b) {
+        delete ctx;
+        return LBM_ERR_OOM;
+    }
     bool ok = cudaMalloc(&ctx->lat[0], lat_bytes) == cudaSuccess &&
               (aa || cudaMalloc(&ctx->lat[1], lat_bytes) == cudaSuccess) &&
               cudaMalloc((void **)&ctx->red_partials, (size_t)RED_BLOCKS * 4 * sizeof(double)) == cudaSuccess &&
