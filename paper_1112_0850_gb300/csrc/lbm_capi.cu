@@ -948,18 +948,6 @@ lbm_status lbm_adjoint_halo_unpack(lbm_ctx *ctx, int side, const void *buf) {
 }
 
 static lbm_status ensure_lambda(lbm_ctx *ctx) {
-    // the reverse step gathers with the push masks (built at create; kept
-    // here for a context whose masks are missing)
-    if (ctx->flags_d && !ctx->mask_d) {
-        cudaError_t e = cudaMalloc((void **)&ctx->mask_d, (size_t)ctx->g.qs * sizeof(uint32_t));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            ctx->mask_d = nullptr;
-            return fail(ctx, LBM_ERR_OOM, "cannot allocate the push masks");
-        }
-        e = build_push_mask(ctx->g, ctx->flags_d, ctx->mask_d, ctx->moving_d, ctx->stream);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "push mask build");
-    }
     const size_t bytes = (size_t)Q * (size_t)ctx->g.qs * real_size(ctx->storage);
     for (int k = 0; k < 2; ++k) {
         if (ctx->lam[k]) continue;

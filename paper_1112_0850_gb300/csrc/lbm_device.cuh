@@ -596,9 +596,6 @@ template <class R> struct OddK;
 template <> struct OddK<float> {
     static constexpr float AXIS = 0x1.555554p-3f, DIAG = 0x1.555556p-4f;
 };
-template <> struct OddK<double> {
-    static constexpr double AXIS = 0x1.5555555555554p-3, DIAG = 0x1.5555555555556p-4;
-};
 
 // BGK relaxation (Eq. 1) with the Qian equilibrium and the Guo source, both
 // cells of the pair, populations in shifted form. Per opposite pair
@@ -615,7 +612,7 @@ template <> struct OddK<double> {
 //   a = w rho1 [- 3 w c' u.F],   b = w rho,   K = 3 w (OddK),
 // A, C and c' = tau - 1/2 those of the source over omega (guo2).
 //
-// Otherwise (FP64, 16-bit storage): s_i <- (1 - omega) s_i + E + P and
+// Otherwise (16-bit storage): s_i <- (1 - omega) s_i + E + P and
 // s_opp(i) <- (1 - omega) s_opp(i) + E - P, with omega folded in:
 //   E = a + b t [+ e A],   P = 3 b e [+ C],   a = omega w rho1 [- 3 w c u.F],
 //   b = omega w rho,   c = 1 - omega/2,

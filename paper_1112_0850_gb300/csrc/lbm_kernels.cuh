@@ -148,8 +148,7 @@ __device__ __forceinline__ void split_ghost(const Dev &d, uint2 *J, int x, int c
     if ((d.g.nx & 1) && x == 0) J[c + d.g.nx] = w;
 }
 
-// Round to the 16-bit format (nearest even) from float or double.
-template <int S> __device__ __forceinline__ unsigned split_pack(float a, float b) { return SplitJ<S>::pack(a, b); }
+// Two values rounded to the 16-bit format (nearest even) from double.
 template <int S> __device__ __forceinline__ unsigned split_pack(double a, double b) {
     union {
         unsigned short h[2];
@@ -165,24 +164,24 @@ template <int S> __device__ __forceinline__ unsigned split_pack(double a, double
     return v.u;
 }
 
-// Write one cell's 19 shifted values v (float or double) at cell c of a
+// Write one cell's 19 shifted values v at cell c of a
 // moment-split lattice: J = sum_i v_i e_i rounded to the format, then the
 // remainders g_i = v_i - K_i (e_i . J) rounded.
-template <int S, class V>
-__device__ __forceinline__ void split_store(const Dev &d, typename Stor<S>::T *P, int x, int c, const V v[Q]) {
-    V jx = V(0), jy = V(0), jz = V(0);
+template <int S>
+__device__ __forceinline__ void split_store(const Dev &d, typename Stor<S>::T *P, int x, int c, const double v[Q]) {
+    double jx = 0.0, jy = 0.0, jz = 0.0;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         if (ex(i)) jx += ex(i) > 0 ? v[i] : -v[i];
         if (ey(i)) jy += ey(i) > 0 ? v[i] : -v[i];
         if (ez(i)) jz += ez(i) > 0 ? v[i] : -v[i];
     }
-    const unsigned wx = split_pack<S>(jx, jy), wy = split_pack<S>(jz, V(0));
+    const unsigned wx = split_pack<S>(jx, jy), wy = split_pack<S>(jz, 0.0);
     const uint2 w = make_uint2(wx, wy);
     P[c] = Rn<typename Stor<S>::T>::of(v[0]);
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-        const V g = fma(V(-split_k(i)), V(split_edot<S>(split_first(i), w)), v[i]);
+        const double g = fma((double)-split_k(i), (double)split_edot<S>(split_first(i), w), v[i]);
         P[(long long)i * d.g.qs + c] = Rn<typename Stor<S>::T>::of(g);
     }
     split_words(d, P)[c] = w;
@@ -209,12 +208,9 @@ template <class R> __device__ __forceinline__ R wall_term(const Dev &d, int i);
 template <> __device__ __forceinline__ float wall_term<float>(const Dev &d, int i) { return d.wcf[i]; }
 template <> __device__ __forceinline__ double wall_term<double>(const Dev &d, int i) { return d.wc[i]; }
 
-// NaN marks solid slots in the NaN-mark form and in the AA pattern. (In the
-// AA pattern they are hygiene only: the odd step's mask-free scatter stores
-// into solid slots, and no reader takes a solid slot's value.)
-template <int S> __device__ __forceinline__ bool nan_marked(const Dev &d) {
-    return bounce_mode(S) == BB_NANS || d.layout != LAYOUT_PULL;
-}
+// NaN marks solid slots in the AA pattern. (It is hygiene only: the odd step's
+// mask-free scatter stores into solid slots, and no reader takes a solid slot's value.)
+__device__ __forceinline__ bool nan_marked(const Dev &d) { return d.layout != LAYOUT_PULL; }
 
 // ---------------------------------------------------------------------------
 // Fused stream-collide (Sec. 2 steps 1-3, Eq. 1; Sec. 6 pull-style update).
@@ -233,14 +229,8 @@ template <int S> __device__ __forceinline__ bool nan_marked(const Dev &d) {
 //    does not wait for it (every load takes the neighbour's address); pairs
 //    with a bounce bit then reload their bounced populations from the cell's
 //    own opposite slots, over the gathered values, before the moments.
-//    Solid slots are never read. 37.5 against 34.0 GFLUPS for NaN marks on
-//    the channel, which test each value and take the moments twice.
-//  - NaN marks (kept as the measured alternative): every slot of a solid cell
-//    holds NaN (written at create, init and set_state, and stored by the step
-//    for solid cells). The gather loads all 19 values without looking at
-//    flags; a NaN marks a solid source, so a NaN rho finds the cells next to a
-//    solid, and only those lanes then load the opposite population of the
-//    cell itself and take their moments again.
+//    Solid slots are never read. 37.5 against 34.0 GFLUPS on the channel for
+//    solid slots that hold NaN, each value tested and the moments taken twice.
 //  - separate kernel (16-bit storage), the paper's arrangement (Sec. 7: the
 //    non-fluid cells are treated in a separate kernel): a solid cell s keeps in
 //    slot i the value that its fluid neighbour s + e_i pulls next step (that
@@ -251,9 +241,10 @@ template <int S> __device__ __forceinline__ bool nan_marked(const Dev &d) {
 // populations, which is what the flag-aware readers (macros, state, reduction,
 // adjoint) gather.
 //
-// Resident blocks of 256 threads per SM the step kernels are compiled for:
-// FP64 arithmetic 1 (<= 255 registers), FP32 storage 3 (<= 80), 16-bit
-// storage 4 (<= 64: fewer bytes per thread, so more threads in flight).
+// Resident blocks of 256 threads per SM (two of 128 for one of 256 in the flat
+// launch): FP32 storage 3 (<= 80 registers), 16-bit storage 4 (<= 64: fewer bytes
+// per thread, so more threads in flight); the FP64 AA steps, two cells a thread,
+// 1 (<= 255). The FP64 two-grid step has its own (k_step64).
 template <int S> struct StepBlocks {
     static constexpr int value = S == LBM_F64 ? 1 : ((S == LBM_F32 || is_split(S)) ? 3 : 4);
 };
@@ -579,8 +570,7 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
     typedef typename Stor<S>::R R;
     typedef typename Pair2<R>::V V;  // lane x: cell x0, lane y: cell x0 + 1
     constexpr bool MFIX = Bounce<S>::mode == BB_MFIX;
-    constexpr bool LINKS = !MFIX;  // flag-free gather (links or NaN marks)
-    constexpr bool NANS = Bounce<S>::mode == BB_NANS;
+    constexpr bool LINKS = !MFIX;  // flag-free gather
     const Geom &g = d.g;
     const bool has1 = x0 + 1 < g.nx;
     const int c = cell_index(g, x0, y, z);
@@ -652,27 +642,7 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
         ld2_real(F + 2 * g.qs + c, Fz.x, Fz.y);
         G = guo2<R>(relax_about_t(S) ? DevR<R>::cs(d) : R(1) - R(0.5) * DevR<R>::omega(d), Fx, Fy, Fz);
     }
-    Mom2<R> m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
-    if (FLAGS && NANS && ((live0 && m.rho.x != m.rho.x) || (live1 && m.rho.y != m.rho.y))) {
-        // A solid source slot holds NaN, and a NaN anywhere makes rho NaN, so
-        // one test per cell finds the cells next to a solid. Only those reload
-        // each NaN population from the opposite slot of the cell itself
-        // (halfway bounce-back, plus the moving-wall term) and take their
-        // moments again.
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            const T *Po = lat_at<I>(src, opp(i), g.qs, c);
-            if (live0 && s[i].x != s[i].x) {
-                s[i].x = Stor<S>::ld(Po);
-                if (d.moving_on && ((__ldg(d.moving + c) >> opp(i)) & 1u)) s[i].x += wall_term<R>(d, i);
-            }
-            if (live1 && s[i].y != s[i].y) {
-                s[i].y = Stor<S>::ld(Po + 1);
-                if (d.moving_on && ((__ldg(d.moving + c + 1) >> opp(i)) & 1u)) s[i].y += wall_term<R>(d, i);
-            }
-        }
-        m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
-    }
+    const Mom2<R> m = moments2<R, FORCE != 0>(s, Fx, Fy, Fz, d.incomp);
     const bool bad0 = live0 && !(m.rho.x > R(0) && m.rho.x < R(1e30));
     const bool bad1 = live1 && !(m.rho.y > R(0) && m.rho.y < R(1e30));
     if (bad0 || bad1) atomicOr(d.status, LBM_STATUS_DIVERGED);
@@ -686,18 +656,12 @@ __device__ __forceinline__ void step_pair(const Dev &d, const Rows &rows, const 
     }
     collide2<R, FORCE != 0, relax_about_t(S)>(s, m, DevR<R>::omega(d), DevR<R>::cs(d), Fx, Fy, Fz, G, d.incomp);
     // The pair is stored whole, a solid cell included, so 32-byte sectors are
-    // written complete: a solid cell's values are never read (load side and
-    // mask-guided reload, where all-solid sectors are left out below), it
-    // stores the NaN that marks it (NaN marks), or its slots are link targets
-    // that k_bounce rewrites (links). When moving-wall links are written into
-    // solid slots by other threads of this launch, a pair with a solid cell
-    // stores its fluid cell alone.
-    if (FLAGS && NANS) {
-        const R nan = quiet_nan<R>();
-#pragma unroll
-        for (int i = 0; i < Q; ++i)
-            Stor<S>::st2(lat_at<I>(dst, i, g.qs, c), live0 ? s[i].x : nan, live1 ? s[i].y : nan);
-    } else if (FLAGS && LinkBounce<S>::value && d.has_moving && !(live0 && live1)) {
+    // written complete: a solid cell's values are never read (mask-guided
+    // reload, where all-solid sectors are left out below), or its slots are
+    // link targets that k_bounce rewrites (links). When moving-wall links are
+    // written into solid slots by other threads of this launch, a pair with a
+    // solid cell stores its fluid cell alone.
+    if (FLAGS && LinkBounce<S>::value && d.has_moving && !(live0 && live1)) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             if (live0) Stor<S>::st(lat_at<I>(dst, i, g.qs, c), s[i].x);
@@ -1774,7 +1738,7 @@ __global__ void __launch_bounds__(128, FLAGS && !is_split(S) && S != LBM_F64 ? 7
     uint32_t m0, m1;
     bool live0, live1;
     pair_masks<FLAGS>(d, c, has1, m0, m1, live0, live1);
-    const bool mark = FLAGS && nan_marked<S>(d);
+    const bool mark = FLAGS && nan_marked(d);
     if (FLAGS && !mark && !live0 && !live1) return;
     V s0[Q], s1[Q];
     if (!is_split(S) && d.layout == LAYOUT_AA_NAT) {  // AA natural layout: s_i(x) at the cell itself
@@ -2139,23 +2103,23 @@ static cudaError_t launch_step3f(const Dev &d, const void *src, void *dst, void 
                             static_cast<R *>(tape));
 }
 
-// The flat launch where whole rows would leave lanes idle, and also where it
-// measured faster with whole-warp rows (its index code compiles to fewer
-// spills): FP32 (walled channel +1%) and 16-bit storage without flags (512^3
-// box +3%). The 16-bit link form with flags keeps whole rows there (the flat
-// form spilled more: -4.5%); so does FP64.
-template <int S, bool FLAGS> constexpr bool flat_preferred() {
-    return S == LBM_F32 || is_split(S) || (S != LBM_F64 && !FLAGS);
-}
+// Always the flat launch where that measured faster with whole-warp rows too (its
+// index code compiles to fewer spills): FP32 (walled channel +1%) and 16-bit storage
+// without flags (512^3 box +3%). The 16-bit link form with flags takes it only where
+// whole rows would leave lanes idle, or on small lattices (the flat form spilled
+// more: -4.5%).
+template <int S, bool FLAGS> constexpr bool always_flat() { return S == LBM_F32 || is_split(S) || !FLAGS; }
 
 template <int S, bool FLAGS, int FORCE>
 static cudaError_t launch_step3(const Dev &d, const void *src, void *dst, void *tape) {
-    if constexpr (is_split(S))  // (always the flat launch)
+    if constexpr (is_split(S))
         return (d.g.nx & 1) ? launch_step3f<S, FLAGS, FORCE, true, true>(d, src, dst, tape)
                             : launch_step3f<S, FLAGS, FORCE, true, false>(d, src, dst, tape);
+    else if constexpr (always_flat<S, FLAGS>())
+        return launch_step3f<S, FLAGS, FORCE, true>(d, src, dst, tape);
     else
-        return d.flat_step || flat_preferred<S, FLAGS>() ? launch_step3f<S, FLAGS, FORCE, true>(d, src, dst, tape)
-                                                         : launch_step3f<S, FLAGS, FORCE, false>(d, src, dst, tape);
+        return d.flat_step ? launch_step3f<S, FLAGS, FORCE, true>(d, src, dst, tape)
+                           : launch_step3f<S, FLAGS, FORCE, false>(d, src, dst, tape);
 }
 
 // Shared memory of the row-staged step: two buffers of 19 padded rows.
@@ -2163,9 +2127,8 @@ constexpr int TMA_SMEM_MAX = 200 * 1024;
 template <int S> inline int tma_smem_bytes(const Dev &d) {
     return 2 * Q * d.g.pitch * (int)sizeof(typename Stor<S>::T) + 16;
 }
-// The row-staged step serves the flag-free gathers (NaN marks, links) of
-// FP32 and 16-bit storage when rows are whole 16-byte multiples and two
-// buffers fit.
+// The row-staged step serves FP32 and 16-bit shifted storage when rows are
+// whole 16-byte multiples and two buffers fit.
 template <int S> inline bool tma_eligible(const Dev &d) {
     const long long rowbytes = (long long)d.g.pitch * sizeof(typename Stor<S>::T);
     return d.row_staging && rowbytes % 16 == 0 && tma_smem_bytes<S>(d) <= TMA_SMEM_MAX;
@@ -2264,19 +2227,29 @@ cudaError_t Ops<S>::bounce(const Dev &d, void *dst) {
     return cudaGetLastError();
 }
 
-// The fused step-reduce kernel for one launch mapping (FLAT) and row parity (ODD).
-template <int S, bool FLAT, bool ODD>
-static void launch_step_reduce2(const Dev &d, const dim3 grid, const dim3 block, const typename Stor<S>::T *s,
-                                typename Stor<S>::T *t, double *partials) {
-    if (d.flags) {
-        if (d.Ffield) k_step_reduce<S, true, 2, FLAT, ODD><<<grid, block, 0, d.stream>>>(d, s, t, partials);
-        else if (d.force_on) k_step_reduce<S, true, 1, FLAT, ODD><<<grid, block, 0, d.stream>>>(d, s, t, partials);
-        else k_step_reduce<S, true, 0, FLAT, ODD><<<grid, block, 0, d.stream>>>(d, s, t, partials);
-    } else {
-        if (d.Ffield) k_step_reduce<S, false, 2, FLAT, ODD><<<grid, block, 0, d.stream>>>(d, s, t, partials);
-        else if (d.force_on) k_step_reduce<S, false, 1, FLAT, ODD><<<grid, block, 0, d.stream>>>(d, s, t, partials);
-        else k_step_reduce<S, false, 0, FLAT, ODD><<<grid, block, 0, d.stream>>>(d, s, t, partials);
+// The fused step-reduce kernel, with the launch mapping of the plain step
+// (launch_step3); grid: its blocks, one partial each.
+template <int S, bool FLAGS, int FORCE>
+static cudaError_t launch_step_reduce3(const Dev &d, const void *src, void *dst, double *partials, dim3 &grid) {
+    typedef typename Stor<S>::T T;
+    const bool flat = always_flat<S, FLAGS>() || d.flat_step;
+    const RowLaunch &P = flat ? d.PF : d.P;
+    const dim3 block(P.bx_threads, P.by_threads);
+    grid = dim3(P.nxb * P.nyb, P.nzr);
+    void (*k)(Dev, const T *, T *, double *) = k_step_reduce<S, FLAGS, FORCE, true>;
+    if constexpr (is_split(S)) {
+        if (d.g.nx & 1) k = k_step_reduce<S, FLAGS, FORCE, true, true>;
+    } else if constexpr (!always_flat<S, FLAGS>()) {
+        if (!flat) k = k_step_reduce<S, FLAGS, FORCE, false>;
     }
+    k<<<grid, block, 0, d.stream>>>(d, static_cast<const T *>(src), static_cast<T *>(dst), partials);
+    return cudaGetLastError();
+}
+template <int S, bool FLAGS>
+static cudaError_t launch_step_reduce2(const Dev &d, const void *src, void *dst, double *partials, dim3 &grid) {
+    if (d.Ffield) return launch_step_reduce3<S, FLAGS, 2>(d, src, dst, partials, grid);
+    if (d.force_on) return launch_step_reduce3<S, FLAGS, 1>(d, src, dst, partials, grid);
+    return launch_step_reduce3<S, FLAGS, 0>(d, src, dst, partials, grid);
 }
 
 template <int S>
@@ -2298,34 +2271,21 @@ cudaError_t Ops<S>::step_reduce(const Dev &d, const void *src, void *dst, double
         const int n = (int)(grid.x * grid.y);
         return sum_partials(partials, n, partials + 4 * (size_t)n, out, d.stream);
     } else {
-        const T *s = static_cast<const T *>(src);
-        T *t = static_cast<T *>(dst);
-        // the launch mapping of the plain step (launch_step3)
-        const bool flat = d.flat_step || (d.flags ? flat_preferred<S, true>() : flat_preferred<S, false>());
-        const RowLaunch &P = flat ? d.PF : d.P;
-        const dim3 grid(P.nxb * P.nyb, P.nzr), block(P.bx_threads, P.by_threads);
-        if constexpr (is_split(S)) {  // (always the flat launch)
-            if (d.g.nx & 1)
-                launch_step_reduce2<S, true, true>(d, grid, block, s, t, partials);
-            else
-                launch_step_reduce2<S, true, false>(d, grid, block, s, t, partials);
-        } else if (flat) {
-            launch_step_reduce2<S, true, false>(d, grid, block, s, t, partials);
-        } else {
-            launch_step_reduce2<S, false, false>(d, grid, block, s, t, partials);
-        }
-        cudaError_t e = cudaGetLastError();
+        dim3 grid;
+        cudaError_t e = d.flags ? launch_step_reduce2<S, true>(d, src, dst, partials, grid)
+                                : launch_step_reduce2<S, false>(d, src, dst, partials, grid);
         if (e != cudaSuccess) return e;
         if (d.flags && LinkBounce<S>::value && d.link_max > 0) {
             const int per_block = 256 * LINKS_PER_THREAD;
-            k_bounce<S><<<dim3(Q - 1, (d.link_max + per_block - 1) / per_block), 256, 0, d.stream>>>(d, t);
+            k_bounce<S><<<dim3(Q - 1, (d.link_max + per_block - 1) / per_block), 256, 0, d.stream>>>(
+                d, static_cast<T *>(dst));
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
         return sum_partials(partials, (int)(grid.x * grid.y), partials + 4 * (size_t)grid.x * grid.y, out, d.stream);
     }
 }
 
-// NaN marks on every slot of every solid cell (NaN-mark form; no-op otherwise).
+// NaN marks on every slot of every solid cell (AA pattern; no-op otherwise).
 template <int S>
 __global__ void __launch_bounds__(256) k_fill_solid(const Dev d, typename Stor<S>::T *__restrict__ P) {
     int x, y, z;
@@ -2339,7 +2299,7 @@ __global__ void __launch_bounds__(256) k_fill_solid(const Dev d, typename Stor<S
 
 template <int S>
 cudaError_t Ops<S>::fill_solid(const Dev &d, void *lat) {
-    if (!d.flags || (Bounce<S>::mode != BB_NANS && d.layout == LAYOUT_PULL)) return cudaSuccess;
+    if (!d.flags || d.layout == LAYOUT_PULL) return cudaSuccess;
     k_fill_solid<S><<<row_grid(d), row_block(d), 0, d.stream>>>(d, static_cast<typename Stor<S>::T *>(lat));
     return cudaGetLastError();
 }

@@ -68,13 +68,14 @@ template <> struct DevR<double> {
     static __device__ __forceinline__ double F(const Dev &d, int a) { return d.F[a]; }
 };
 
-// Bounce-back form per storage format (see k_step), the measured fastest on
-// the walled channel: FP64 and FP32 mask-guided reload, 16-bit link
-// kernel (BB_NANS, NaN marks with a rho-gated fix-up, is kept as the
-// measured alternative). The moment-split formats take the mask-guided
-// reload: a bounced value is rebuilt from the cell's own momentum, which a
-// copy into a solid slot could not carry.
-enum { BB_LINKS = 1, BB_NANS = 2, BB_MFIX = 3 };
+// Bounce-back form per storage format (see k_step): FP64, FP32 and the
+// moment-split formats the mask-guided reload (a bounced split value is rebuilt
+// from the cell's own momentum, which a copy into a solid slot could not carry),
+// 16-bit storage the link kernel. (On whole rows in blocks of 256 the reload was
+// slower than it there; on the flat launch with 32-bit offsets and 7 blocks of 128
+// it took 76.5 us on the walled FP16 channel against 61.5 + 26.5. What is left to
+// settle is a moving wall's values, which the links round once.)
+enum { BB_LINKS = 1, BB_MFIX = 2 };
 __host__ __device__ constexpr int bounce_mode(int s) {
     return s == LBM_F64 || s == LBM_F32 || is_split(s) ? BB_MFIX : BB_LINKS;
 }
@@ -84,9 +85,9 @@ __host__ __device__ constexpr bool bounce_in_solid(int s) { return bounce_mode(s
 
 // The collision's rounding form per storage format (collide2): FP32 relaxes
 // about T = s_eq + S/omega with the momentum-exact odd part, which keeps
-// rounding from biasing mass and momentum step after step; FP64 (bias at the
-// 1e-16 level, ALU-bound) and 16-bit storage (error set by the storage
-// rounding) keep the cheaper omega-scaled form.
+// rounding from biasing mass and momentum step after step; 16-bit storage (error
+// set by the storage rounding) keeps the cheaper omega-scaled form, and FP64 has
+// its own (lbm_fixed.cuh).
 __host__ __device__ constexpr bool relax_about_t(int s) { return s == LBM_F32; }
 
 // Links each k_bounce block copies at most (256 threads x 4), and the most
@@ -102,8 +103,7 @@ template <int S> struct Ops {
     // One fused stream-collide step: dst = C(G(src)); tape (nullable) gets
     // (rho, ux, uy, uz) of the pre-collision state, padded [4][qs] of R.
     static cudaError_t step(const Dev &d, const void *src, void *dst, void *tape);
-    // Mark the solid cells of lat for the NaN-mark form of bounce-back and the
-    // AA pattern (no-op otherwise).
+    // Mark the solid cells of lat in the AA pattern (no-op otherwise).
     static cudaError_t fill_solid(const Dev &d, void *lat);
     // lat = P^{-1} such that gathering it gives f_eq(rho0, u0); rho0 nullable.
     static cudaError_t init_eq(const Dev &d, void *lat, const void *rho0, const void *u0);
