@@ -1141,14 +1141,15 @@ int64_t lbm_check_launch_indices(int nx, int ny, int nz, lbm_storage fmt, int ro
     if (visited2 != N) ++bad;
     };
     walk_pairs(Prows, false);
-    walk_pairs(flat_launch(Prows, 128), true);  // the two-grid step's launch when rows leave lanes idle
-    walk_pairs(flat_launch(Prows, 64), true);  // and of small lattices
-    // the FP32 reverse step, one cell per thread over the box rows in order
-    {
+    // flat launches: every block size of flat_threads and step_flat_threads
+    for (int threads : {64, 128, 256}) walk_pairs(flat_launch(Prows, threads), true);
+    // one cell per thread over the box rows in order: the FP32 reverse step and the
+    // FP64 two-grid step, in both of their block sizes
+    for (int threads : {64, 128}) {
         long long visited1 = 0;
-        const long long cells = (long long)Prows.nyr * nx, nblk = (cells + 255) / 256;
+        const long long cells = (long long)Prows.nyr * nx, nblk = (cells + threads - 1) / threads;
         for (int bz = 0; bz < Prows.nzr; ++bz)
-            for (long long k = 0; k < nblk * 256; ++k) {
+            for (long long k = 0; k < nblk * threads; ++k) {
                 const long long r = k / nx;
                 if (r >= Prows.nyr) continue;
                 ++visited1;
@@ -1156,7 +1157,7 @@ int64_t lbm_check_launch_indices(int nx, int ny, int nz, lbm_storage fmt, int ro
                 const int c = cell_index(g, x, y, z);
                 if (!cell_ok(c) || canon_index(g, x, y, z) >= N) ++bad;
                 for (int i = 0; i < Q; ++i)
-                    if (!cell_ok(push_dst(g, x, y, z, i))) ++bad;
+                    if (!cell_ok(push_dst(g, x, y, z, i)) || !cell_ok(pull_src(g, x, y, z, i))) ++bad;
             }
         if (visited1 != N) ++bad;
     }
@@ -1183,12 +1184,19 @@ int64_t lbm_check_launch_indices(int nx, int ny, int nz, lbm_storage fmt, int ro
                 if (k != 5) ++bad;
             }
     }
-    // reduction: canonical walk
-    for (long long cc = 0; cc < N; ++cc) {
-        const int x = (int)(cc % nx);
-        const long long r = cc / nx;
-        const int y = (int)(r % ny), z = (int)(r / ny);
-        if (!cell_ok(cell_index(g, x, y, z))) ++bad;
+    // reduction: the pairs of a range of planes, decoded as k_reduce does
+    {
+        long long visited3 = 0;
+        const int W = (nx + 1) / 2, per = W * ny, z0 = nz > 2 ? 1 : 0, z1 = nz;
+        for (long long q = 0; q < (long long)per * (z1 - z0); ++q) {
+            int x0, y, z;
+            reduce_pair((int)q, W, per, z0, x0, y, z);
+            const bool has1 = x0 + 1 < nx;
+            visited3 += has1 ? 2 : 1;
+            const int c = cell_index(g, x0, y, z);
+            if (z >= z1 || !cell_ok(c) || (has1 && !cell_ok(c + 1))) ++bad;
+        }
+        if (visited3 != (long long)nx * ny * (z1 - z0)) ++bad;
     }
     return bad;
 }

@@ -377,6 +377,14 @@ LBM_HD bool pair_cell(const Geom &g, const RowLaunch &P, int bdx, int bdy, int b
     return x0 < g.nx && y < P.y0 + P.nyr && z < P.z0 + P.nzr;
 }
 
+// Pair q of the planes from z0 on: the reduction's walk, W pairs a row, per a plane.
+LBM_HD void reduce_pair(int q, int W, int per, int z0, int &x0, int &y, int &z) {
+    const int zz = q / per, r = q - zz * per;
+    y = r / W;
+    x0 = 2 * (r - y * W);
+    z = z0 + zz;
+}
+
 // Push mask of a cell (precomputed on the host from the flags): bit j,
 // 1 <= j <= 18, is set when the neighbour x + e_j is solid, so population j
 // bounces back; SOLID_BIT is set on solid cells and on row padding.

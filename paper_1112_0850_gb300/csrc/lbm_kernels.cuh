@@ -1939,8 +1939,8 @@ __global__ void __launch_bounds__(RED_THREADS, FLAGS || is_split(S) ? 2 : FieldB
         PairTotals<R> tot;
         tot.clear();
         if (q < pairs) {
-            const int zz = (int)q / per, r = (int)q - zz * per, y = r / W;  // (pairs < 2^31)
-            const int x0 = 2 * (r - y * W), z = z0 + zz;
+            int x0, y, z;
+            reduce_pair((int)q, W, per, z0, x0, y, z);  // (pairs < 2^31)
             const bool has1 = x0 + 1 < d.g.nx;
             const int c = cell_index(d.g, x0, y, z);
             uint32_t m0, m1;

@@ -53,7 +53,7 @@ def test_compiled_table_matches_textbook_and_oracle(lib, golden_dir):
 
 
 SIZES = [(1, 1, 1), (1, 3, 2), (3, 1, 1), (2, 2, 2), (5, 4, 3), (8, 6, 5), (31, 3, 2), (32, 2, 2), (33, 7, 5),
-         (64, 3, 3), (65, 2, 3), (100, 5, 2), (256, 2, 2), (257, 3, 2), (300, 2, 1), (513, 1, 2)]
+         (64, 3, 3), (65, 2, 3), (100, 5, 2), (256, 2, 2), (257, 3, 2), (300, 2, 1), (513, 1, 2), (512, 2, 2), (1024, 1, 2)]
 
 
 @pytest.mark.parametrize("align", ["default", "128"])
