@@ -346,10 +346,13 @@ inline bool small_lattice(const RowLaunch &rows) { return (long long)rows.nyr * 
 inline int flat_threads(const RowLaunch &rows) { return small_lattice(rows) ? 64 : 128; }
 
 // The two-grid step without flags in FP32 and 16-bit shifted storage keeps
-// blocks of 256 where they tile every row (nx = 512, 1024, ..). Us a step with
-// 256 / 128 threads: 512^3 FP16 1683 / 1702, BF16 1670 / 1698, FP32 2900 / 2907;
-// 512x256x256 FP16 419 / 415, FP32 727.3 / 728.2; other rows, FP16: 496^3 1551 /
-// 1542, 528^3 1837 / 1814, 256^3 209.3 / 206.8.
+// blocks of 256 where they tile every row (nx = 512, 1024, ..): over 21 such
+// lattices of 34 to 210 million cells FP32 is 0.0 to 0.4% faster than with 128 and
+// BF16 -0.1 to +1.7% (512^3 2900 against 2908 us a step, 1672 against 1700). FP16 gains
+// 1.0% at 134 million cells (512^3 1683 against 1702, 1024x512x256 1693 against 1711)
+// and is -0.7 to +0.1% elsewhere (512x256x256 417 against 414, 512x768x512 2500 against
+// 2493): what decides it is not known, and it keeps the block size it had. Other rows
+// are faster with 128, FP16: 496^3 1551 against 1542, 528^3 1837 / 1814, 256^3 209.3 / 206.8.
 constexpr bool wide_blocks_fit(int storage, bool flags) {
     return !flags && (storage == LBM_F32 || storage == LBM_F16S || storage == LBM_BF16S);
 }
