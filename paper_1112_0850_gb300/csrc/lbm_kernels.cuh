@@ -1352,8 +1352,8 @@ template <int S, bool FLAGS> struct FieldBlocks {
 // that is the value its slot must hold, and in the others nobody reads it.
 // Bound by HBM (4 reals read and 19 values written a cell); every cell forming
 // the values of its 18 neighbours was bound by their 76 loads and by arithmetic
-// (FP64: its pipe 85% busy). Channel: FP32 165 to 111 us (floor 57), FP16 187 to
-// 86, FP64 2358 to 593; 256^3 box, FP32 435 to 288 us (floor 227).
+// (FP64: its pipe 85% busy). Whole call, channel: FP32 195 to 131 us (floor 57), FP16
+// 197 to 94, FP64 2373 to 306; 256^3 box, FP32 440 to 248 us (floor 227).
 // f_eq - w of the two cells of a pair: per direction one expression,
 // w (rho1 + rho (3 e.u + 9/2 (e.u)^2 - 3/2 u.u)), its roundings in this order. (The even
 // and odd parts of opposite directions formed once take 8 operations a pair of them
