@@ -1699,11 +1699,25 @@ static __device__ __noinline__ void split_store_moving(const Dev &d, typename St
 // Bound by HBM (19 values read and 19 written a cell). One cell a thread with
 // 18 flag loads and every value converted over double took 1622 us for the
 // 384x256x256 porous channel (FP16 to BF16: 1.9 GB, 0.17 of copy bandwidth).
-template <int S, int D, bool FLAGS>
-__global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
+// Blocks of 128 per SM: FP64 storage to narrower states 5 (4 before: channel to BF16
+// 185 to 165 us, AA 157 to 137), FP32 and 16-bit storage to FP64 states 8 and 7 (6:
+// channel 191 to 178 us and 165 to 157).
+template <int S, int D, bool FLAGS> constexpr int get_state_blocks() {
+    if (is_split(S)) return 2 * FieldBlocks<S, FLAGS>::value;
+    if (S == LBM_F64) return D == LBM_F64 ? 4 : 5;
+    return D == LBM_F64 ? (S == LBM_F32 ? 8 : 7) : 2 * FieldBlocks<S, FLAGS>::value;
+}
+
+// ALT: rows of odd length to FP64 states, where a pair is aligned in every other row
+// and population: each thread looks, and stores whole pairs where it can (cavity
+// 127x129x125, FP16 104 to 80 us, FP32 110 to 91; on small lattices the look costs
+// more than it gives, 95x61x53 18.4 to 22).
+template <int S, int D, bool FLAGS, bool ALT = false>
+__global__ void __launch_bounds__(128, get_state_blocks<S, D, FLAGS>())
     k_get_state(const Dev d, const typename Stor<S>::T *__restrict__ P, typename IOFmt<D>::T *__restrict__ out,
                 bool pair) {
     typedef typename Stor<S>::R R;
+    typedef typename IOFmt<D>::T TD;
     int x0, y, z;
     if (!pair_cell<true>(d.g, d.PF, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, x0, y,
                          z))
@@ -1722,8 +1736,20 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
     typename Pair2<R>::V s[Q];
     gather_pair<S, FLAGS>(d, P, x0, y, z, c, has1, m0, m1, s);
 #pragma unroll
-    for (int i = 0; i < Q; ++i)
-        put2(out + i * N + cc, pair, has1, !FLAGS || live0 ? s[i].x : R(0), !FLAGS || live1 ? s[i].y : R(0));
+    for (int i = 0; i < Q; ++i) {
+        TD *p = out + i * N + cc;
+        const bool whole = ALT ? has1 && (reinterpret_cast<uintptr_t>(p) & (2 * sizeof(TD) - 1)) == 0 : pair;
+        put2(p, whole, has1, !FLAGS || live0 ? s[i].x : R(0), !FLAGS || live1 ? s[i].y : R(0));
+    }
+}
+
+// Blocks of 128 per SM of set_state. Narrower storage from FP64 states, whose 38
+// values are held as doubles, 5 (96 registers): with the 7 of the narrower states the
+// kernels with flags spilled 312 to 416 bytes (AA channel FP32 163
+// to 142 us, FP16 169 to 145; two-grid 206 to 156 and 232 to 208).
+template <int S, int D, bool FLAGS> constexpr int set_state_blocks() {
+    if (D == LBM_F64 && S != LBM_F64) return 5;
+    return FLAGS && !is_split(S) && S != LBM_F64 ? 7 : 2 * FieldBlocks<S, FLAGS>::value;
 }
 
 // set_state: P_i(y) = s_i(y + e_i) if fluid there, else s_{opp(i)}(y). The
@@ -1732,7 +1758,7 @@ __global__ void __launch_bounds__(128, 2 * FieldBlocks<S, FLAGS>::value)
 // 19 values its cells hold and rounds momentum and remainders once, whatever format
 // they come in (256^3 box from FP32 301 us; in double 3017).
 template <int S, int D, bool FLAGS>
-__global__ void __launch_bounds__(128, FLAGS && !is_split(S) && S != LBM_F64 ? 7 : 2 * FieldBlocks<S, FLAGS>::value)
+__global__ void __launch_bounds__(128, set_state_blocks<S, D, FLAGS>())
     k_set_state(const Dev d, typename Stor<S>::T *__restrict__ P, const typename IOFmt<D>::T *__restrict__ in,
                 bool pair) {
     typedef typename Stor<S>::T T;
@@ -2351,12 +2377,11 @@ static cudaError_t launch_get(const Dev &d0, const void *lat, void *dst) {
     Dev d = d0;
     d.PF = all_pairs(d.g);
     const bool pair = pair_aligned(d.g, dst, sizeof(TD));
-    if (d.flags)
-        k_get_state<S, D, true><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(d, static_cast<const T *>(lat),
-                                                                                   static_cast<TD *>(dst), pair);
-    else
-        k_get_state<S, D, false><<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(d, static_cast<const T *>(lat),
-                                                                                    static_cast<TD *>(dst), pair);
+    void (*k)(Dev, const T *, TD *, bool) = d.flags ? k_get_state<S, D, true> : k_get_state<S, D, false>;
+    if constexpr (D == LBM_F64 && S != LBM_F64 && !is_split(S)) {
+        if ((d.g.nx & 1) && d.PF.bx_threads > 64) k = d.flags ? k_get_state<S, D, true, true> : k_get_state<S, D, false, true>;
+    }
+    k<<<pairs_grid(d.PF), d.PF.bx_threads, 0, d.stream>>>(d, static_cast<const T *>(lat), static_cast<TD *>(dst), pair);
     return cudaGetLastError();
 }
 
