@@ -6,13 +6,13 @@
 // form). Here a cell's 19 deviations s_i (and half its force)
 // are aligned to one exponent, that of the largest of them, as 64-bit integers
 // with the largest in [2^57, 2^58): 5 bits finer than its FP64 spacing. Sums
-// of them are exact. Products are rounded to nearest and keep 3 more bits. What is
+// of them are exact. Products are rounded to nearest and keep 2 more bits. What is
 // added to (1 - omega) s_i comes back as a double, correctly rounded, and one FP64
 // multiply-add per population is left.
 //
 // Against extended precision, relative to the cell's largest value, the
 // post-collision values are off (rms) by 0.2 to 1.0 times what the FP64 form is, the
-// momentum they carry by 0.1 to 1.02 times, with no mean in it: for tau from 0.5005
+// momentum they carry by 0.1 to 1.04 times, with no mean in it: for tau from 0.5005
 // to 50, flows of 1e-9 to 0.2 with density deviations up to 0.2, noise, and forces
 // from none to the largest value of the cell (tests/test_fixed64_cpu.py). Equilibria
 // and moments are off by 0.4 to 0.7 times. (With inputs cut at 2^-56, products rounded
@@ -40,14 +40,14 @@ namespace lbm {
 // taken as 1 - (1 - omega), so that it and the rounded 1 - omega add up to 1: else
 // every step would scale mass and momentum by the rounding (tau = 5: 1 + 5.6e-17).
 struct FixedK {
-    long long w29, w12, c6;  // 2/9 omega, omega/12, (1 - omega/2)/6
-    double omc;              // 1 - omega
+    long long w9, w12, c6;  // omega/9, omega/12, (1 - omega/2)/6
+    double omc;             // 1 - omega
 };
 inline FixedK fixed_k(double omega) {
     FixedK k;
     k.omc = 1.0 - omega;
     const long long w = (long long)ldexp(1.0 - k.omc, 61);  // omega < 2
-    k.w29 = w / 9 * 4 + (w % 9 * 4 + 4) / 9;
+    k.w9 = (w * 2 + 4) / 9;
     k.w12 = (w + 3) / 6;
     k.c6 = ((1LL << 62) - w + 3) / 6;  // (2^62 - omega 2^61) / 6
     return k;
@@ -162,9 +162,10 @@ struct FixedMom {
 };
 
 // False where the cell is outside the range of the fixed-point collision
-// (|s_i| or |F| >= 1/4, |rho - 1| or |j'| >= 1/2 or 8 to 16 times the largest of the
-// s_i and F, not finite): the caller then takes FP64 arithmetic. (A flow near
-// equilibrium has |rho - 1| < 4 and |j'| < 6 times its largest s_i.)
+// (|s_i| or |F|, |rho - 1| or |j'| >= 1/4, or the latter 8 to 16 times the largest of
+// the s_i and F, or not finite): the caller then takes FP64 arithmetic. (A flow near
+// equilibrium has |rho - 1| < 4 and |j'| < 6 times its largest s_i. With these limits
+// |u| <= 1/3, and every sum and product below stays within its 62 or 63 bits.)
 template <bool FORCE>
 LBM_HD bool fixed_moments(const double s[Q], double Fx, double Fy, double Fz, FixedMom &m) {
     uint32_t top = 128u << 20;  // (values below 2^-895 count as zero; keeps every result a normal number)
@@ -201,16 +202,16 @@ LBM_HD bool fixed_moments(const double s[Q], double Fx, double Fy, double Fz, Fi
         m.jy += m.fy;
         m.jz += m.fz;
     }
-    // |r|, |j| < 2^61 units and 1/2 (compared in the high halves)
+    // |r|, |j| < 2^61 units and 1/4 (compared in the high halves)
     const int n = 1023 - E;  // >= 3: the unit is 2^-(57 + n)
     const int rh = (int)(m.r >> 32), xh = (int)(m.jx >> 32), yh = (int)(m.jy >> 32), zh = (int)(m.jz >> 32);
     const int o = (rh ^ (rh >> 31)) | (xh ^ (xh >> 31)) | (yh ^ (yh >> 31)) | (zh ^ (zh >> 31));
-    return (o >> (n < 5 ? 24 + n : 29)) == 0;
+    return (o >> (n < 6 ? 23 + n : 29)) == 0;
 }
 // s <- (1 - omega) s + E +- P (see the head of this file), or with EQ
 // s <- E +- P: at omega = 1 and no force that is the equilibrium. g, h, X and B are
-// held in eighths of m's unit, so that 2 (B + X) +- 2 g and 12 B are whole in
-// quarters and halves of it.
+// held in quarters of m's unit, so that 2 (B + X) +- 2 g is whole in halves of it and
+// 12 B in units.
 template <bool FORCE, bool EQ = false>
 LBM_HD void fixed_collide(double s[Q], const FixedMom &m, const FixedK &k, bool incomp) {
     const int n = 1023 - m.E;  // >= 3
@@ -239,11 +240,11 @@ LBM_HD void fixed_collide(double s[Q], const FixedMom &m, const FixedK &k, bool 
     }
     const L31 iv = limbs(inv15);
     const L31 w12 = limbs(k.w12);
-    long long gx = mulk<3>(limbs(m.jx), w12), gy = mulk<3>(limbs(m.jy), w12), gz = mulk<3>(limbs(m.jz), w12);
+    long long gx = mulk<2>(limbs(m.jx), w12), gy = mulk<2>(limbs(m.jy), w12), gz = mulk<2>(limbs(m.jz), w12);
     long long hx = gx, hy = gy, hz = gz;
     if (FORCE) {
         const L31 c6 = limbs(k.c6);
-        const long long cx = mulk<3>(limbs(m.fx), c6), cy = mulk<3>(limbs(m.fy), c6), cz = mulk<3>(limbs(m.fz), c6);
+        const long long cx = mulk<2>(limbs(m.fx), c6), cy = mulk<2>(limbs(m.fy), c6), cz = mulk<2>(limbs(m.fz), c6);
         gx += cx;
         gy += cy;
         gz += cz;
@@ -259,13 +260,13 @@ LBM_HD void fixed_collide(double s[Q], const FixedMom &m, const FixedK &k, bool 
     const long long XZ = FORCE ? mulk<2>(vx, lz) + mulk<2>(vz, lx) : mulk<2>(vx, lz) << 1;
     const long long YZ = FORCE ? mulk<2>(vy, lz) + mulk<2>(vz, ly) : mulk<2>(vy, lz) << 1;
     constexpr long long third = 1537228672809129301LL;  // 2^62 / 3
-    const long long B = mulk<0>(limbs(m.r), limbs(k.w29)) - mulk<0>(limbs(X + Y + Z), limbs(third));
+    const long long B = mulk<0>(limbs(m.r), limbs(k.w9)) - mulk<0>(limbs(X + Y + Z), limbs(third));
     const int E = m.E;
-    s[0] = EQ ? fx_out(3 * B, E - 1) : fma(k.omc, s[0], fx_out(3 * B, E - 1));
+    s[0] = EQ ? fx_out(3 * B, E) : fma(k.omc, s[0], fx_out(3 * B, E));
 #pragma unroll
     for (int p = 0; p < NPAIR; ++p) {
         const int i = pair_first(p);
-        const int Ep = p < 3 ? E - 2 : E - 3;
+        const int Ep = p < 3 ? E - 1 : E - 2;
         long long e, o;
         if (p == 0) { e = B + X; o = gx; }
         else if (p == 1) { e = B + Y; o = gy; }
@@ -303,7 +304,7 @@ LBM_HD bool fixed_equilibrium(double f[Q], double rho1, double ux, double uy, do
         m.jy += mulk<1>(r, limbs(m.jy));
         m.jz += mulk<1>(r, limbs(m.jz));
     }
-    fixed_collide<false, true>(f, m, FixedK{0x0e38e38e38e38e39LL, 0x0555555555555555LL, 0, 0.0}, incomp);
+    fixed_collide<false, true>(f, m, FixedK{0x071c71c71c71c71cLL, 0x0555555555555555LL, 0, 0.0}, incomp);
     return true;
 }
 

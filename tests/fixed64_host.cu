@@ -1,6 +1,8 @@
 // Errors of the block fixed-point collision (lbm_fixed.cuh, compiled for the host)
 // and of the same collision in FP64 against long double, by kind of flow and tau.
-// Prints one line each: kind model tau, rms error of the values (FP64 form, fixed
+// First a line "wild" with the largest error, in units of the cell's largest value, over
+// cells far from equilibrium at every size the range takes in, and how many it took in.
+// Then one line each: kind model tau, rms error of the values (FP64 form, fixed
 // point), rms and mean error of the x momentum (FP64 form, fixed point) and the
 // number of cells; everything relative to the largest |s_i| or |F| of the cell.
 #include <cmath>
@@ -66,7 +68,44 @@ struct Sum {
     }
 };
 
+// Populations that add up in rho and j as far as the range allows: signs that follow a
+// random direction, or one for all, sizes near the cell's largest.
+static void wild() {
+    std::mt19937_64 gen(5);
+    std::uniform_real_distribution<double> U(-1, 1);
+    X worst = 0;
+    int n = 0;
+    for (int t = 0; t < 400000; ++t) {
+        const double size = ldexp(1.0, -2 - t % 9) * (0.75 + 0.25 * U(gen)), bias = U(gen), d[3] = {U(gen), U(gen), U(gen)};
+        const bool inc = t & 1, force = t & 2;
+        const double om = 1.0 + 0.999 * U(gen), flat = U(gen) * U(gen);
+        double s[Q], f[Q], F[3] = {0, 0, 0}, top = 0;
+        for (int i = 0; i < Q; ++i) {
+            const double p = ex(i) * d[0] + ey(i) * d[1] + ez(i) * d[2];
+            s[i] = f[i] = size * (1 + 0.1 * U(gen)) * (i == 0 || p == 0 ? bias : (p > 0 ? 1 : -1) * (1 - fabs(flat)) + flat);
+            top = fmax(top, fabs(s[i]));
+        }
+        for (int c = 0; c < 3 && force; ++c) F[c] = size * U(gen);
+        FixedMom m;
+        if (!(force ? fixed_moments<true>(f, F[0], F[1], F[2], m) : fixed_moments<false>(f, 0, 0, 0, m))) continue;
+        if (force)
+            fixed_collide<true>(f, m, fixed_k(om), inc);
+        else
+            fixed_collide<false>(f, m, fixed_k(om), inc);
+        X x[Q];
+        extended(s, om, F, inc, x);
+        for (int i = 0; i < Q; ++i) {
+            top = fmax(top, (double)fabsl(x[i]));
+            top = fmax(top, fabs(F[i % 3]));
+        }
+        for (int i = 0; i < Q; ++i) worst = fmaxl(worst, fabsl(f[i] - x[i]) / top);
+        ++n;
+    }
+    printf("wild %Lg %d\n", worst, n);
+}
+
 int main() {
+    wild();
     const struct { const char *name; double rho, u, noise, F; } kinds[] = {
         {"flow", 0.01, 0.03, 1e-3, 0},      {"rough", 0.02, 0.05, 0.05, 0}, {"still", 0.2, 1e-9, 1e-3, 0},
         {"slow", 0.01, 1e-4, 1e-2, 0},      {"fast", 0.2, 0.2, 1e-2, 0},    {"noise", 0, 0, 1.0, 0},

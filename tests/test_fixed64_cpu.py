@@ -17,6 +17,10 @@ def test_fixed_point_is_no_further_off_than_fp64(tmp_path):
                            os.path.join(HERE, "fixed64_host.cu"), "-o", exe])
     out = subprocess.run([exe], check=True, capture_output=True, text=True, timeout=300).stdout
     lines = [ln.split() for ln in out.splitlines()]
+    # no sum or product overflows in a cell that is taken in, however far from
+    # equilibrium: a few roundings of its largest value
+    _, worst, n = lines.pop(0)
+    assert int(n) >= 100000 and float(worst) <= 8 * 2.0 ** -53, (worst, n)
     assert len(lines) == 9 * 2 * 8
     for name, inc, tau, *v in lines:
         e64, efix, j64, jfix, _, mean, n = (float(x) for x in v)

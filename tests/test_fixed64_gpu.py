@@ -1,6 +1,6 @@
 """FP64 storage collides in block fixed point and, outside its range, in FP64:
-one step from states inside the range, across its edges (|s| = 1/4, rho - 1 and
-j = 1/2) and beyond it, from values of 1e-200 and of mixed size in one cell, and
+one step from states inside the range, across its edges (|s|, rho - 1 and j = 1/4)
+and beyond it, from values of 1e-200 and of mixed size in one cell, and
 of exact zeros, against the same step in extended precision; both streaming
 patterns, and a state that is not a number."""
 import numpy as np
